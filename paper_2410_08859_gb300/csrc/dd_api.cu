@@ -553,11 +553,12 @@ int domdec_init(domdec_t* out, const double* mu, const double* nu, int N, const 
   DevState& S = h->S;
   std::memset(&S, 0, sizeof(S));
   S.N = N; S.s = h->s; S.nb = h->nb; S.nbasic = h->nbasic;
-  S.h = 1.0 / N; S.eps = pin->eps; S.lam = pin->lambda; S.thr = pin->trunc_thr; S.err = pin->err;
+  S.h = 1.0 / N; S.lam = pin->lambda; S.thr = pin->trunc_thr; S.err = pin->err;
   S.ti = pin->cell_ti ? 1 : 0;
   S.balance = pin->balance ? 1 : 0;
   S.tau = pin->tau; S.maxit = pin->maxit; S.newton_maxit = pin->newton_maxit; S.strategy = pin->strategy;
   S.margin = pin->box_margin;
+  set_eps_scalars(S, pin->eps);
   // shared-memory capacity of the cell kernel
   int dev = 0, smem_optin = 0;
   cudaGetDevice(&dev);
@@ -792,7 +793,8 @@ int domdec_reset(domdec_t h, const double* mu, const double* nu, const double* a
   if (alpha0 && !(eps_init > 0.0 && std::isfinite(eps_init))) return DOMDEC_EINVAL;
   if (cudaStreamSynchronize(h->st) != cudaSuccess) return fail(h, DOMDEC_ECUDA);
   prof_collect(h);
-  h->S.eps = h->p.eps = h->eps0;
+  h->p.eps = h->eps0;
+  set_eps_scalars(h->S, h->eps0);
   h->S.err = h->p.err = h->err0;
   const int rc = load_problem(h, mu, nu, alpha0, beta0, eps_init);
   return rc ? fail(h, rc) : DOMDEC_OK;
@@ -802,7 +804,7 @@ int domdec_set_eps(domdec_t h, double eps) {
   if (!h) return DOMDEC_EINVAL;
   if (h->sticky) return DOMDEC_ESTATE;
   if (!(eps > 0.0) || !std::isfinite(eps)) return DOMDEC_EINVAL;
-  h->S.eps = eps;
+  set_eps_scalars(h->S, eps);
   h->p.eps = eps;
   return DOMDEC_OK;
 }

@@ -183,81 +183,282 @@ __device__ __forceinline__ int lanes_per_target(int nt, int M, int nthr) {
   return P;
 }
 
-// Root u of g(u) = (1+s) u + c0 + softplus(lr - u) = 0, i.e. of
+// Quotient u / w of non-negative integers by a multiplication with iw ~ 1/w.
+__device__ __forceinline__ int quot(int u, int w, float iw) {
+  int q = (int)((float)u * iw);
+  const int r = u - q * w;
+  q += r >= w ? 1 : 0;
+  q -= r < 0 ? 1 : 0;
+  return q;
+}
+
+// A rounded product that is not contracted into a later sum.
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+
+// Maximum that is NaN if either argument is.
+__device__ __forceinline__ float max_nan(float a, float b) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+
+// ---- float passes: a tile of B consecutive targets of one line per thread.
+// Chunks of kChunk sources whose terms all lie more than kCut (log2 units) below
+// their targets' shifts are left out.  A sum made that way is accepted between
+// kAccLo and 1e25, so what is left out is below 256 * 2^-60 / 2^-12 = 2^-40 of
+// it: it vanishes in the float sum.  (The floats are summed in one fixed order,
+// eight partial sums by the source index modulo eight: where the background
+// dominates, the Newton root amplifies a rounding of its argument by lam/eps, so
+// a value must not depend on the tile it was computed in.)
+constexpr float kCut = 60.0f, kAccLo = 2.44140625e-4f;
+constexpr int kChunk = 8;
+
+// acc[k] = sum_m 2^{src[m sm] - q2 (m - ctr0 - k)^2 - S[k]}, k < B.  The distances
+// of a chunk are formed once for the whole tile (kChunk + B - 1 of them); a
+// term is then an FFMA, a subtraction, an ex2 and an addition.
+template <int B>
+__device__ __forceinline__ void tile_sum(const float* src, int sm, int M, int ctr0, float q2, const float (&S)[B],
+                                         bool cull, float (&acc)[B]) {
+  float a[B][kChunk];
+#pragma unroll
+  for (int k = 0; k < B; ++k)
+#pragma unroll
+    for (int i = 0; i < kChunk; ++i) a[k][i] = 0.0f;
+  int m0 = 0;
+  for (; m0 + kChunk <= M; m0 += kChunk) {
+    float s[kChunk];
+#pragma unroll
+    for (int i = 0; i < kChunk; ++i) s[i] = src[(m0 + i) * sm];
+    if (cull) {
+      float cm = s[0];
+#pragma unroll
+      for (int i = 1; i < kChunk; ++i) cm = max_nan(cm, s[i]);
+      bool need = false;   // a NaN keeps the chunk
+#pragma unroll
+      for (int k = 0; k < B; ++k) {
+        const int j = ctr0 + k;
+        const float d = (float)(j - min(max(j, m0), m0 + kChunk - 1));
+        need |= !(fmaf(-q2 * d, d, cm) - S[k] < -kCut);
+      }
+      if (!need) continue;
+    }
+    float d[kChunk + B - 1], t[kChunk + B - 1];
+    const float d0 = (float)(m0 - ctr0 - (B - 1));
+#pragma unroll
+    for (int i = 0; i < kChunk + B - 1; ++i) {
+      d[i] = d0 + (float)i;
+      t[i] = q2 * d[i];
+    }
+#pragma unroll
+    for (int i = 0; i < kChunk; ++i)
+#pragma unroll
+      for (int k = 0; k < B; ++k)
+        a[k][i] += dd_ex2(fmaf(-t[i - k + B - 1], d[i - k + B - 1], s[i]) - S[k]);
+  }
+  for (; m0 < M; ++m0) {
+    const float s = src[m0 * sm], d0 = (float)(m0 - ctr0);
+#pragma unroll
+    for (int k = 0; k < B; ++k) {
+      const float d = d0 - (float)k;
+      a[k][0] += dd_ex2(fmaf(-(q2 * d), d, s) - S[k]);
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < B; ++k)
+    acc[k] = ((a[k][0] + a[k][1]) + (a[k][2] + a[k][3])) + ((a[k][4] + a[k][5]) + (a[k][6] + a[k][7]));
+}
+
+// out[k] = log2 sum_m 2^{src[m sm] - q2 (m - ctr0 - k)^2} for the first n targets
+// of the tile.  With `have`, S holds a previous value of each target as its
+// shift (one pass); a target whose sum leaves the accepted range is summed again
+// in full, and against its exact maximum if that does not help; so are all
+// targets without a previous value.
+template <int B>
+__device__ __forceinline__ void lse_tile(const float* src, int sm, int M, int ctr0, float q2, float (&S)[B],
+                                         bool have, int n, float (&out)[B]) {
+  const bool long_line = M > 4 * kChunk;   // shorter ones gain less than the test costs
+  bool need[B];
+#pragma unroll
+  for (int k = 0; k < B; ++k) {
+    need[k] = k < n;
+    if (k >= n) S[k] = INFINITY;   // no term of a target beyond the line's end
+  }
+  for (int level = have ? (long_line ? 0 : 1) : 2;; ++level) {
+    if (level == 2) {
+      float mx[B];
+#pragma unroll
+      for (int k = 0; k < B; ++k) mx[k] = -INFINITY;
+      for (int m = 0; m < M; ++m) {
+        const float s = src[m * sm], d = (float)(m - ctr0);
+#pragma unroll
+        for (int k = 0; k < B; ++k) mx[k] = fmaxf(mx[k], fmaf(-(q2 * (d - (float)k)), d - (float)k, s));
+      }
+#pragma unroll
+      for (int k = 0; k < B; ++k)
+        if (need[k]) S[k] = mx[k] > -INFINITY ? mx[k] : 0.0f;
+    }
+    float acc[B];
+    tile_sum<B>(src, sm, M, ctr0, q2, S, long_line && level != 1, acc);
+    const float lo = level == 0 ? kAccLo : 1e-25f;
+    bool bad = false;
+#pragma unroll
+    for (int k = 0; k < B; ++k) {
+      if (!need[k]) continue;
+      out[k] = S[k] + dd_lg2(acc[k]);
+      need[k] = !(acc[k] > lo && acc[k] < 1e25f);
+      bad |= need[k];
+    }
+    if (level == 2 || !bad) return;
+  }
+}
+
+// One 1-D log-sum-exp pass: lines l < L, targets j < J (source m at distance
+// m - j - off of target j), sources src[l sl + m sm], m < M.  `prev` holds the
+// previous iteration's values at [l ol + j oj] (unless `first`).  put(l, j, n, v)
+// receives n <= B consecutive values v[0..n).  Threads tid, tid + nthr, ... of
+// the pass; consecutive threads take consecutive lines.
+template <int B, typename Put>
+__device__ __forceinline__ void pass_tiles(const float* src, int sl, int sm, const float* prev, int ol, int oj, int L,
+                                           int J, int M, int off, float q2, bool first, int tid, int nthr, Put put) {
+  const int nitem = L * ((J + B - 1) / B);
+  const float iL = 1.0f / (float)L;
+  for (int it = tid; it < nitem; it += nthr) {
+    const int t = quot(it, L, iL), l = it - t * L, j0 = t * B, n = min(B, J - j0);
+    float S[B], v[B];
+#pragma unroll
+    for (int k = 0; k < B; ++k) S[k] = first ? 0.0f : prev[l * ol + min(j0 + k, J - 1) * oj];
+    lse_tile<B>(src + l * sl, sm, M, j0 + off, q2, S, !first, n, v);
+    put(l, j0, n, v);
+  }
+}
+
+// One target at a time on a group of P lanes (P a power of two), target j L + l.
+template <typename R, typename Put>
+__device__ __forceinline__ void pass_lanes(const R* src, int sl, int sm, const R* prev, int ol, int oj, int L, int J,
+                                           int M, int off, R q2, bool first, int P, int tid, int nthr, Put put) {
+  const int nt = L * J, ni = (nt * P + 31) & ~31, lp = 31 - __clz(P);
+  const float iL = 1.0f / (float)L;
+  for (int i = tid; i < ni; i += nthr) {
+    const int tg0 = i >> lp, part = i & (P - 1), tg = min(tg0, nt - 1);
+    const int j = quot(tg, L, iL), l = tg - j * L;
+    const R* row = src + l * sl;
+    R v[1];
+    v[0] = lse2_group<R>([&](int m) { return row[m * sm]; }, M, R(j + off), q2, prev[l * ol + j * oj], !first, part, P);
+    __syncwarp();
+    if (part == 0 && tg0 < nt) put(l, j, 1, v);
+  }
+}
+
+// Few targets: a group of lanes each.  Otherwise tiles of four targets when
+// they occupy three quarters of the threads, of two when those occupy a quarter
+// of them, else single targets: a larger tile spends fewer instructions per
+// term (about 6, 7.5 and 10), a smaller one keeps more warps busy on the small
+// cells.  `linear`: target j L + l on thread (j L + l) mod nthr in any case (for
+// sums over a thread's targets whose order must not depend on the tile).
+template <typename Put>
+__device__ __forceinline__ void run_pass(const float* src, int sl, int sm, const float* prev, int ol, int oj, int L,
+                                         int J, int M, int off, float q2, bool first, int tid, int nthr, Put put,
+                                         bool linear = false) {
+  const int P = lanes_per_target(L * J, M, nthr);
+  if (P > 1)
+    pass_lanes<float>(src, sl, sm, prev, ol, oj, L, J, M, off, q2, first, P, tid, nthr, put);
+  else if (!linear && 4 * L * ((J + 3) / 4) >= 3 * nthr)
+    pass_tiles<4>(src, sl, sm, prev, ol, oj, L, J, M, off, q2, first, tid, nthr, put);
+  else if (!linear && 4 * L * ((J + 1) / 2) >= nthr)
+    pass_tiles<2>(src, sl, sm, prev, ol, oj, L, J, M, off, q2, first, tid, nthr, put);
+  else
+    pass_tiles<1>(src, sl, sm, prev, ol, oj, L, J, M, off, q2, first, tid, nthr, put);
+}
+
+template <typename Put>
+__device__ __forceinline__ void run_pass(const double* src, int sl, int sm, const double* prev, int ol, int oj, int L,
+                                         int J, int M, int off, double q2, bool first, int tid, int nthr, Put put,
+                                         bool = false) {
+  pass_lanes<double>(src, sl, sm, prev, ol, oj, L, J, M, off, q2, first, lanes_per_target(L * J, M, nthr), tid, nthr,
+                     put);
+}
+
+// Roots u of g(u) = (1+s) u + c0 + softplus(lr - u) = 0, i.e. of
 // log(rho + e^u) + s u + c0 = 0 with lr = log rho (Eq. proxdiv-problem with
 // u = beta/eps + z).  g is convex and increasing (g' = 1 + s - sigmoid(lr - u) >= s).
 // Both lines (1+s)u + c0 and s u + c0 + lr lie below g, so g >= 0 at
 // min(u0, u1), their roots; Newton from there decreases monotonically to the root.
+// The Newton iterate after w, and its step *du (the same operations wherever a
+// target is advanced).
 template <typename R>
-__device__ __forceinline__ R newton_u(R lr, R c0, R s, int maxit) {
+__device__ __forceinline__ R newton_next(R lr, R c0, R w, R one_s, R* du = nullptr) {
   const R L2E = R(DD_LOG2E), LN2 = R(DD_LN2);
-  const R one_s = R(1) + s;
-  R u = -c0 / one_s;
-  if (!(lr > -dd_inf<R>())) return u;  // rho = 0: closed form (Eq. sinkhorn-iters-ot)
-  if (s > R(0)) u = min(u, -(lr + c0) / s);
-  const R tol = sizeof(R) == 4 ? R(2e-6) : R(1e-14);
-  for (int k = 0; k < maxit; ++k) {
-    R t = lr - u;
-    R e = dd_ex2(-fabs(t) * L2E);
-    R ie = dd_rcp(R(1) + e);
-    R sp = max(t, R(0)) + dd_lg2(R(1) + e) * LN2;
-    R sig = t >= R(0) ? ie : e * ie;
-    R g = one_s * u + c0 + sp;
-    R du = g * dd_rcp(one_s - sig);
-    u -= du;
+  R t = lr - w;
+  R e = dd_ex2(-fabs(t) * L2E);
+  R ie = dd_rcp(R(1) + e);
+  R sp = max(t, R(0)) + dd_lg2(R(1) + e) * LN2;
+  R sig = t >= R(0) ? ie : e * ie;
+  R g = one_s * w + c0 + sp;
+  R r = dd_rcp(one_s - sig);
+  if (!du) return fma(-g, r, w);
+  *du = mul_rn(g, r);
+  return w - *du;
+}
+template <typename R> __device__ __forceinline__ R newton_tol() { return sizeof(R) == 4 ? R(2e-6) : R(1e-14); }
+
+// A tile of B targets advances in lock-step (their dependency chains interleave;
+// each stops on its own tolerance).  `uw` holds a previous root per target (or
+// +inf: none): one Newton step from it lands right of the root (g is convex and
+// increasing), and the start is the smaller of that point and the bound
+// min(u0, u1), so the iteration still descends monotonically.
+// At most `steps` steps are made; act[k] tells which targets are still short of
+// the tolerance.  Where the background dominates, g' is close to s and the
+// rounding of g moves u by more than the tolerance, so a few targets (2-5 %) run
+// to the cap of 30 while the mean is 2.2: the caller finishes those from a list,
+// packed into full warps, instead of holding every warp for them.
+template <typename R, int B>
+__device__ __forceinline__ void newton_tile(const R (&lr)[B], const R (&c0)[B], const R (&uw)[B], R s, int steps,
+                                            R (&u)[B], bool (&act)[B]) {
+  const R one_s = R(1) + s, tol = newton_tol<R>();
+  bool any = false;
+#pragma unroll
+  for (int k = 0; k < B; ++k) {
+    u[k] = -c0[k] / one_s;
+    act[k] = lr[k] > -dd_inf<R>();   // rho = 0: closed form (Eq. sinkhorn-iters-ot)
+    if (act[k] && s > R(0)) u[k] = min(u[k], -(lr[k] + c0[k]) / s);
+    any |= act[k];
+  }
+  // probe step from the previous roots
+#pragma unroll
+  for (int k = 0; k < B; ++k) {
+    R wn = newton_next(lr[k], c0[k], uw[k], one_s);
+    if (act[k] && wn == wn && wn < u[k]) u[k] = wn;
+  }
+  for (int it = 0; it < steps && any; ++it) {
+    any = false;
+#pragma unroll
+    for (int k = 0; k < B; ++k) {
+      R du = R(0);
+      const R un = newton_next(lr[k], c0[k], u[k], one_s, &du);
+      if (act[k]) {
+        u[k] = un;
+        act[k] = !(fabs(du) <= tol * max(R(1), fabs(un)));
+        any |= act[k];
+      }
+    }
+  }
+}
+
+// At most `steps` further steps of one target.
+template <typename R>
+__device__ __forceinline__ R newton_rest(R lr, R c0, R u, R s, int steps) {
+  const R one_s = R(1) + s, tol = newton_tol<R>();
+  for (int it = 0; it < steps; ++it) {
+    R du;
+    u = newton_next(lr, c0, u, one_s, &du);
     if (fabs(du) <= tol * max(R(1), fabs(u))) break;
   }
   return u;
 }
 
-// Two independent roots of newton_u advanced in lock-step (their dependency
-// chains interleave; each stops on its own tolerance).  `uw` holds a previous
-// root per target (or NaN): one Newton step from it lands right of the root
-// (g is convex and increasing), and the start is the smaller of that point and
-// the bound min(u0, u1), so the iteration still descends monotonically.
-template <typename R>
-__device__ __forceinline__ void newton_u2(const R (&lr)[2], const R (&c0)[2], const R (&uw)[2], R s, int maxit,
-                                          R (&u)[2]) {
-  const R L2E = R(DD_LOG2E), LN2 = R(DD_LN2);
-  const R one_s = R(1) + s;
-  const R tol = sizeof(R) == 4 ? R(2e-6) : R(1e-14);
-  bool act[2];
-#pragma unroll
-  for (int k = 0; k < 2; ++k) {
-    u[k] = -c0[k] / one_s;
-    act[k] = lr[k] > -dd_inf<R>();
-    if (act[k] && s > R(0)) u[k] = min(u[k], -(lr[k] + c0[k]) / s);
-  }
-  // probe step from the previous roots
-#pragma unroll
-  for (int k = 0; k < 2; ++k) {
-    R w = uw[k];
-    R t = lr[k] - w;
-    R e = dd_ex2(-fabs(t) * L2E);
-    R ie = dd_rcp(R(1) + e);
-    R sp = max(t, R(0)) + dd_lg2(R(1) + e) * LN2;
-    R sig = t >= R(0) ? ie : e * ie;
-    R g = one_s * w + c0[k] + sp;
-    R wn = w - g * dd_rcp(one_s - sig);
-    if (act[k] && wn == wn && wn < u[k]) u[k] = wn;
-  }
-  for (int it = 0; it < maxit && (act[0] || act[1]); ++it) {
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      R t = lr[k] - u[k];
-      R e = dd_ex2(-fabs(t) * L2E);
-      R ie = dd_rcp(R(1) + e);
-      R sp = max(t, R(0)) + dd_lg2(R(1) + e) * LN2;
-      R sig = t >= R(0) ? ie : e * ie;
-      R g = one_s * u[k] + c0[k] + sp;
-      R du = g * dd_rcp(one_s - sig);
-      if (act[k]) {
-        u[k] -= du;
-        if (fabs(du) <= tol * max(R(1), fabs(u[k]))) act[k] = false;
-      }
-    }
-  }
-}
+constexpr int kLock = 4;     // Newton steps made in lock-step by every warp (float cells)
+constexpr int kPend = 512;   // targets listed for the remaining steps (more are finished in place)
 
 // mu phi((p0 + d)/mu) - mu phi(p0/mu) with phi(s) = s log s - s + 1, written as
 //   d (log(p0/mu) - 1) + (p0 + d) log1p(d/p0),
@@ -291,6 +492,40 @@ __device__ __forceinline__ double box_value(const BoxRec& b, const double* arena
 
 }  // namespace
 
+// Block sums of a cell: doubles for the double cells, pairs of floats for the float ones.
+template <typename R, int K>
+__device__ __forceinline__ void cell_sum(double (&v)[K], double* scratch) {
+  if constexpr (sizeof(R) == 4) block_sum_ff<K>(v, scratch);
+  else block_sum<K>(v, scratch);
+}
+
+// Scalars of one cell in the working precision.  One thread computes them from
+// the doubles and the CTA reads them from shared memory: the same dozen
+// double operations on every thread took 20 k clocks a cell (the FP64 pipe
+// gives two lanes a clock), a tenth of a small cell's solve.
+template <typename R>
+struct CellScalars {
+  double A, qD2;   // alpha/eps = A + a + 2 q D.xi; beta/eps = q|D|^2 - A + b - 2 q D.eta
+  R q2, qR, sR, rR, sB, cEta1, cEta2, cA, gA, cD1, cD2, tol;
+  __device__ __forceinline__ void set_A(const DevState& S, double a) {
+    A = a;
+    sB = R(S.sl * (qD2 - A));   // s B
+    cA = R(-(1.0 - S.rr) * A);
+    gA = R(-S.sl * A);          // -s A: the A part of -alpha/lam
+  }
+  __device__ __forceinline__ void set(const DevState& S, int D1, int D2, double a, double muJ) {
+    qD2 = S.q * (double)(D1 * D1 + D2 * D2);
+    q2 = R(S.q * DD_LOG2E); qR = R(S.q); sR = R(S.sl); rR = R(S.rr);
+    cEta1 = R(S.sl * 2.0 * S.q * D1); cEta2 = R(S.sl * 2.0 * S.q * D2);
+    cD1 = R(2.0 * (1.0 - S.rr) * S.q * D1); cD2 = R(2.0 * (1.0 - S.rr) * S.q * D2);
+    // gap <= err |mu_J| in the working precision: the largest value not above the bound
+    const double t = S.err * muJ;
+    if constexpr (sizeof(R) == 4) tol = __double2float_rd(t);
+    else tol = t;
+    set_A(S, a);
+  }
+};
+
 // One composite cell on one CTA: cell `cd` at position `cidx` of a sub-batch
 // of `nbatch` cells.
 template <typename R>
@@ -300,11 +535,12 @@ __device__ __forceinline__ void cell_solve_body(const DevState& S, const CellDes
   double* red = reinterpret_cast<double*>(smem_raw);  // 32 * 16 doubles (block reductions)
   __shared__ BoxRec sbox[4];
   __shared__ int sgeo[8];
+  __shared__ CellScalars<R> sk;
+  __shared__ int npend;
   CellOut* out = S.cout + cidx;
   const unsigned long long t_start = dd_global_ns();
   const double* __restrict__ arena = S.arena[*S.cur];
   const int tid = threadIdx.x, nthr = blockDim.x;
-  const int gtid = tid, gthr = nthr;
   const int N = S.N, s = S.s;
   const int nx1 = cd.nx1, nx2 = cd.nx2, nx = nx1 * nx2;
   auto csync = [&]() { __syncthreads(); };
@@ -362,18 +598,24 @@ __device__ __forceinline__ void cell_solve_body(const DevState& S, const CellDes
   // X-side arrays always live in shared memory; the Y-side arrays too unless
   // the box exceeds the shared capacity, then in the cell's spill slot
   // (global memory, L2-resident) sized for an N x N box.
-  const int cap_nx = 4 * s * s;
+  // Rows of X, of T and U and of the Y-side arrays have odd pitches where those
+  // fit (xp, Wp, Up), so that both a line of consecutive elements and a column
+  // of consecutive lines are read without bank conflicts.
+  const int cap_nx = 4 * s * s, cap_xp = cap_nx + 2 * s, xp = nx2 | 1;
   const int slot = sgeo[7];
   const bool spilled = slot >= 0;
   const int tsz = spilled ? 2 * s * N : 2 * s * S.cap_side;
   const int cap_ny = spilled ? N * N : S.cap_ny;
+  const int Wo = W | 1;
+  const int Wp = !spilled && nx1 * Wo <= tsz && H * Wo <= cap_ny && 3 * nx1 * Wo <= 2 * tsz + 3 * cap_ny ? Wo : W;
+  const int Up = !spilled && H * (nx2 | 1) <= tsz ? nx2 | 1 : nx2;
   R* xa = reinterpret_cast<R*>(smem_raw + 32 * 16 * sizeof(double));
-  R* av = xa + cap_nx;
+  R* av = xa + cap_xp;
   R* g0 = av + cap_nx;
   R* Wv = g0 + cap_nx;
   R* lm = Wv + cap_nx;
   R* xa_nx = lm + cap_nx;    // next iterate of xa / a (double buffer of the X-update)
-  R* av_nx = xa_nx + cap_nx;
+  R* av_nx = xa_nx + cap_xp;
   R* T = spilled ? reinterpret_cast<R*>(S.spill + (long long)slot * S.spill_stride) : av_nx + cap_nx;
   R* U = T + tsz;
   R* bl = U + tsz;
@@ -386,11 +628,12 @@ __device__ __forceinline__ void cell_solve_body(const DevState& S, const CellDes
   // rho = max(0, P_Y - nu_J)/nu and log nu on B_J; the same pass accumulates
   // the barycentre of nu_J, whose nearest pixel is the Y frame origin (so
   // that 2 q D.xi carries the cell's mean displacement).
+  const float iW = 1.0f / (float)W, inx2 = 1.0f / (float)nx2;
   double a_tot = 0.0;   // |nu_{-J}| on B_J (translation step)
   {
     double m3[4] = {0.0, 0.0, 0.0, 0.0};
     for (int u = tid; u < ny; u += nthr) {
-      int kk = u / W, ll = u - kk * W;
+      const int kk = quot(u, W, iW), ll = u - kk * W, v = kk * Wp + ll;
       int y1 = k0 + kk, y2 = l0 + ll, y = y1 * N + y2;
       double nuJ = 0.0;
 #pragma unroll
@@ -398,11 +641,12 @@ __device__ __forceinline__ void cell_solve_body(const DevState& S, const CellDes
       double nuy = S.nu[y];
       const double num = fmax(0.0, S.PY[y] - nuJ);
       R rho = R(num) / R(nuy);
-      lrho[u] = rho > R(0) ? dd_lg2(rho) * R(DD_LN2) : -dd_inf<R>();
-      lnu[u] = R(S.lognu[y]);
-      m3[0] += nuJ; m3[1] += nuJ * kk; m3[2] += nuJ * ll; m3[3] += num;
+      lrho[v] = rho > R(0) ? dd_lg2(rho) * R(DD_LN2) : -dd_inf<R>();
+      lnu[v] = R(S.lognu[y]);
+      m3[0] += nuJ; m3[1] += nuJ * kk; m3[2] += nuJ * ll;
+      if (S.ti) m3[3] += num;
     }
-    block_sum<4>(m3, red);
+    cell_sum<R, 4>(m3, red);
     a_tot = m3[3];
     if (tid == 0) {
       int c1 = H / 2, c2 = W / 2;
@@ -418,33 +662,27 @@ __device__ __forceinline__ void cell_solve_body(const DevState& S, const CellDes
   const int yc1 = k0 + sgeo[5], yc2 = l0 + sgeo[6];
   const int D1 = xc1 - yc1, D2 = xc2 - yc2;
   const int offr = (k0 - cd.i0) + D1, offc = (l0 - cd.j0) + D2;
-  const double eps = S.eps, lam = S.lam;
-  const double q = S.h * S.h / eps;
-  const double sl = eps / lam;            // s = eps/lam
-  const double rr = lam / (eps + lam);    // r = lam/(eps+lam)
-  const R q2 = R(q * DD_LOG2E), qR = R(q), sR = R(sl), rR = R(rr);
+  const double eps = S.eps, q = S.q, sl = S.sl;   // q = h^2/eps, s = eps/lam
 
   // ------------------------------------------------------- load X side
-  const double inv_eps = 1.0 / eps;
+  const double inv_eps = S.inv_eps;
   double acc2[2] = {0.0, 0.0};
   for (int t = tid; t < nx; t += nthr) {
-    int r = t / nx2, c = t - r * nx2;
+    const int r = quot(t, nx2, inx2), c = t - r * nx2;
     int x = (cd.i0 + r) * N + cd.j0 + c;
     int xi1 = cd.i0 + r - xc1, xi2 = cd.j0 + c - xc2;
     acc2[0] += S.alpha[x] * inv_eps - 2.0 * q * (double)(D1 * xi1 + D2 * xi2);
     acc2[1] += S.mu[x];
   }
   block_sum<2>(acc2, red);
-  double A = acc2[0] / nx;
-  const double muJ = acc2[1];
-  const double qD2 = q * (double)(D1 * D1 + D2 * D2);
-  R sB = R(sl * (qD2 - A));   // s B with B = q|D|^2 - A
-  const R cEta1 = R(sl * 2.0 * q * D1), cEta2 = R(sl * 2.0 * q * D2);
-  R cA = R(-(1.0 - rr) * A);
-  R gA = R(-sl * A);          // -s A: the A part of -alpha/lam
-  const R cD1 = R(2.0 * (1.0 - rr) * q * D1), cD2 = R(2.0 * (1.0 - rr) * q * D2);
+  if (tid == 0) sk.set(S, D1, D2, acc2[0] / nx, acc2[1]);
+  __syncthreads();
+  double A = sk.A;
+  const R q2 = sk.q2, qR = sk.qR, sR = sk.sR, rR = sk.rR, cEta1 = sk.cEta1, cEta2 = sk.cEta2, cD1 = sk.cD1,
+          cD2 = sk.cD2, tol = sk.tol;
+  R sB = sk.sB, cA = sk.cA, gA = sk.gA;
   for (int t = tid; t < nx; t += nthr) {
-    int r = t / nx2, c = t - r * nx2;
+    const int r = quot(t, nx2, inx2), c = t - r * nx2;
     int x = (cd.i0 + r) * N + cd.j0 + c;
     int xi1 = cd.i0 + r - xc1, xi2 = cd.j0 + c - xc2;
     double lin = 2.0 * q * (double)(D1 * xi1 + D2 * xi2);
@@ -453,7 +691,7 @@ __device__ __forceinline__ void cell_solve_body(const DevState& S, const CellDes
     av[t] = a;
     lm[t] = l;
     g0[t] = R(-sl * lin);
-    xa[t] = (a + l) * R(DD_LOG2E);
+    xa[r * xp + c] = (a + l) * R(DD_LOG2E);
   }
   csync();
 
@@ -461,99 +699,105 @@ __device__ __forceinline__ void cell_solve_body(const DevState& S, const CellDes
   // Barriers per iteration: after each of the five passes.  The X-update is
   // computed speculatively inside the last pass into the second buffer, and
   // the gap is reduced from per-warp partials after that pass's barrier.
-  const double tol = S.err * muJ;
   const R LN2 = R(DD_LN2), L2E = R(DD_LOG2E);
+  const bool stops = S.err >= 0.0;
   R* gpart = reinterpret_cast<R*>(red) + 32 * 12;   // per-warp gap partials
   R* apart = gpart + 32;                             // per-warp <e^{-alpha/lam}, mu> (translation step)
   R* bpart = gpart + 64;                             // per-warp <e^{-beta/lam}, nu>
+  int* pend = reinterpret_cast<int*>(red + 256);    // kPend list entries (the last 2 KB of red)
+  const int lock = sizeof(R) == 4 ? kLock : S.newton_maxit;
   const bool ti = S.ti && sl > 0.0;
   const int lane = tid & 31, wid = tid >> 5, nwarp = nthr >> 5;
   int it = 0;
-  double gap = 0.0;
+  R gap = R(0);
   bool first = true;
-  const bool fused_y = ny * 2 > gthr;   // large boxes: one lane per y, LSE and Newton fused
+  // translation step: nu e^{-beta/lam} per y, in the cell's buffer of new marginals (written by the epilogue only)
+  R* tib;
+  {
+    CellOut tmp;
+    tmp.slot = slot;
+    int st;
+    tib = reinterpret_cast<R*>(cell_nut(S, tmp, cidx, &st));
+  }
   R *xa_c = xa, *av_c = av;          // current iterate
   R *xa_n = xa_nx, *av_n = av_nx;    // next iterate
   for (;;) {
     ++it;
+    if (tid == 0) npend = 0;
     // Y-half, pass over columns of X: T(r, ll) = log2 sum_c 2^{xa(r,c) - q2 (c - ll - offc)^2}
-    {
-      const int nt = nx1 * W, P = lanes_per_target(nt, nx2, gthr), ni = (nt * P + 31) & ~31;
-      for (int i = gtid; i < ni; i += gthr) {
-        const int tg0 = i / P, part = i - tg0 * P, tg = min(tg0, nt - 1);
-        const int r = tg / W, ll = tg - r * W;
-        const R* row = xa_c + r * nx2;
-        R v = lse2_group<R>([&](int m) { return row[m]; }, nx2, R(ll + offc), q2, T[tg], !first, part, P);
-        __syncwarp();
-        if (part == 0 && tg0 < nt) T[tg] = v;
-      }
-    }
+    run_pass(xa_c, xp, 1, T, Wp, 1, nx1, W, nx2, offc, q2, first, tid, nthr, [&](int r, int ll, int n, const auto& v) {
+      for (int k = 0; k < n; ++k) T[r * Wp + ll + k] = v[k];
+    });
     csync();
-    // Y-half, pass over rows of X: Z(kk, ll), then the Newton root per y (a3)
+    // Y-half, pass over rows of X: Z(kk, ll), then the Newton roots of the tile (a3)
     R bsum = R(0);
-    if (fused_y) {
-      // every lane runs the same number of rounds (lse2_group is warp-collective)
-      const int rounds = (ny + 2 * gthr - 1) / (2 * gthr);
-      for (int rd = 0; rd < rounds; ++rd) {
-        const int u = gtid + rd * 2 * gthr;
-        const int uu[2] = {min(u, ny - 1), min(u + gthr, ny - 1)};
-        const bool ok[2] = {u < ny, u + gthr < ny};
-        R lr[2], c0[2], uw[2], root[2], Zn[2];
+    const bool fused_y = sizeof(R) == 4 && ny * 2 > nthr;
+    // root u of one y: Z, beta and beta + log nu (Zx: Z in natural units, or, for
+    // the small boxes that are not fused, in log2 units)
+    auto y_store = [&](int v, int y, R u, R Zx, R Zn, R c0) {
+      const R b = fused_y ? u - Zx : fma(-Zx, LN2, u);
+      Zv[v] = fused_y ? mul_rn(Zx, L2E) : Zx;
+      bv[v] = b;
+      bl[v] = (b + lnu[v]) * L2E;
+      // nu e^{-beta/lam}: -s beta/eps = -(s root + c0)
+      if (ti) tib[y] = dd_ex2((lnu[v] - sR * u - c0) * L2E);
+    };
+    auto y_root = [&](int ll, int kk, int n, const auto& Z2) {
+      constexpr int B = sizeof(Z2) / sizeof(R);
+      R lr[B], c0[B], uw[B], root[B], Zn[B];
+      const R eta2 = R(l0 + ll - yc2);
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-          const int kk = uu[k] / W, ll = uu[k] - kk * W;
-          R Z2 = lse2_group<R>([&](int m) { return T[m * W + ll]; }, nx1, R(kk + offr), q2, Zv[uu[k]], !first, 0, 1);
-          Zn[k] = Z2 * LN2;
-          R eta1 = R(k0 + kk - yc1), eta2 = R(l0 + ll - yc2);
-          c0[k] = sB - cEta1 * eta1 - cEta2 * eta2 - sR * Zn[k];
-          lr[k] = lrho[uu[k]];
-          uw[k] = first ? dd_inf<R>() : bv[uu[k]] + Zn[k];
-        }
-        newton_u2<R>(lr, c0, uw, sR, S.newton_maxit, root);
-        __syncwarp();
+      for (int k = 0; k < B; ++k) {
+        const int v = (kk + min(k, n - 1)) * Wp + ll;
+        Zn[k] = mul_rn(k < n ? Z2[k] : Z2[0], LN2);
+        const R eta1 = R(k0 + kk + min(k, n - 1) - yc1);
+        c0[k] = sB - cEta1 * eta1 - cEta2 * eta2 - sR * Zn[k];
+        lr[k] = lrho[v];
+        uw[k] = first ? dd_inf<R>() : bv[v] + Zn[k];
+      }
+      bool open[B];
+      newton_tile<R, B>(lr, c0, uw, sR, min(S.newton_maxit, lock), root, open);
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-          if (!ok[k]) continue;
-          Zv[uu[k]] = Zn[k] * L2E;
-          R b = root[k] - Zn[k];
-          bv[uu[k]] = b;
-          bl[uu[k]] = (b + lnu[uu[k]]) * L2E;
-          // nu e^{-beta/lam}: -s beta/eps = -(s root + c0)
-          if (ti) bsum += dd_ex2((lnu[uu[k]] - sR * root[k] - c0[k]) * L2E);
+      for (int k = 0; k < B; ++k) {
+        if (k >= n) break;
+        if (lock < S.newton_maxit && open[k]) {
+          const int v = (kk + k) * Wp + ll, e = atomicAdd(&npend, 1);
+          if (e < kPend) {   // finished below from the list
+            pend[e] = v;
+            bv[v] = root[k];
+            Zv[v] = fused_y ? Zn[k] : Z2[k];
+            continue;
+          }
+          root[k] = newton_rest(lr[k], c0[k], root[k], sR, S.newton_maxit - lock);
         }
+        y_store((kk + k) * Wp + ll, (kk + k) * W + ll, root[k], fused_y ? Zn[k] : Z2[k], Zn[k], c0[k]);
+      }
+    };
+    if constexpr (sizeof(R) == 4) {
+      run_pass(T, 1, Wp, Zv, 1, Wp, W, H, nx1, offr, q2, first, tid, nthr, y_root);
+      __syncthreads();
+      const int np = min(npend, kPend);
+      const float iWp = 1.0f / (float)Wp;
+      for (int e = tid; e < np; e += nthr) {
+        const int v = pend[e], kk = quot(v, Wp, iWp), ll = v - kk * Wp;
+        const R Zx = Zv[v], Zn = fused_y ? Zx : mul_rn(Zx, LN2);
+        const R eta1 = R(k0 + kk - yc1), eta2 = R(l0 + ll - yc2);
+        const R c0 = sB - cEta1 * eta1 - cEta2 * eta2 - sR * Zn;
+        y_store(v, kk * W + ll, newton_rest(lrho[v], c0, bv[v], sR, S.newton_maxit - lock), Zx, Zn, c0);
       }
     } else {
-      const int P = lanes_per_target(ny, nx1, gthr), ni = (ny * P + 31) & ~31;
-      for (int i = gtid; i < ni; i += gthr) {
-        const int u0 = i / P, part = i - u0 * P, u = min(u0, ny - 1);
-        const int kk = u / W, ll = u - kk * W;
-        R Z2 = lse2_group<R>([&](int m) { return T[m * W + ll]; }, nx1, R(kk + offr), q2, Zv[u], !first, part, P);
-        __syncwarp();
-        if (part == 0 && u0 < ny) Zv[u] = Z2;
-      }
+      run_pass(T, 1, Wp, Zv, 1, Wp, W, H, nx1, offr, q2, first, tid, nthr,
+               [&](int ll, int kk, int, const auto& v) { Zv[kk * Wp + ll] = v[0]; });
       csync();
-      for (int u = gtid; u < ny; u += 2 * gthr) {
-        const int uu[2] = {u, min(u + gthr, ny - 1)};
-        R lr[2], c0[2], uw[2], root[2];
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-          const int kk = uu[k] / W, ll = uu[k] - kk * W;
-          R Zn = Zv[uu[k]] * LN2;
-          R eta1 = R(k0 + kk - yc1), eta2 = R(l0 + ll - yc2);
-          c0[k] = sB - cEta1 * eta1 - cEta2 * eta2 - sR * Zn;
-          lr[k] = lrho[uu[k]];
-          uw[k] = first ? dd_inf<R>() : bv[uu[k]] + Zn;
-        }
-        newton_u2<R>(lr, c0, uw, sR, S.newton_maxit, root);
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-          if (k == 1 && u + gthr >= ny) break;
-          R b = root[k] - Zv[uu[k]] * LN2;
-          bv[uu[k]] = b;
-          bl[uu[k]] = (b + lnu[uu[k]]) * L2E;
-          if (ti) bsum += dd_ex2((lnu[uu[k]] - sR * root[k] - c0[k]) * L2E);
-        }
+      for (int u = tid; u < ny; u += nthr) {
+        const int kk = quot(u, W, iW), ll = u - kk * W;
+        const R z[1] = {Zv[kk * Wp + ll]};
+        y_root(ll, kk, 1, z);
       }
+    }
+    if (ti) {
+      csync();
+      for (int u = tid; u < ny; u += nthr) bsum += tib[u];
     }
     if (ti) {
       bsum = warp_sum(bsum);
@@ -561,28 +805,18 @@ __device__ __forceinline__ void cell_solve_body(const DevState& S, const CellDes
     }
     csync();
     // X-half, pass over columns of B_J: U(kk, c) = log2 sum_ll 2^{bl(kk,ll) - q2 (ll - (c - offc))^2}
-    {
-      const int nt = H * nx2, P = lanes_per_target(nt, W, gthr), ni = (nt * P + 31) & ~31;
-      for (int i = gtid; i < ni; i += gthr) {
-        const int tg0 = i / P, part = i - tg0 * P, tg = min(tg0, nt - 1);
-        const int kk = tg / nx2, c = tg - kk * nx2;
-        const R* row = bl + kk * W;
-        R v = lse2_group<R>([&](int m) { return row[m]; }, W, R(c - offc), q2, U[tg], !first, part, P);
-        __syncwarp();
-        if (part == 0 && tg0 < nt) U[tg] = v;
-      }
-    }
+    run_pass(bl, Wp, 1, U, Up, 1, H, nx2, W, -offc, q2, first, tid, nthr, [&](int kk, int c, int n, const auto& v) {
+      for (int k = 0; k < n; ++k) U[kk * Up + c + k] = v[k];
+    });
     csync();
     // X-half, pass over rows of B_J: W, the gap terms (a4) and the next a (a2)
     {
       R gl = R(0), asum = R(0);
-      const int P = lanes_per_target(nx, H, gthr), ni = (nx * P + 31) & ~31;
-      for (int i = gtid; i < ni; i += gthr) {
-        const int tg0 = i / P, part = i - tg0 * P, t = min(tg0, nx - 1);
-        const int r = t / nx2, c = t - r * nx2;
-        R W2 = lse2_group<R>([&](int m) { return U[m * nx2 + c]; }, H, R(r - offr), q2, Wv[t], !first, part, P);
-        __syncwarp();
-        if (part == 0 && tg0 < nx) {
+      run_pass(U, 1, Up, Wv, 1, nx2, nx2, nx1, H, -offr, q2, first, tid, nthr,
+               [&](int c, int r0, int n, const auto& v) {
+        for (int k = 0; k < n; ++k) {
+          const int r = r0 + k, t = r * nx2 + c;
+          const R W2 = v[k];
           Wv[t] = W2;
           R a = av_c[t];
           R tt = a + W2 * LN2;         // log(P_X pi / mu)
@@ -591,10 +825,10 @@ __device__ __forceinline__ void cell_solve_body(const DevState& S, const CellDes
           R xi1 = R(cd.i0 + r - xc1), xi2 = R(cd.j0 + c - xc2);
           R an = cA - rR * W2 * LN2 - cD1 * xi1 - cD2 * xi2;
           av_n[t] = an;
-          xa_n[t] = (an + lm[t]) * L2E;
+          xa_n[r * xp + c] = (an + lm[t]) * L2E;
           if (ti) asum += dd_ex2((lm[t] + gA + g0[t] - sR * an) * L2E);   // mu e^{-alpha_new/lam}
         }
-      }
+      }, ti);
       gl = warp_sum(gl);
       if (lane == 0) gpart[wid] = gl;
       if (ti) {
@@ -606,26 +840,26 @@ __device__ __forceinline__ void cell_solve_body(const DevState& S, const CellDes
     {
       R gs = R(0);
       for (int w = 0; w < nwarp; ++w) gs += gpart[w];
-      gap = (double)gs;
+      gap = gs;
     }
     first = false;
-    if ((S.err >= 0.0 && gap <= tol) || it >= S.maxit || !(gap == gap)) break;
+    if ((stops && gap <= tol) || it >= S.maxit || !(gap == gap)) break;
     if (ti) {
       // translation step: alpha += t*, e^{t*/lam} = (a + sqrt(a^2 + 4 A_s B_s)) / (2 B_s); in the
-      // cell frame alpha/eps = A + a(xi) + 2qD.xi it moves A by t*/eps = log(u)/s (same in
-      // every thread: the partials are replicated)
-      double As = 0.0, Bs = 0.0;
-      for (int w = 0; w < nwarp; ++w) {
-        As += (double)apart[w];
-        Bs += (double)bpart[w];
+      // cell frame alpha/eps = A + a(xi) + 2qD.xi it moves A by t*/eps = log(u)/s.  One thread
+      // computes it: the double root and logarithm on every thread kept the narrow FP64 pipe busy
+      // for most of the iteration.
+      if (tid == 0) {
+        double As = 0.0, Bs = 0.0;
+        for (int w = 0; w < nwarp; ++w) {
+          As += (double)apart[w];
+          Bs += (double)bpart[w];
+        }
+        const double uu = (a_tot + sqrt(a_tot * a_tot + 4.0 * As * Bs)) / (2.0 * Bs);
+        if (uu > 0.0 && uu < INFINITY) sk.set_A(S, A + log(uu) / sl);
       }
-      const double uu = (a_tot + sqrt(a_tot * a_tot + 4.0 * As * Bs)) / (2.0 * Bs);
-      if (uu > 0.0 && uu < INFINITY) {
-        A += log(uu) / sl;
-        sB = R(sl * (qD2 - A));
-        cA = R(-(1.0 - rr) * A);
-        gA = R(-sl * A);
-      }
+      __syncthreads();
+      A = sk.A; sB = sk.sB; cA = sk.cA; gA = sk.gA;
     }
     // accept the X-update: swap the buffers
     R* tp = av_c; av_c = av_n; av_n = tp;
@@ -642,7 +876,7 @@ __device__ __forceinline__ void cell_solve_body(const DevState& S, const CellDes
   double mubar[4] = {0.0, 0.0, 0.0, 0.0};   // balancing: mu_bar(X_q), X-marginal after one more X-half
   {
     for (int t = tid; t < nx; t += nthr) {
-      int r = t / nx2, c = t - r * nx2;
+      const int r = quot(t, nx2, inx2), c = t - r * nx2;
       int x = (cd.i0 + r) * N + cd.j0 + c;
       int xi1 = cd.i0 + r - xc1, xi2 = cd.j0 + c - xc2;
       double a = (double)av_c[t];
@@ -672,7 +906,7 @@ __device__ __forceinline__ void cell_solve_body(const DevState& S, const CellDes
       }
     }
     if (bal) block_sum<4>(mubar, red);
-    else block_sum<2>(dk, red);
+    else cell_sum<R, 2>(dk, red);
   }
 
   R hs[12];
@@ -694,9 +928,9 @@ __device__ __forceinline__ void cell_solve_body(const DevState& S, const CellDes
   for (int hc = 0; hc < nhc; ++hc) {
     const int cb = hc * s, ce = min(nx2, cb + s);
     // rows of X_J against columns of B_J, restricted to the column half hc
-    for (int t = gtid; t < nx1 * W; t += gthr) {
-      int r = t / W, ll = t - r * W;
-      const R* row = xa_c + r * nx2;
+    for (int t = tid; t < nx1 * W; t += nthr) {
+      const int r = quot(t, W, iW), ll = t - r * W;
+      const R* row = xa_c + r * xp;
       R ma, md;
       const R T2 = lse_moments<R>([&](int m) { return row[m]; }, [&](int m) { return av_c[r * nx2 + m]; },
                                   [&](int) { return R(0); }, qR, R(D2), cb, ce, R(ll + offc), q2, R(0), false, ma,
@@ -706,14 +940,14 @@ __device__ __forceinline__ void cell_solve_body(const DevState& S, const CellDes
       Md[t] = md;
     }
     csync();
-    for (int u = gtid; u < ny; u += gthr) {
-      int kk = u / W, ll = u - kk * W;
+    for (int u = tid; u < ny; u += nthr) {
+      const int kk = quot(u, W, iW), ll = u - kk * W, v = kk * Wp + ll;
       int y = (k0 + kk) * N + l0 + ll;
       R ctr = R(kk + offr);
       double nuy = S.nu[y];
       // Z of the last iteration: the log-sum-exp over all rows of the full-row
       // T, an upper bound of every quadrant's sum at this y
-      const R zsh = zok ? Zv[u] : R(0);
+      const R zsh = zok ? Zv[v] : R(0);
       for (int hr = 0; hr < nhr; ++hr) {
         const int rb = hr * s, re = min(nx1, rb + s);
         R ma, md;
@@ -721,9 +955,9 @@ __device__ __forceinline__ void cell_solve_body(const DevState& S, const CellDes
             [&](int m) { return Te[m * W + ll]; }, [&](int m) { return Ma[m * W + ll]; },
             [&](int m) { return Md[m * W + ll]; }, qR, R(D1), rb, re, ctr, q2, zsh, zok, ma, md);
         const int qd = 2 * hr + hc;
-        R nt = R(nuy) * dd_ex2(bv[u] * L2E + P2);
+        R nt = R(nuy) * dd_ex2(bv[v] * L2E + P2);
         nut[qd * nst + u] = (double)nt;
-        hs[qd] += nt * (ma + bv[u]);
+        hs[qd] += nt * (ma + bv[v]);
         hs[4 + qd] += nt * md;
         hs[8 + qd] += nt;
       }
@@ -778,7 +1012,7 @@ __device__ __forceinline__ void cell_solve_body(const DevState& S, const CellDes
         const int cb = hc * s, ce = min(nx2, cb + s);
         for (int t = tid; t < nx1 * W; t += nthr) {
           int r = t / W, ll = t - r * W;
-          const R* row = xa_c + r * nx2;
+          const R* row = xa_c + r * xp;
           R ctr = R(ll + offc);
           R T2 = lse2_1d<R>([&](int m) { return row[cb + m]; }, ce - cb, ctr - R(cb), q2, R(0), false);
           R sw = 0, sa = 0, sd = 0;
@@ -818,7 +1052,7 @@ __device__ __forceinline__ void cell_solve_body(const DevState& S, const CellDes
             const double nt = nut[qd * nst + u];
             const double rh = pick4(rho, qd);
             const double nh = rh * nt;
-            hs[qd] += R(nh * ((double)(sa * isw) + (double)bv[u] + (rh > 0.0 ? log(rh) : 0.0)));
+            hs[qd] += R(nh * ((double)(sa * isw) + (double)bv[kk * Wp + ll] + (rh > 0.0 ? log(rh) : 0.0)));
             hs[4 + qd] += R(nh * (double)(sd * isw));
             hs[8 + qd] += R(nh);
           }
@@ -837,7 +1071,8 @@ __device__ __forceinline__ void cell_solve_body(const DevState& S, const CellDes
         rho_at(u, rho);
         const double rq = pick4(rho, qd);
         const double lr = rq > 0.0 ? log2(rq) : -INFINITY;
-        Lq[u] = R(((double)bv[u] + (double)lnu[u]) * DD_LOG2E + lr);
+        const int v = u / W * Wp + u % W;
+        Lq[u] = R(((double)bv[v] + (double)lnu[v]) * DD_LOG2E + lr);
       }
       __syncthreads();
       for (int t = tid; t < H * (ce - cb); t += nthr) {
@@ -876,8 +1111,8 @@ __device__ __forceinline__ void cell_solve_body(const DevState& S, const CellDes
     __syncthreads();
   }
   // change of P_Y pi for the step-size decision
-  for (int u = gtid; u < ny; u += gthr) {
-    int kk = u / W, ll = u - kk * W;
+  for (int u = tid; u < ny; u += nthr) {
+    const int kk = quot(u, W, iW), ll = u - kk * W;
     int y1 = k0 + kk, y2 = l0 + ll;
     double dlt = 0.0;
 #pragma unroll
@@ -892,16 +1127,16 @@ __device__ __forceinline__ void cell_solve_body(const DevState& S, const CellDes
   double hsd[12];
 #pragma unroll
   for (int k = 0; k < 12; ++k) hsd[k] = (double)hs[k];
-  block_sum<12>(hsd, red);
+  cell_sum<R, 12>(hsd, red);
   if (tid == 0) {
     CellOut o;
     o.k0 = k0; o.l0 = l0; o.H = H; o.W = W;
     o.iters = it;
-    o.status = nonfinite ? CELL_NONFINITE : ((S.err >= 0.0 && gap > tol) ? CELL_MAXIT : CELL_OK);
+    o.status = nonfinite ? CELL_NONFINITE : (stops && gap > tol ? CELL_MAXIT : CELL_OK);
     o.D1 = D1; o.D2 = D2;
     o.slot = slot;
     o.usec = (int)min((dd_global_ns() - t_start) / 1000ull, 2147483647ull);
-    o.gap = gap;
+    o.gap = (double)gap;
     o.dKX[0] = dk[0]; o.dKX[1] = dk[1];
     for (int q4 = 0; q4 < 4; ++q4) {
       int bi = cd.mem[q4];
@@ -943,6 +1178,8 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
   double* red = reinterpret_cast<double*>(smem_raw);   // 32 * 16 doubles (block reductions)
   __shared__ BoxRec dbox[4];
   __shared__ int dgeo[8];
+  __shared__ int npend;
+  __shared__ CellScalars<R> sk;
   __shared__ double dx[kDistMaxC * 16];                 // partial sums of every CTA of the cluster
   CellOut* out = S.cout + cidx;
   const unsigned long long t_start = dd_global_ns();
@@ -1017,19 +1254,24 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
   const int Hl = ke - kb, nyl = Hl * W;
 
   // ------------------------------------------------------- shared layout
-  const int cap_nx = 4 * s * s;
+  // odd row pitches where they fit, as in cell_solve_body
+  const int cap_nx = 4 * s * s, cap_xp = cap_nx + 2 * s, xp = nx2 | 1, Wo = W | 1;
+  const int tszT = 2 * s * S.dist_cap_w, tszU = 2 * s * S.dist_cap_hl, Hc = (H + C - 1) / C;   // the same in every CTA
+  const int Wp = nx1 * Wo <= tszT && Hc * Wo <= S.dist_cap_nyl ? Wo : W;
+  const int Up = Hc * (nx2 | 1) <= tszU ? nx2 | 1 : nx2;
+  const float iW = 1.0f / (float)W, inx2 = 1.0f / (float)nx2;
   R* xa = reinterpret_cast<R*>(smem_raw + 32 * 16 * sizeof(double));
-  R* av = xa + cap_nx;
+  R* av = xa + cap_xp;
   R* g0 = av + cap_nx;
   R* Wv = g0 + cap_nx;       // W of the X-half, combined over the cluster
   R* lm = Wv + cap_nx;
   R* xa_nx = lm + cap_nx;
-  R* av_nx = xa_nx + cap_nx;
-  R* Wp = av_nx + cap_nx;    // own rows' part of W (the shift of the next iteration)
-  R* Wx = Wp + cap_nx;       // C x cap_nx: the parts of all CTAs
+  R* av_nx = xa_nx + cap_xp;
+  R* Wl = av_nx + cap_nx;    // own rows' part of W (the shift of the next iteration)
+  R* Wx = Wl + cap_nx;       // C x cap_nx: the parts of all CTAs
   R* T = Wx + C * cap_nx;    // nx1 x W
-  R* U = T + 2 * s * S.dist_cap_w;   // Hl x nx2
-  R* bl = U + 2 * s * S.dist_cap_hl;
+  R* U = T + tszT;           // Hl x nx2
+  R* bl = U + tszU;
   R* lrho = bl + S.dist_cap_nyl;
   R* Zv = lrho + S.dist_cap_nyl;
   R* bv = Zv + S.dist_cap_nyl;
@@ -1042,18 +1284,18 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
   {
     double m3[3] = {0.0, 0.0, 0.0};
     for (int ul = tid; ul < nyl; ul += nthr) {
-      const int kl = ul / W, ll = ul - kl * W, kk = kb + kl;
+      const int kl = quot(ul, W, iW), ll = ul - kl * W, kk = kb + kl, v = kl * Wp + ll;
       const int y1 = k0 + kk, y2 = l0 + ll, y = y1 * N + y2;
       double nuJ = 0.0;
 #pragma unroll
       for (int q4 = 0; q4 < 4; ++q4) nuJ += box_value(dbox[q4], arena, y1, y2);
       const double num = fmax(0.0, S.PY[y] - nuJ);
       const R rho = R(num) / R(S.nu[y]);
-      lrho[ul] = rho > R(0) ? dd_lg2(rho) * R(DD_LN2) : -dd_inf<R>();
-      lnu[ul] = R(S.lognu[y]);
+      lrho[v] = rho > R(0) ? dd_lg2(rho) * R(DD_LN2) : -dd_inf<R>();
+      lnu[v] = R(S.lognu[y]);
       m3[0] += nuJ; m3[1] += nuJ * kk; m3[2] += nuJ * ll;
     }
-    block_sum<3>(m3, red);
+    cell_sum<R, 3>(m3, red);
     if (tid == 0)
       for (int r = 0; r < C; ++r) {
         double* px = cl.map_shared_rank(dx, r);
@@ -1072,33 +1314,26 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
   const int yc1 = k0 + c1, yc2 = l0 + c2;
   const int D1 = xc1 - yc1, D2 = xc2 - yc2;
   const int offr = (k0 - cd.i0) + D1, offc = (l0 - cd.j0) + D2;
-  const double eps = S.eps, lam = S.lam;
-  const double q = S.h * S.h / eps;
-  const double sl = eps / lam;
-  const double rr = lam / (eps + lam);
-  const R q2 = R(q * DD_LOG2E), qR = R(q), sR = R(sl), rR = R(rr);
+  const double eps = S.eps, q = S.q, sl = S.sl;
 
   // ------------------------------------------------------- load X side (every CTA)
-  const double inv_eps = 1.0 / eps;
+  const double inv_eps = S.inv_eps;
   double acc2[2] = {0.0, 0.0};
   for (int t = tid; t < nx; t += nthr) {
-    const int r = t / nx2, c = t - r * nx2;
+    const int r = quot(t, nx2, inx2), c = t - r * nx2;
     const int x = (cd.i0 + r) * N + cd.j0 + c;
     const int xi1 = cd.i0 + r - xc1, xi2 = cd.j0 + c - xc2;
     acc2[0] += S.alpha[x] * inv_eps - 2.0 * q * (double)(D1 * xi1 + D2 * xi2);
     acc2[1] += S.mu[x];
   }
   block_sum<2>(acc2, red);
-  const double A = acc2[0] / nx;
-  const double muJ = acc2[1];
-  const double qD2 = q * (double)(D1 * D1 + D2 * D2);
-  const R sB = R(sl * (qD2 - A));
-  const R cEta1 = R(sl * 2.0 * q * D1), cEta2 = R(sl * 2.0 * q * D2);
-  const R cA = R(-(1.0 - rr) * A);
-  const R gA = R(-sl * A);
-  const R cD1 = R(2.0 * (1.0 - rr) * q * D1), cD2 = R(2.0 * (1.0 - rr) * q * D2);
+  if (tid == 0) sk.set(S, D1, D2, acc2[0] / nx, acc2[1]);
+  __syncthreads();
+  const double A = sk.A;
+  const R q2 = sk.q2, qR = sk.qR, sR = sk.sR, rR = sk.rR, sB = sk.sB, cEta1 = sk.cEta1, cEta2 = sk.cEta2, cA = sk.cA,
+          gA = sk.gA, cD1 = sk.cD1, cD2 = sk.cD2, tol = sk.tol;
   for (int t = tid; t < nx; t += nthr) {
-    const int r = t / nx2, c = t - r * nx2;
+    const int r = quot(t, nx2, inx2), c = t - r * nx2;
     const int x = (cd.i0 + r) * N + cd.j0 + c;
     const int xi1 = cd.i0 + r - xc1, xi2 = cd.j0 + c - xc2;
     const double lin = 2.0 * q * (double)(D1 * xi1 + D2 * xi2);
@@ -1107,131 +1342,115 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
     av[t] = a;
     lm[t] = l;
     g0[t] = R(-sl * lin);
-    xa[t] = (a + l) * R(DD_LOG2E);
+    xa[r * xp + c] = (a + l) * R(DD_LOG2E);
   }
   __syncthreads();
 
   // ------------------------------------------------------- Sinkhorn loop
-  const double tol = S.err * muJ;
   const R LN2 = R(DD_LN2), L2E = R(DD_LOG2E);
+  const bool stops = S.err >= 0.0;
+  int* pend = reinterpret_cast<int*>(red + 256);    // as in cell_solve_body
+  const int lock = sizeof(R) == 4 ? kLock : S.newton_maxit;
   int it = 0;
-  double gap = 0.0;
+  R gap = R(0);
   bool first = true;
   R *xa_c = xa, *av_c = av, *xa_n = xa_nx, *av_n = av_nx;
   for (;;) {
     ++it;
+    if (tid == 0) npend = 0;
     // Y-half, T(r, ll) = log2 sum_c 2^{xa(r,c) - q2 (c - ll - offc)^2}: split, to every CTA
-    {
-      const int nt = nx1 * W, P = lanes_per_target(nt, nx2, gthr), ni = (nt * P + 31) & ~31;
-      for (int i = gtid; i < ni; i += gthr) {
-        const int tg0 = i / P, part = i - tg0 * P, tg = min(tg0, nt - 1);
-        const int r = tg / W, ll = tg - r * W;
-        const R* row = xa_c + r * nx2;
-        const R v = lse2_group<R>([&](int m) { return row[m]; }, nx2, R(ll + offc), q2, T[tg], !first, part, P);
-        __syncwarp();
-        if (part == 0 && tg0 < nt)
-          for (int rk = 0; rk < C; ++rk) *cl.map_shared_rank(T + tg, rk) = v;
+    run_pass(xa_c, xp, 1, T, Wp, 1, nx1, W, nx2, offc, q2, first, gtid, gthr,
+             [&](int r, int ll, int n, const auto& v) {
+      for (int rk = 0; rk < C; ++rk) {
+        R* Tr = cl.map_shared_rank(T, rk);
+        for (int k = 0; k < n; ++k) Tr[r * Wp + ll + k] = v[k];
       }
-    }
+    });
     csync();
     // Y-half on the own rows: Z(kk, ll) = log2 sum_r 2^{T(r,ll) - q2 (r - kk - offr)^2}, Newton (a3)
-    if (nyl * 2 > nthr) {
-      const int rounds = (nyl + 2 * nthr - 1) / (2 * nthr);
-      for (int rd = 0; rd < rounds; ++rd) {
-        const int u = tid + rd * 2 * nthr;
-        const int uu[2] = {min(u, nyl - 1), min(u + nthr, nyl - 1)};
-        const bool ok[2] = {u < nyl, u + nthr < nyl};
-        R lr[2], c0[2], uw[2], root[2], Zn[2];
+    const bool fused_y = sizeof(R) == 4 && nyl * 2 > nthr;
+    auto y_store = [&](int v, R u, R Zx) {   // as in cell_solve_body
+      const R b = fused_y ? u - Zx : fma(-Zx, LN2, u);
+      Zv[v] = fused_y ? mul_rn(Zx, L2E) : Zx;
+      bv[v] = b;
+      bl[v] = (b + lnu[v]) * L2E;
+    };
+    auto y_root = [&](int ll, int kl, int n, const auto& Z2) {
+      constexpr int B = sizeof(Z2) / sizeof(R);
+      R lr[B], c0[B], uw[B], root[B], Zn[B];
+      const R eta2 = R(l0 + ll - yc2);
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-          const int kl = uu[k] / W, ll = uu[k] - kl * W, kk = kb + kl;
-          const R Z2 =
-              lse2_group<R>([&](int m) { return T[m * W + ll]; }, nx1, R(kk + offr), q2, Zv[uu[k]], !first, 0, 1);
-          Zn[k] = Z2 * LN2;
-          const R eta1 = R(k0 + kk - yc1), eta2 = R(l0 + ll - yc2);
-          c0[k] = sB - cEta1 * eta1 - cEta2 * eta2 - sR * Zn[k];
-          lr[k] = lrho[uu[k]];
-          uw[k] = first ? dd_inf<R>() : bv[uu[k]] + Zn[k];
-        }
-        newton_u2<R>(lr, c0, uw, sR, S.newton_maxit, root);
-        __syncwarp();
+      for (int k = 0; k < B; ++k) {
+        const int v = (kl + min(k, n - 1)) * Wp + ll;
+        Zn[k] = mul_rn(k < n ? Z2[k] : Z2[0], LN2);
+        const R eta1 = R(k0 + kb + kl + min(k, n - 1) - yc1);
+        c0[k] = sB - cEta1 * eta1 - cEta2 * eta2 - sR * Zn[k];
+        lr[k] = lrho[v];
+        uw[k] = first ? dd_inf<R>() : bv[v] + Zn[k];
+      }
+      bool open[B];
+      newton_tile<R, B>(lr, c0, uw, sR, min(S.newton_maxit, lock), root, open);
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-          if (!ok[k]) continue;
-          Zv[uu[k]] = Zn[k] * L2E;
-          const R b = root[k] - Zn[k];
-          bv[uu[k]] = b;
-          bl[uu[k]] = (b + lnu[uu[k]]) * L2E;
+      for (int k = 0; k < B; ++k) {
+        if (k >= n) break;
+        if (lock < S.newton_maxit && open[k]) {
+          const int v = (kl + k) * Wp + ll, e = atomicAdd(&npend, 1);
+          if (e < kPend) {   // finished below from the list
+            pend[e] = v;
+            bv[v] = root[k];
+            Zv[v] = fused_y ? Zn[k] : Z2[k];
+            continue;
+          }
+          root[k] = newton_rest(lr[k], c0[k], root[k], sR, S.newton_maxit - lock);
         }
+        y_store((kl + k) * Wp + ll, root[k], fused_y ? Zn[k] : Z2[k]);
+      }
+    };
+    if constexpr (sizeof(R) == 4) {
+      run_pass(T, 1, Wp, Zv, 1, Wp, W, Hl, nx1, offr + kb, q2, first, tid, nthr, y_root);
+      __syncthreads();
+      const int np = min(npend, kPend);
+      const float iWp = 1.0f / (float)Wp;
+      for (int e = tid; e < np; e += nthr) {
+        const int v = pend[e], kl = quot(v, Wp, iWp), ll = v - kl * Wp;
+        const R Zx = Zv[v], Zn = fused_y ? Zx : mul_rn(Zx, LN2);
+        const R eta1 = R(k0 + kb + kl - yc1), eta2 = R(l0 + ll - yc2);
+        const R c0 = sB - cEta1 * eta1 - cEta2 * eta2 - sR * Zn;
+        y_store(v, newton_rest(lrho[v], c0, bv[v], sR, S.newton_maxit - lock), Zx);
       }
     } else {
-      const int P = lanes_per_target(nyl, nx1, nthr), ni = (nyl * P + 31) & ~31;
-      for (int i = tid; i < ni; i += nthr) {
-        const int u0 = i / P, part = i - u0 * P, u = min(u0, nyl - 1);
-        const int kl = u / W, ll = u - kl * W, kk = kb + kl;
-        const R Z2 = lse2_group<R>([&](int m) { return T[m * W + ll]; }, nx1, R(kk + offr), q2, Zv[u], !first,
-                                   part, P);
-        __syncwarp();
-        if (part == 0 && u0 < nyl) Zv[u] = Z2;
-      }
+      run_pass(T, 1, Wp, Zv, 1, Wp, W, Hl, nx1, offr + kb, q2, first, tid, nthr,
+               [&](int ll, int kl, int, const auto& v) { Zv[kl * Wp + ll] = v[0]; });
       __syncthreads();
-      for (int u = tid; u < nyl; u += 2 * nthr) {
-        const int uu[2] = {u, min(u + nthr, nyl - 1)};
-        R lr[2], c0[2], uw[2], root[2];
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-          const int kl = uu[k] / W, ll = uu[k] - kl * W, kk = kb + kl;
-          const R Zn = Zv[uu[k]] * LN2;
-          const R eta1 = R(k0 + kk - yc1), eta2 = R(l0 + ll - yc2);
-          c0[k] = sB - cEta1 * eta1 - cEta2 * eta2 - sR * Zn;
-          lr[k] = lrho[uu[k]];
-          uw[k] = first ? dd_inf<R>() : bv[uu[k]] + Zn;
-        }
-        newton_u2<R>(lr, c0, uw, sR, S.newton_maxit, root);
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-          if (k == 1 && u + nthr >= nyl) break;
-          const R b = root[k] - Zv[uu[k]] * LN2;
-          bv[uu[k]] = b;
-          bl[uu[k]] = (b + lnu[uu[k]]) * L2E;
-        }
+      for (int ul = tid; ul < nyl; ul += nthr) {
+        const int kl = quot(ul, W, iW), ll = ul - kl * W;
+        const R z[1] = {Zv[kl * Wp + ll]};
+        y_root(ll, kl, 1, z);
       }
     }
     __syncthreads();
     // X-half on the own rows: U(kl, c) = log2 sum_ll 2^{bl(kl,ll) - q2 (ll - (c - offc))^2}
-    {
-      const int nt = Hl * nx2, P = lanes_per_target(nt, W, nthr), ni = (nt * P + 31) & ~31;
-      for (int i = tid; i < ni; i += nthr) {
-        const int tg0 = i / P, part = i - tg0 * P, tg = min(tg0, nt - 1);
-        const int kl = tg / nx2, c = tg - kl * nx2;
-        const R* row = bl + kl * W;
-        const R v = lse2_group<R>([&](int m) { return row[m]; }, W, R(c - offc), q2, U[tg], !first, part, P);
-        __syncwarp();
-        if (part == 0 && tg0 < nt) U[tg] = v;
-      }
-    }
+    run_pass(bl, Wp, 1, U, Up, 1, Hl, nx2, W, -offc, q2, first, tid, nthr, [&](int kl, int c, int n, const auto& v) {
+      for (int k = 0; k < n; ++k) U[kl * Up + c + k] = v[k];
+    });
     __syncthreads();
     // the own rows' part of W(r, c) = log2 sum_kk 2^{U(kk,c) - q2 (kk - (r - offr))^2}, to every CTA
     if (Hl > 0) {
-      const int P = lanes_per_target(nx, Hl, nthr), ni = (nx * P + 31) & ~31;
-      for (int i = tid; i < ni; i += nthr) {
-        const int tg0 = i / P, part = i - tg0 * P, t = min(tg0, nx - 1);
-        const int r = t / nx2, c = t - r * nx2;
-        const R v = lse2_group<R>([&](int m) { return U[m * nx2 + c]; }, Hl, R(r - offr - kb), q2, Wp[t], !first,
-                                  part, P);
-        __syncwarp();
-        if (part == 0 && tg0 < nx) {
-          Wp[t] = v;
-          for (int rk = 0; rk < C; ++rk) *cl.map_shared_rank(Wx + crank * cap_nx + t, rk) = v;
+      run_pass(U, 1, Up, Wl, 1, nx2, nx2, nx1, Hl, -offr - kb, q2, first, tid, nthr,
+               [&](int c, int r0, int n, const auto& v) {
+        for (int k = 0; k < n; ++k) Wl[(r0 + k) * nx2 + c] = v[k];
+        for (int rk = 0; rk < C; ++rk) {
+          R* Wr = cl.map_shared_rank(Wx + crank * cap_nx, rk);
+          for (int k = 0; k < n; ++k) Wr[(r0 + k) * nx2 + c] = v[k];
         }
-      }
+      });
     } else {
       for (int t = tid; t < nx; t += nthr)
         for (int rk = 0; rk < C; ++rk) *cl.map_shared_rank(Wx + crank * cap_nx + t, rk) = -dd_inf<R>();
     }
     csync();
     // combine the parts (rank order: every CTA gets the same W), gap terms (a4), next alpha (a2)
-    double gl = 0.0;
+    R gl = R(0);
     for (int t = tid; t < nx; t += nthr) {
       R mx = -dd_inf<R>();
       for (int rk = 0; rk < C; ++rk) mx = max(mx, Wx[rk * cap_nx + t]);
@@ -1242,23 +1461,27 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
         W2 = mx + dd_lg2(acc);
       }
       Wv[t] = W2;
-      const int r = t / nx2, c = t - r * nx2;
+      const int r = quot(t, nx2, inx2), c = t - r * nx2;
       const R a = av_c[t];
       const R tt = a + W2 * LN2;         // log(P_X pi / mu)
       const R g = gA + g0[t] - sR * a;   // -alpha/lam
-      gl += (double)(dd_ex2((lm[t] + g) * L2E) * dd_psi<R>(tt - g));
+      gl += dd_ex2((lm[t] + g) * L2E) * dd_psi<R>(tt - g);
       const R xi1 = R(cd.i0 + r - xc1), xi2 = R(cd.j0 + c - xc2);
       const R an = cA - rR * W2 * LN2 - cD1 * xi1 - cD2 * xi2;
       av_n[t] = an;
-      xa_n[t] = (an + lm[t]) * L2E;
+      xa_n[r * xp + c] = (an + lm[t]) * L2E;
     }
     {
-      double gv[1] = {gl};
-      block_sum<1>(gv, red);
-      gap = gv[0];
+      // every CTA adds the same values in the same order
+      R* gpart = reinterpret_cast<R*>(red);
+      gl = warp_sum(gl);
+      if ((tid & 31) == 0) gpart[tid >> 5] = gl;
+      __syncthreads();
+      gap = R(0);
+      for (int w = 0; w < (nthr >> 5); ++w) gap += gpart[w];
     }
     first = false;
-    if ((S.err >= 0.0 && gap <= tol) || it >= S.maxit || !(gap == gap)) break;
+    if ((stops && gap <= tol) || it >= S.maxit || !(gap == gap)) break;
     R* tp = av_c; av_c = av_n; av_n = tp;
     tp = xa_c; xa_c = xa_n; xa_n = tp;
   }
@@ -1269,7 +1492,7 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
   double dk[2] = {0.0, 0.0};
   if (crank == 0) {
     for (int t = tid; t < nx; t += nthr) {
-      const int r = t / nx2, c = t - r * nx2;
+      const int r = quot(t, nx2, inx2), c = t - r * nx2;
       const int x = (cd.i0 + r) * N + cd.j0 + c;
       const int xi1 = cd.i0 + r - xc1, xi2 = cd.j0 + c - xc2;
       S.alphanew[x] = eps * (A + (double)av_c[t] + 2.0 * q * (double)(D1 * xi1 + D2 * xi2));
@@ -1287,7 +1510,7 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
         dk[1] += kl_change_f(p0, th_s * (p1 - p0), lm[t]);
       }
     }
-    block_sum<2>(dk, red);
+    cell_sum<R, 2>(dk, red);
   }
   R hs[12];
 #pragma unroll
@@ -1309,8 +1532,8 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
   for (int hc = 0; hc < nhc; ++hc) {
     const int cb = hc * s, ce = min(nx2, cb + s);
     for (int t = gtid; t < nx1 * W; t += gthr) {
-      const int r = t / W, ll = t - r * W;
-      const R* row = xa_c + r * nx2;
+      const int r = quot(t, W, iW), ll = t - r * W;
+      const R* row = xa_c + r * xp;
       R ma, md;
       const R T2 = lse_moments<R>([&](int m) { return row[m]; }, [&](int m) { return av_c[r * nx2 + m]; },
                                   [&](int) { return R(0); }, qR, R(D2), cb, ce, R(ll + offc), q2, R(0), false, ma,
@@ -1323,12 +1546,12 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
     }
     csync();
     for (int ul = tid; ul < nyl; ul += nthr) {
-      const int kl = ul / W, ll = ul - kl * W, kk = kb + kl;
+      const int kl = quot(ul, W, iW), ll = ul - kl * W, kk = kb + kl, v = kl * Wp + ll;
       const int u = kk * W + ll;
       const int y = (k0 + kk) * N + l0 + ll;
       const R ctr = R(kk + offr);
       const double nuy = S.nu[y];
-      const R zsh = zok ? Zv[ul] : R(0);   // the final Z: an upper bound of every quadrant's sum
+      const R zsh = zok ? Zv[v] : R(0);   // the final Z: an upper bound of every quadrant's sum
       for (int hr = 0; hr < nhr; ++hr) {
         const int rb = hr * s, re = min(nx1, rb + s);
         R ma, md;
@@ -1336,9 +1559,9 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
             [&](int m) { return Te[m * W + ll]; }, [&](int m) { return Ma[m * W + ll]; },
             [&](int m) { return Md[m * W + ll]; }, qR, R(D1), rb, re, ctr, q2, zsh, zok, ma, md);
         const int qd = 2 * hr + hc;
-        const R ntv = R(nuy) * dd_ex2(bv[ul] * L2E + P2);
+        const R ntv = R(nuy) * dd_ex2(bv[v] * L2E + P2);
         nut[qd * nst + u] = (double)ntv;
-        hs[qd] += ntv * (ma + bv[ul]);
+        hs[qd] += ntv * (ma + bv[v]);
         hs[4 + qd] += ntv * md;
         hs[8 + qd] += ntv;
       }
@@ -1347,7 +1570,7 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
   }
   // change of P_Y pi for the step-size decision (own rows)
   for (int ul = tid; ul < nyl; ul += nthr) {
-    const int kl = ul / W, ll = ul - kl * W, kk = kb + kl;
+    const int kl = quot(ul, W, iW), ll = ul - kl * W, kk = kb + kl;
     const int u = kk * W + ll;
     const int y1 = k0 + kk, y2 = l0 + ll;
     double dlt = 0.0;
@@ -1363,7 +1586,7 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
   double hsd[12];
 #pragma unroll
   for (int k = 0; k < 12; ++k) hsd[k] = (double)hs[k];
-  block_sum<12>(hsd, red);
+  cell_sum<R, 12>(hsd, red);
   if (tid == 0) {
     double* p0 = cl.map_shared_rank(dx, 0);
     for (int k = 0; k < 12; ++k) p0[crank * 16 + k] = hsd[k];
@@ -1378,11 +1601,11 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
   CellOut o;
   o.k0 = k0; o.l0 = l0; o.H = H; o.W = W;
   o.iters = it;
-  o.status = nonfinite ? CELL_NONFINITE : ((S.err >= 0.0 && gap > tol) ? CELL_MAXIT : CELL_OK);
+  o.status = nonfinite ? CELL_NONFINITE : (stops && gap > tol ? CELL_MAXIT : CELL_OK);
   o.D1 = D1; o.D2 = D2;
   o.slot = slot;
   o.usec = (int)min((dd_global_ns() - t_start) / 1000ull, 2147483647ull);
-  o.gap = gap;
+  o.gap = (double)gap;
   o.dKX[0] = dk[0]; o.dKX[1] = dk[1];
   for (int q4 = 0; q4 < 4; ++q4) {
     const int bi = cd.mem[q4];
@@ -1697,14 +1920,14 @@ k_ref_order(const DevState* __restrict__ states, const CellRef* __restrict__ ref
 size_t cell_smem_bytes(int s, int cap_side, int cap_ny, int precision) {
   size_t rs = precision ? sizeof(double) : sizeof(float);
   size_t cap_nx = 4 * (size_t)s * s, tsz = 2 * (size_t)s * cap_side;
-  return 32 * 16 * sizeof(double) + rs * (7 * cap_nx + 2 * tsz + 5 * (size_t)cap_ny);
+  return 32 * 16 * sizeof(double) + rs * (7 * cap_nx + 4 * (size_t)s + 2 * tsz + 5 * (size_t)cap_ny);
 }
 
 // Shared memory of the cluster-distributed layout (cell_solve_dist).
 size_t dist_smem_bytes(int s, int C, int cap_w, int cap_hl, int cap_nyl, int precision) {
   const size_t rs = precision ? sizeof(double) : sizeof(float), cap_nx = 4 * (size_t)s * s;
   return 32 * 16 * sizeof(double) +
-         rs * ((8 + (size_t)C) * cap_nx + 2 * (size_t)s * cap_w + 2 * (size_t)s * cap_hl + 5 * (size_t)cap_nyl);
+         rs * ((8 + (size_t)C) * cap_nx + 4 * (size_t)s + 2 * (size_t)s * cap_w + 2 * (size_t)s * cap_hl + 5 * (size_t)cap_nyl);
 }
 
 // Static shared memory of the cell kernels, the larger of the single- and the

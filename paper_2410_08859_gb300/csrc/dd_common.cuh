@@ -54,6 +54,7 @@ struct BoxRec {
 struct DevState {
   int N, s, nb, nbasic;
   double h, eps, lam, thr, err, tau;
+  double inv_eps, q, sl, rr;    // 1/eps, h^2/eps, eps/lam, lam/(eps+lam): set with eps (set_eps_scalars)
   int maxit, newton_maxit, strategy, margin;
   int ti;                       // translation step after each cell X-half (0/1)
   double* line;                 // GetWeights_line state (16 doubles)
@@ -103,6 +104,14 @@ struct DevState {
   int dist_cap_hl;              // largest number of Y rows per CTA
   int dist_cap_nyl;             // largest number of Y points per CTA
 };
+
+inline void set_eps_scalars(DevState& S, double eps) {
+  S.eps = eps;
+  S.inv_eps = 1.0 / eps;
+  S.q = S.h * S.h / eps;
+  S.sl = eps / S.lam;
+  S.rr = S.lam / (eps + S.lam);
+}
 
 #define DD_LOGCAP 4096          // decision-log records kept per instance
 
@@ -227,14 +236,44 @@ __device__ __forceinline__ void block_sum(T (&v)[K], T* scratch) {
 #pragma unroll
     for (int k = 0; k < K; ++k) scratch[wid * K + k] = v[k];
   __syncthreads();
-  if (wid == 0) {
+  // warp k (mod the number of warps) combines the partials of value k in a fixed order
+  for (int k = wid; k < K; k += nw) {
+    T a = lane < nw ? scratch[lane * K + k] : T(0);
+    a = warp_sum(a);
+    if (lane == 0) scratch[32 * K + k] = a;
+  }
+  __syncthreads();
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
-      T a = lane < nw ? scratch[lane * K + k] : T(0);
-      // fixed-order pairwise combination across the lanes
-      a = warp_sum(a);
-      if (lane == 0) scratch[32 * K + k] = a;
+  for (int k = 0; k < K; ++k) v[k] = scratch[32 * K + k];
+  __syncthreads();
+}
+
+// block_sum of doubles carried as unevaluated sums of two floats through the warp
+// shuffles (TwoSum, Knuth): 48 bits of the running sum on the FP32 pipe, where
+// the double shuffles of 16 warps take 16 clocks an addition on the FP64 pipe
+// (12 values: 27 k clocks before, 4 k now).  For finite values within float range
+// (smaller than 2^-126: flushed).
+template <int K>
+__device__ __forceinline__ void block_sum_ff(double (&v)[K], double* scratch) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    float hi = (float)v[k], lo = (float)(v[k] - (double)hi);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const float h2 = __shfl_xor_sync(0xffffffffu, hi, o), l2 = __shfl_xor_sync(0xffffffffu, lo, o);
+      const float s = __fadd_rn(hi, h2), b = __fsub_rn(s, hi);
+      const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(h2, b));
+      lo = __fadd_rn(__fadd_rn(lo, l2), e);
+      hi = s;
     }
+    if (lane == 0) scratch[wid * K + k] = (double)hi + (double)lo;
+  }
+  __syncthreads();
+  for (int k = wid; k < K; k += nw) {
+    double a = lane < nw ? scratch[lane * K + k] : 0.0;
+    a = warp_sum(a);
+    if (lane == 0) scratch[32 * K + k] = a;
   }
   __syncthreads();
 #pragma unroll
