@@ -528,7 +528,9 @@ struct CellScalars {
 
 // One composite cell on one CTA: cell `cd` at position `cidx` of a sub-batch
 // of `nbatch` cells.
-template <typename R>
+// BAL: with the balancing step (an instance of its own: its registers cost the plain
+// solve spills).
+template <typename R, bool BAL>
 __device__ __forceinline__ void cell_solve_body(const DevState& S, const CellDesc cd, int cidx, int nbatch,
                                                 unsigned char* smem_raw) {
   namespace cg = cooperative_groups;
@@ -606,9 +608,14 @@ __device__ __forceinline__ void cell_solve_body(const DevState& S, const CellDes
   const bool spilled = slot >= 0;
   const int tsz = spilled ? 2 * s * N : 2 * s * S.cap_side;
   const int cap_ny = spilled ? N * N : S.cap_ny;
-  const int Wo = W | 1;
-  const int Wp = !spilled && nx1 * Wo <= tsz && H * Wo <= cap_ny && 3 * nx1 * Wo <= 2 * tsz + 3 * cap_ny ? Wo : W;
-  const int Up = !spilled && H * (nx2 | 1) <= tsz ? nx2 | 1 : nx2;
+  const int Wo = W | 1, Uo = nx2 | 1;
+  // A spilled box keeps T, U and beta + log nu, which the passes read many times,
+  // in shared memory if those fit; the arrays that each y touches once an
+  // iteration stay in the slot (143 x 81 at s = 8: 3200 -> 1500 kclk a solve).
+  const int rsz = 4 * s * S.cap_side + 5 * S.cap_ny;
+  const bool hyb = spilled && nx1 * Wo + H * Uo + H * Wo <= rsz && 3 * nx1 * W <= rsz && H * Wo <= N * N;
+  const int Wp = hyb || (!spilled && nx1 * Wo <= tsz && H * Wo <= cap_ny && 3 * nx1 * Wo <= rsz) ? Wo : W;
+  const int Up = hyb || (!spilled && H * Uo <= tsz) ? Uo : nx2;
   R* xa = reinterpret_cast<R*>(smem_raw + 32 * 16 * sizeof(double));
   R* av = xa + cap_xp;
   R* g0 = av + cap_nx;
@@ -616,10 +623,11 @@ __device__ __forceinline__ void cell_solve_body(const DevState& S, const CellDes
   R* lm = Wv + cap_nx;
   R* xa_nx = lm + cap_nx;    // next iterate of xa / a (double buffer of the X-update)
   R* av_nx = xa_nx + cap_xp;
-  R* T = spilled ? reinterpret_cast<R*>(S.spill + (long long)slot * S.spill_stride) : av_nx + cap_nx;
-  R* U = T + tsz;
-  R* bl = U + tsz;
-  R* lrho = bl + cap_ny;
+  R* gslot = spilled ? reinterpret_cast<R*>(S.spill + (long long)slot * S.spill_stride) : nullptr;
+  R* T = spilled && !hyb ? gslot : av_nx + cap_nx;
+  R* U = T + (hyb ? nx1 * Wp : tsz);
+  R* bl = U + (hyb ? H * Up : tsz);
+  R* lrho = hyb ? gslot : bl + cap_ny;
   R* Zv = lrho + cap_ny;
   R* bv = Zv + cap_ny;
   R* lnu = bv + cap_ny;
@@ -870,7 +878,7 @@ __device__ __forceinline__ void cell_solve_body(const DevState& S, const CellDes
   // ------------------------------------------------------- epilogue (a5)
   // alpha, P_X of the new plan and the KL_X change: first CTA only.  With
   // balancing (one CTA per cell) P_X and the KL_X change follow the balancing.
-  const bool bal = S.balance;
+  constexpr bool bal = BAL;
   const double th_s = 1.0 / nbatch;
   double dk[2] = {0.0, 0.0};
   double mubar[4] = {0.0, 0.0, 0.0, 0.0};   // balancing: mu_bar(X_q), X-marginal after one more X-half
@@ -924,7 +932,7 @@ __device__ __forceinline__ void cell_solve_body(const DevState& S, const CellDes
   R* Ma = T + nx1 * W;
   R* Md = Ma + nx1 * W;
   // Zv (the final Z) serves as the shift of the quadrant sums unless Md reaches it
-  const bool zok = Md + nx1 * W <= Zv;
+  const bool zok = hyb || Md + nx1 * W <= Zv;
   for (int hc = 0; hc < nhc; ++hc) {
     const int cb = hc * s, ce = min(nx2, cb + s);
     // rows of X_J against columns of B_J, restricted to the column half hc
@@ -965,7 +973,7 @@ __device__ __forceinline__ void cell_solve_body(const DevState& S, const CellDes
     __threadfence();
     csync();
   }
-  if (bal) {
+  if constexpr (bal) {
     // ---- balancing (Section 5.3, Eq. balancing): targets m_q = mu_bar(X_q) |nu_J| / mu_bar(X_J);
     // donors scale their rows by m_q/|nu_q|, receivers by 1 + D(y) w_q / nu_q(y) with the donated
     // field D(y) = sum_d (|nu_d| - m_d) nu_d(y)/|nu_d| and w_q = deficit_q / total excess.
@@ -1168,6 +1176,21 @@ __device__ __forceinline__ void cell_solve_body(const DevState& S, const CellDes
 //           hold the same W, gap and next alpha) -- no further exchange.
 // The epilogue splits the rows-of-X pass the same way and sums the
 // per-quadrant terms of the own rows; the first CTA adds the cluster's sums.
+// Whether a cell with Y box H x W fits the shared memory of a cluster of C CTAs.
+__device__ __forceinline__ bool fits_cluster(const DevState& S, int H, int W, int C) {
+  const int hl = (H + C - 1) / C;
+  return C > 1 && C <= S.dist_c && H >= C && W <= S.dist_cap_w && hl <= S.dist_cap_hl && hl * W <= S.dist_cap_nyl;
+}
+// Whether it does with the per-y arrays in a spill slot: T, U and beta + log nu,
+// and the epilogue's three rows-of-X arrays, share the cluster layout's space.
+// (234 x 257 at s = 16: 4.65 ms on one CTA from its slot, 0.5 ms so on eight.)
+__device__ __forceinline__ bool fits_hybrid(const DevState& S, int nx1, int nx2, int H, int W, int C) {
+  if (C < 2 || C > S.dist_c || H < C || S.spill_slots <= 0) return false;
+  const long long Wo = W | 1, Hc = (H + C - 1) / C;
+  const long long room = 2LL * S.s * S.dist_cap_w + 2LL * S.s * S.dist_cap_hl + 5LL * S.dist_cap_nyl;
+  return nx1 * Wo + Hc * (nx2 | 1) + Hc * Wo <= room && 3LL * nx1 * W <= room && H * Wo <= (long long)S.N * S.N;
+}
+
 constexpr int kDistMaxC = 8;
 
 template <typename R>
@@ -1216,10 +1239,10 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
     dgeo[0] = k0; dgeo[1] = l0; dgeo[2] = H; dgeo[3] = W;
     if (crank == 0) {
       int slot = -1;
-      const int hl = (H + C - 1) / C;
-      if (st == CELL_OK && (H < C || W > S.dist_cap_w || hl > S.dist_cap_hl || hl * W > S.dist_cap_nyl))
+      const bool fits = fits_cluster(S, H, W, C);
+      if (st == CELL_OK && !fits && !fits_hybrid(S, nx1, nx2, H, W, C))
         st = CELL_TOOBIG;   // excluded by k_cell_order; kept as a guard
-      if (st == CELL_OK && H * W > S.cap_nut) {
+      if (st == CELL_OK && (!fits || H * W > S.cap_nut)) {
         const int sl = S.spill_slots > 0 ? (int)atomicAdd(S.spill_count, 1u) : S.spill_slots;
         if (sl >= S.spill_slots) st = CELL_TOOBIG;
         else slot = sl;
@@ -1256,9 +1279,11 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
   // ------------------------------------------------------- shared layout
   // odd row pitches where they fit, as in cell_solve_body
   const int cap_nx = 4 * s * s, cap_xp = cap_nx + 2 * s, xp = nx2 | 1, Wo = W | 1;
-  const int tszT = 2 * s * S.dist_cap_w, tszU = 2 * s * S.dist_cap_hl, Hc = (H + C - 1) / C;   // the same in every CTA
-  const int Wp = nx1 * Wo <= tszT && Hc * Wo <= S.dist_cap_nyl ? Wo : W;
-  const int Up = Hc * (nx2 | 1) <= tszU ? nx2 | 1 : nx2;
+  const int Uo = nx2 | 1, Hc = (H + C - 1) / C;   // the same in every CTA
+  const bool hyb = !fits_cluster(S, H, W, C);     // then fits_hybrid
+  const int tszT = hyb ? nx1 * Wo : 2 * s * S.dist_cap_w, tszU = hyb ? Hc * Uo : 2 * s * S.dist_cap_hl;
+  const int Wp = hyb || (nx1 * Wo <= tszT && Hc * Wo <= S.dist_cap_nyl) ? Wo : W;
+  const int Up = hyb || Hc * Uo <= tszU ? Uo : nx2;
   const float iW = 1.0f / (float)W, inx2 = 1.0f / (float)nx2;
   R* xa = reinterpret_cast<R*>(smem_raw + 32 * 16 * sizeof(double));
   R* av = xa + cap_xp;
@@ -1272,10 +1297,13 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
   R* T = Wx + C * cap_nx;    // nx1 x W
   R* U = T + tszT;           // Hl x nx2
   R* bl = U + tszU;
-  R* lrho = bl + S.dist_cap_nyl;
-  R* Zv = lrho + S.dist_cap_nyl;
-  R* bv = Zv + S.dist_cap_nyl;
-  R* lnu = bv + S.dist_cap_nyl;
+  // a box beyond the cluster's shared memory: the arrays that each y touches once
+  // an iteration lie in the cell's spill slot, the own rows from kb on
+  R* lrho = hyb ? reinterpret_cast<R*>(S.spill + (long long)slot * S.spill_stride) + kb * Wp : bl + S.dist_cap_nyl;
+  const int capy = hyb ? N * N : S.dist_cap_nyl;
+  R* Zv = lrho + capy;
+  R* bv = Zv + capy;
+  R* lnu = bv + capy;
 
   // ------------------------------------------------- load Y side (a1), own rows
   // rho = max(0, P_Y - nu_J)/nu and log nu; the barycentre of nu_J (the Y frame
@@ -1528,7 +1556,7 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
   R* Te = T;
   R* Ma = T + nx1 * W;
   R* Md = Ma + nx1 * W;
-  const bool zok = Md + nx1 * W <= Zv;   // Zv (the final Z, own rows) is intact: the quadrant sums' shift
+  const bool zok = hyb || Md + nx1 * W <= Zv;   // Zv (the final Z, own rows) is intact: the quadrant sums' shift
   for (int hc = 0; hc < nhc; ++hc) {
     const int cb = hc * s, ce = min(nx2, cb + s);
     for (int t = gtid; t < nx1 * W; t += gthr) {
@@ -1628,7 +1656,7 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
 // classified the cells for it); `cluster`: this launch's -- crun for the main
 // grid, 1 for a helper grid that runs phase 2 only on the SMs the clusters
 // leave idle (both take phase-2 cells from the same queue).
-template <typename R>
+template <typename R, bool BAL>
 __global__ void __launch_bounds__(kCellThreads, 1)
 k_cell_solve(DevState S, const CellDesc* __restrict__ cells, const int* __restrict__ order,
              const int* __restrict__ nbig_p, int begin, int nbatch, int crun, int cluster) {
@@ -1667,7 +1695,7 @@ k_cell_solve(DevState S, const CellDesc* __restrict__ cells, const int* __restri
     const int j = nbig + sj;
     if (j >= nbatch) break;
     const int cidx = order ? order[begin + j] : j;
-    cell_solve_body<R>(S, cells[begin + cidx], cidx, nbatch, smem_raw);
+    cell_solve_body<R, BAL>(S, cells[begin + cidx], cidx, nbatch, smem_raw);
   }
 }
 
@@ -1695,12 +1723,9 @@ __device__ __forceinline__ unsigned int cell_cost(const DevState& S, const CellD
   return (unsigned int)min(c + 1, 0x7fffffffLL);
 }
 
-// Whether a cell with Y box H x W fits a cluster of the layout's largest size
-// (S.dist_c CTAs, each holding a block of ceil(H / dist_c) rows).
+// Whether it fits a cluster of the layout's largest size.
 __device__ __forceinline__ bool fits_layout(const DevState& S, int H, int W) {
-  if (S.dist_c < 2) return false;
-  const int hl = (H + S.dist_c - 1) / S.dist_c;
-  return H >= S.dist_c && W <= S.dist_cap_w && hl <= S.dist_cap_hl && hl * W <= S.dist_cap_nyl;
+  return fits_cluster(S, H, W, S.dist_c);
 }
 
 constexpr int kOrderMax = 4096;   // largest batch sorted (larger ones keep their index order)
@@ -1749,10 +1774,9 @@ __global__ void __launch_bounds__(1024) k_cell_order(DevState S, int part, int m
     if (i < n) {
       int H, W;
       const unsigned int cost = cell_cost(S, cells[begin + i], &H, &W);
-      const int hl = C > 0 ? (H + C - 1) / C : H;
-      const bool fits_dist = C > 1 && C <= S.dist_c && H >= C && W <= S.dist_cap_w && hl <= S.dist_cap_hl &&
-                             hl * W <= S.dist_cap_nyl;
       const bool fits_one = H <= S.cap_side && W <= S.cap_side && H * W <= S.cap_ny;
+      const CellDesc& cd = cells[begin + i];
+      const bool fits_dist = fits_cluster(S, H, W, C) || (!fits_one && fits_hybrid(S, cd.nx1, cd.nx2, H, W, C));
       const bool big = mode != 2 && fits_dist && (mode == 1 || !fits_one || (double)cost > thr);
       if (!fits_one && !big && fits_layout(S, H, W) && (mode == 2 || C < S.dist_c)) atomicOr(S.status, ST_REGROUP);
       k = ((unsigned long long)big << 62) | ((unsigned long long)cost << 30) | (0x3fffffffu - (unsigned)i);
@@ -1846,7 +1870,7 @@ k_cell_solve_multi(const DevState* __restrict__ states, const CellRef* __restric
     if (j >= nref) break;
     const CellRef rf = refs[order ? order[j] : j];
     load_state(rf.inst);
-    if (!halted(rf)) cell_solve_body<R>(sS, sS.cells[part][rf.cell], rf.pos, rf.nbatch, smem_raw);
+    if (!halted(rf)) cell_solve_body<R, false>(sS, sS.cells[part][rf.cell], rf.pos, rf.nbatch, smem_raw);
   }
 }
 
@@ -1884,10 +1908,9 @@ k_ref_order(const DevState* __restrict__ states, const CellRef* __restrict__ ref
       const DevState& S = states[rf.inst];
       int H, W;
       const unsigned int cost = cell_cost(S, S.cells[part][rf.cell], &H, &W);
-      const int hl = (H + C - 1) / C;
-      const bool fits_dist = C > 1 && C <= S.dist_c && H >= C && W <= S.dist_cap_w && hl <= S.dist_cap_hl &&
-                             hl * W <= S.dist_cap_nyl;
       const bool fits_one = H <= S.cap_side && W <= S.cap_side && H * W <= S.cap_ny;
+      const CellDesc& cd = S.cells[part][rf.cell];
+      const bool fits_dist = fits_cluster(S, H, W, C) || (!fits_one && fits_hybrid(S, cd.nx1, cd.nx2, H, W, C));
       const bool big = fits_dist && (!fits_one || (double)cost > thr);
       if (!fits_one && !big && fits_layout(S, H, W) && C < S.dist_c) atomicOr(S.status, ST_REGROUP);
       k = ((unsigned long long)big << 62) | ((unsigned long long)cost << 30) | (0x3fffffffu - (unsigned)i);
@@ -1933,16 +1956,26 @@ size_t dist_smem_bytes(int s, int C, int cap_w, int cap_hl, int cap_nyl, int pre
 // Static shared memory of the cell kernels, the larger of the single- and the
 // many-instance kernel (the dynamic part must leave room for it).
 int cell_static_smem(int precision) {
-  cudaFuncAttributes a1, a2;
-  cudaError_t e1 = precision ? cudaFuncGetAttributes(&a1, k_cell_solve<double>)
-                             : cudaFuncGetAttributes(&a1, k_cell_solve<float>);
-  cudaError_t e2 = precision ? cudaFuncGetAttributes(&a2, k_cell_solve_multi<double>)
-                             : cudaFuncGetAttributes(&a2, k_cell_solve_multi<float>);
-  if (e1 != cudaSuccess || e2 != cudaSuccess) {
-    cudaGetLastError();
-    return 4096;
+  cudaFuncAttributes a[3];
+  cudaError_t e[3];
+  if (precision) {
+    e[0] = cudaFuncGetAttributes(&a[0], k_cell_solve<double, false>);
+    e[1] = cudaFuncGetAttributes(&a[1], k_cell_solve<double, true>);
+    e[2] = cudaFuncGetAttributes(&a[2], k_cell_solve_multi<double>);
+  } else {
+    e[0] = cudaFuncGetAttributes(&a[0], k_cell_solve<float, false>);
+    e[1] = cudaFuncGetAttributes(&a[1], k_cell_solve<float, true>);
+    e[2] = cudaFuncGetAttributes(&a[2], k_cell_solve_multi<float>);
   }
-  return (int)std::max(a1.sharedSizeBytes, a2.sharedSizeBytes);
+  size_t m = 0;
+  for (int k = 0; k < 3; ++k) {
+    if (e[k] != cudaSuccess) {
+      cudaGetLastError();
+      return 4096;
+    }
+    m = std::max(m, a[k].sharedSizeBytes);
+  }
+  return (int)m;
 }
 
 // Resident CTAs of the single-instance cell kernel with `smem` dynamic bytes:
@@ -1953,16 +1986,16 @@ int cell_resident_ctas(size_t smem, int C, int precision) {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   cudaError_t e;
-  if (precision) e = cudaFuncSetAttribute(k_cell_solve<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  else e = cudaFuncSetAttribute(k_cell_solve<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (precision) e = cudaFuncSetAttribute(k_cell_solve<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  else e = cudaFuncSetAttribute(k_cell_solve<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
   if (C <= 1) {
     int per = 0;
-    e = precision ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_cell_solve<double>, kCellThreads, smem)
-                  : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_cell_solve<float>, kCellThreads, smem);
+    e = precision ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_cell_solve<double, false>, kCellThreads, smem)
+                  : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_cell_solve<float, false>, kCellThreads, smem);
     if (e != cudaSuccess) {
       cudaGetLastError();
       return nsm > 0 ? nsm : 1;
@@ -1981,8 +2014,8 @@ int cell_resident_ctas(size_t smem, int C, int precision) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   int n = 0;
-  e = precision ? cudaOccupancyMaxActiveClusters(&n, k_cell_solve<double>, &cfg)
-                : cudaOccupancyMaxActiveClusters(&n, k_cell_solve<float>, &cfg);
+  e = precision ? cudaOccupancyMaxActiveClusters(&n, k_cell_solve<double, false>, &cfg)
+                : cudaOccupancyMaxActiveClusters(&n, k_cell_solve<float, false>, &cfg);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return 0;
@@ -2009,12 +2042,12 @@ cudaError_t launch_cell_solve(const DevState& S, const CellDesc* cells, const in
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = C > 1 ? 1 : 0;
-  if (precision) {
-    cudaFuncSetAttribute(k_cell_solve<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    return cudaLaunchKernelEx(&cfg, k_cell_solve<double>, S, cells, order, nbig_p, begin, nbatch, crun, C);
-  }
-  cudaFuncSetAttribute(k_cell_solve<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  return cudaLaunchKernelEx(&cfg, k_cell_solve<float>, S, cells, order, nbig_p, begin, nbatch, crun, C);
+  auto run = [&](auto kernel) {
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    return cudaLaunchKernelEx(&cfg, kernel, S, cells, order, nbig_p, begin, nbatch, crun, C);
+  };
+  if (S.balance) return precision ? run(k_cell_solve<double, true>) : run(k_cell_solve<float, true>);
+  return precision ? run(k_cell_solve<double, false>) : run(k_cell_solve<float, false>);
 }
 
 // One many-instance launch: order the references (k_ref_order), then `nctas`
