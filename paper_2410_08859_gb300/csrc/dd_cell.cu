@@ -350,12 +350,12 @@ __device__ __forceinline__ void pass_lanes(const R* src, int sl, int sm, const R
   }
 }
 
-// Few targets: a group of lanes each.  Otherwise tiles of four targets when
-// they occupy three quarters of the threads, of two when those occupy a quarter
-// of them, else single targets: a larger tile spends fewer instructions per
-// term (about 6, 7.5 and 10), a smaller one keeps more warps busy on the small
-// cells.  `linear`: target j L + l on thread (j L + l) mod nthr in any case (for
-// sums over a thread's targets whose order must not depend on the tile).
+// Few targets: a group of lanes each.  Otherwise tiles of two targets when
+// those occupy a quarter of the threads, else single targets: the larger tile
+// spends fewer instructions per term (about 7.5 against 10), the smaller one
+// keeps more warps busy on the small cells.  (Tiles of four spilled registers.)
+// `linear`: target j L + l on thread (j L + l) mod nthr in any case (for sums
+// over a thread's targets whose order must not depend on the tile).
 template <typename Put>
 __device__ __forceinline__ void run_pass(const float* src, int sl, int sm, const float* prev, int ol, int oj, int L,
                                          int J, int M, int off, float q2, bool first, int tid, int nthr, Put put,
@@ -363,8 +363,6 @@ __device__ __forceinline__ void run_pass(const float* src, int sl, int sm, const
   const int P = lanes_per_target(L * J, M, nthr);
   if (P > 1)
     pass_lanes<float>(src, sl, sm, prev, ol, oj, L, J, M, off, q2, first, P, tid, nthr, put);
-  else if (!linear && 4 * L * ((J + 3) / 4) >= 3 * nthr)
-    pass_tiles<4>(src, sl, sm, prev, ol, oj, L, J, M, off, q2, first, tid, nthr, put);
   else if (!linear && 4 * L * ((J + 1) / 2) >= nthr)
     pass_tiles<2>(src, sl, sm, prev, ol, oj, L, J, M, off, q2, first, tid, nthr, put);
   else

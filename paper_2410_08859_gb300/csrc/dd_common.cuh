@@ -144,9 +144,41 @@ __device__ __forceinline__ float dd_rcp(float x) {
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-__device__ __forceinline__ double dd_ex2(double x) { return exp2(x); }
-__device__ __forceinline__ double dd_lg2(double x) { return log2(x); }
-__device__ __forceinline__ double dd_rcp(double x) { return 1.0 / x; }
+
+// 2^x in double by Tang's table-driven method (ACM TOMS 15, 1989): x = k/64 + r,
+// |r| <= 1/128, 2^x = 2^(k div 64) T[k mod 64] (1 + expm1(r log 2)) with the Taylor
+// polynomial to degree 5 (remainder below 2^-54).  Nine FP64 operations (the FP64
+// pipe gives two lanes a clock; CUDA's exp2 takes about twice as many).  At
+// |x| >= 1022 (results outside the normal range) and NaN: CUDA's exp2.
+__device__ __forceinline__ double dd_ex2(double x) {
+  if ((__double2hiint(x) & 0x7fffffff) >= 0x408ff000) return exp2(x);
+  const double big = 6755399441055744.0;   // 1.5 2^52: the sum's low word is round(64 x)
+  const double t = fma(x, 64.0, big);
+  const int k = __double2loint(t);
+  const double r = fma(t - big, -0.015625, x);
+  double p = fma(r, 1.3333558146428443e-03, 9.6181291076284772e-03);
+  p = fma(p, r, 5.5504108664821580e-02);
+  p = fma(p, r, 2.4022650695910072e-01);
+  p = fma(p, r, 6.9314718055994531e-01);
+  const double T = kExp2T[k & 63];
+  const double y = fma(T, p * r, T);
+  return __hiloint2double(__double2hiint(y) + (int)((unsigned)(k >> 6) << 20), __double2loint(y));
+}
+__device__ __forceinline__ double dd_log(double x);
+__device__ __forceinline__ double dd_lg2(double x) {
+  // positive finite: the table logarithm; 0, negative, infinite, NaN: CUDA's
+  const unsigned hi = (unsigned)__double2hiint(x);
+  if (hi >= 0x7ff00000u || x == 0.0) return log2(x);
+  return dd_log(x) * DD_LOG2E;
+}
+// 1/x from the float reciprocal by two Newton steps (2^-23 -> 2^-46 -> rounding).
+__device__ __forceinline__ double dd_rcp(double x) {
+  const int e = (__double2hiint(x) >> 20) & 0x7ff;
+  if (e < 1023 - 120 || e > 1023 + 120) return 1.0 / x;
+  double r = (double)dd_rcp((float)x);
+  r = fma(fma(-x, r, 1.0), r, r);
+  return fma(fma(-x, r, 1.0), r, r);
+}
 
 template <typename R> __device__ __forceinline__ R dd_inf() { return R(INFINITY); }
 

@@ -256,7 +256,7 @@ cudaError_t adjoint_impl(const double* mu, const double* nu, const double* alpha
 
   const int G = red_blocks(n, 512, partials);
   k_adj_masses<<<G, 512, 0, st>>>(mu, nu, (int)n, partials);
-  k_sum_partials<<<1, 32, 0, st>>>(partials, G, 2, sums);
+  k_sum_partials<<<1, 32 * 2, 0, st>>>(partials, G, 2, sums);
   // X side: f = beta/eps + log nu summed over y for every x, with moments.
   k_adj_prep<<<eb, 256, 0, st>>>(beta, nu, 1.0 / eps, f, fs, (int)n, d_bad);
   k_adj_rows<R, true><<<N, thr_rows, smem_rows, st>>>(B, N, Q);
@@ -268,7 +268,7 @@ cudaError_t adjoint_impl(const double* mu, const double* nu, const double* alpha
   AdjOut OY{nu, beta, grad_nu, nullptr, py, sums, 1, eps, lam, h};
   k_adj_cols<R, false><<<gcols, 256, 0, st>>>(B, OY, N, Q);
   k_adj_value<<<G, 512, 0, st>>>(mu, nu, alpha, beta, px, py, lam, (int)n, partials);
-  k_sum_partials<<<1, 32, 0, st>>>(partials, G, 4, sums + 4);
+  k_sum_partials<<<1, 32 * 4, 0, st>>>(partials, G, 4, sums + 4);
   k_adj_finish<<<1, 32, 0, st>>>(sums, sums + 4, eps, d_out);
   return cudaGetLastError();
 }

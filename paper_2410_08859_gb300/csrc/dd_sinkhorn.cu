@@ -8,6 +8,7 @@
 //  * separable  : |x-y|^2 = (x1-y1)^2 + (x2-y2)^2, so L is a 1-D log-sum-exp along rows
 //                 followed by one along columns: 2 N^3 terms instead of N^4.
 // Values are kept in log2 units (ex2/lg2); float or double arithmetic.
+#include <algorithm>
 #include <cmath>
 
 #include "dd_common.cuh"
@@ -19,109 +20,200 @@ namespace {
 // of them change the sum by N 2^-cut relative (< 1e-15 in double, < 1e-7 in float).
 template <typename R> __device__ __forceinline__ R cut_log2() { return sizeof(R) == 4 ? R(32) : R(64); }
 
-// One 1-D log-sum-exp per target with P lanes: the maximum and the window
-// test run in float on the shadow values; only terms within `cut` of the
-// maximum are evaluated (in R) and summed.
-// FAST (double only): each kept term's exponent is formed in double and only its
-// exponential (at most `cut` below the maximum) is taken in float (ex2.approx);
-// the sums stay double.  The sum's relative error is ~1e-7, i.e. ~1e-7 absolute
-// in log2 units, whatever the magnitude of the exponents.
-template <typename R, bool FAST = false, typename FS, typename FF>
-__device__ __forceinline__ R lse_window(FS src, FF srcf, int M, int ctr, double q2, int part, int P) {
-  const float q2f = (float)q2;
-  float mxf = -INFINITY;
-  for (int m = part; m < M; m += P) {
-    float d = (float)(ctr - m);
-    mxf = fmaxf(mxf, srcf(m) - q2f * d * d);
-  }
-  for (int o = 1; o < P; o <<= 1) mxf = fmaxf(mxf, __shfl_xor_sync(0xffffffffu, mxf, o));
-  if (!(mxf > -INFINITY)) return R(mxf);
-  const float cutf = (float)cut_log2<R>() + 1.0f;
-  const R mx = R(mxf), q2r = R(q2);
-  R acc = R(0);
-  for (int m = part; m < M; m += P) {
-    float d = (float)(ctr - m);
-    if (srcf(m) - q2f * d * d - mxf > -cutf) {
-      R dr = R(ctr - m);
-      if (FAST) acc += R(dd_ex2(float(src(m) - q2r * dr * dr - mx)));
-      else acc += dd_ex2(src(m) - q2r * dr * dr - mx);
-    }
-  }
-  for (int o = 1; o < P; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  return mx + dd_lg2(acc);
+// float(x) rounded to nearest and double(f) for positive normal f, on the integer
+// pipe: conversions to and from double share the two-lane FP64 path.
+__device__ __forceinline__ float narrow(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  if ((hi & 0x7fffffffu) < 0x38100000u) return 0.0f;   // below 2^-126
+  unsigned f = __funnelshift_l(lo, hi, 3) - (896u << 23);
+  f += (lo & 0x1fffffffu) + (f & 1u) > 0x10000000u ? 1u : 0u;
+  return __uint_as_float((f & 0x7fffffffu) | (hi & 0x80000000u));
+}
+__device__ __forceinline__ double widen_pos(float f) {
+  const unsigned u = __float_as_uint(f);
+  return __hiloint2double((int)((u >> 3) + 0x38000000u), (int)(u << 29));
 }
 
-// The same log-sum-exp against a shift `sig` (the previous iteration's value of
-// this target) in one pass: terms more than `cut` below the shift are skipped,
-// so the skipped mass is below N 2^-cut of the sum, as for the max-shifted
-// window.  When the shift is unusable -- NaN, a term more than 60 above it,
-// or a sum outside [2^-30, 2^60] -- the lane group falls back to lse_window
-// (warp-collective: every lane of the warp runs the fallback if one group needs it).
-template <typename R, bool FAST = false, typename FS, typename FF>
-__device__ __forceinline__ R lse_window_shift(FS src, FF srcf, int M, int ctr, double q2, int part, int P, R sig) {
-  const float q2f = (float)q2, sigf = (float)sig;
-  const float cutf = (float)cut_log2<R>() + 1.0f;
-  const R q2r = R(q2);
-  R acc = R(0);
-  bool bad = !(sigf > -INFINITY && sigf < INFINITY);
-  if (!bad) {
-    for (int m = part; m < M; m += P) {
-      const float d = (float)(ctr - m);
-      const float vf = srcf(m) - q2f * d * d - sigf;
-      if (vf > -cutf) {
-        bad |= vf > 60.0f;
-        const R dr = R(ctr - m);
-        if (FAST) acc += R(dd_ex2(float(src(m) - q2r * dr * dr - sig)));
-        else acc += dd_ex2(src(m) - q2r * dr * dr - sig);
-      }
-    }
-  }
-  for (int o = 1; o < P; o <<= 1) {
-    acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    bad |= __shfl_xor_sync(0xffffffffu, (int)bad, o) != 0;
-  }
-  bad |= !(acc >= R(9.313225746154785e-10) && acc <= R(1.152921504606847e18));   // [2^-30, 2^60]
-  if (__any_sync(0xffffffffu, bad)) {
-    const R v = lse_window<R, FAST>(src, srcf, M, ctr, q2, part, P);
-    if (bad) return v;
-  }
-  return sig + dd_lg2(acc);
-}
+// After a second pass: the half-step's potential and the next pass's input, in
+// place of two launches (pot == NULL: none).  For each pixel, pot = -kappa z and
+// in2 = (pot/eps + log m) log2 e (and its float shadow).
+template <typename R>
+struct SepHalf {
+  double* pot;
+  const double* logm;
+  R* in2;
+  float* in2f;
+  double kappa, inv_eps;
+};
 
-constexpr int kSepLanes = 4;   // lanes per target in the separable passes
+constexpr int kSepLanes = 4;    // lanes per target, one residue of the source index modulo 4 each
+constexpr int kSepBlock = 16;   // sources per block maximum
 
 // Row pass with a transposed store: dst[j*N + k] = log2 sum_l 2^{src[k*N + l] - q2 (j - l)^2}
-// (block = row k).  Applied twice it gives the 2-D log-sum-exp in the original
-// layout (the second pass runs along the columns of the original image), with
-// every source read from shared memory instead of strided global loads.
+// (blockIdx.x = row k; blockIdx.y: a range of targets).  Applied twice it gives the
+// 2-D log-sum-exp in the original layout (the second pass runs along the columns
+// of the original image), with every source read from shared memory.
+//
 // With `shifted`, dst holds the previous iteration's values on entry and each
-// target is evaluated in one pass against its previous value
-// (lse_window_shift); otherwise max-shifted (lse_window).
+// target is summed against its previous value: terms more than `cut` below the
+// shift are left out, so the skipped mass is below N 2^-cut of the sum.  When the
+// shift is unusable -- not finite, a term more than 60 above it, or a sum outside
+// [2^-30, 2^60] -- and without `shifted`, the target is summed against its
+// maximum.  The tests run in float on the shadow values; only kept terms are
+// evaluated in R.  FAST (double only): a kept term's exponent is formed in double
+// and only its exponential (at most `cut` below the shift) in float (ex2.approx);
+// the sums stay double.  The sum's relative error is ~1e-7, i.e. ~1e-7 absolute
+// in log2 units, whatever the magnitude of the exponents.
+//
+// Bound: the FP64 pipe (two lanes a clock): 3 (FAST) or 12 operations per kept
+// term.  So a target's window of sources is found first, in float and by the
+// maxima of blocks of 16 sources: the lanes of a warp (8 neighbouring targets)
+// then run over nearly the same window, where a test of every source held all of
+// them for any one's term; the products q2 d come from a table and the
+// logarithms are taken by full warps at the end.  Measured, before -> now:
+// 256 x 256 FAST at eps = 8 h^2 71 -> 33 us, 32 h^2 103 -> 47; float 12.5 -> 9.5 (128 h^2) and
+// 12.7 -> 14.8 (8192 h^2: every source kept); 1024 x 1024 FAST 802 -> 317 (2 h^2), float
+// 542 -> 127 (128 h^2); 64 x 64 double 27 -> 12 (the rows split over several CTAs
+// to reach all SMs).
 template <typename R, bool FAST>
 __global__ void __launch_bounds__(1024)
-k_sep_rows_t(const R* __restrict__ src, const float* __restrict__ srcf, R* dst,
-             float* __restrict__ dstf, int N, double q2, int shifted) {
+k_sep_rows_t(const R* __restrict__ src, const float* __restrict__ srcf, R* dst, float* __restrict__ dstf, int N,
+             double q2, int shifted, int per, SepHalf<R> half) {
   extern __shared__ __align__(16) unsigned char sm[];
+  constexpr bool DBL = sizeof(R) == 8;
   R* row = reinterpret_cast<R*>(sm);
-  float* rowf = reinterpret_cast<float*>(row + N);
-  const int k = blockIdx.x;
+  R* accS = row + N;
+  R* sigS = accS + per;
+  double* qd = reinterpret_cast<double*>(sigS + per + (N & 1));   // double: (q2 d, d), 16-byte aligned
+  float* rowf = DBL ? reinterpret_cast<float*>(qd + 2 * N) : reinterpret_cast<float*>(row);
+  float* bm = DBL ? rowf + N : reinterpret_cast<float*>(qd);
+  const int k = blockIdx.x, nb = (N + kSepBlock - 1) / kSepBlock;
+  const int j_lo = blockIdx.y * per, j_n = min(per, N - j_lo);
   for (int l = threadIdx.x; l < N; l += blockDim.x) {
     row[l] = src[(long long)k * N + l];
-    rowf[l] = srcf[(long long)k * N + l];
+    if (DBL) {
+      rowf[l] = srcf[(long long)k * N + l];
+      reinterpret_cast<double2*>(qd)[l] = make_double2(q2 * (double)l, (double)l);
+    }
   }
   __syncthreads();
-  const int P = kSepLanes, nt = (N * P + 31) & ~31;
+  for (int b = threadIdx.x; b < nb; b += blockDim.x) {
+    float m = -INFINITY;
+    for (int l = b * kSepBlock; l < min(N, (b + 1) * kSepBlock); ++l) m = fmaxf(m, rowf[l]);
+    bm[b] = m;
+  }
+  __syncthreads();
+  const float q2f = (float)q2, cutf = (float)cut_log2<R>() + 1.0f;
+  const int P = kSepLanes, part = threadIdx.x & (P - 1), nt = (j_n * P + 31) & ~31;
+  // upper bound of the terms of block b at target j (a few ulp are added for the rounding)
+  auto bound = [&](int b, int j) {
+    const float d = (float)(j - min(max(j, b * kSepBlock), b * kSepBlock + kSepBlock - 1));
+    const float u = fmaf(-q2f * d, d, bm[b]);
+    return fmaf(1e-6f, fabsf(bm[b]) + fabsf(u), u);
+  };
+  auto term_f = [&](int m, int j) {
+    const float d = (float)(j - m);
+    return fmaf(-(q2f * d), d, rowf[m]);
+  };
+  auto term = [&](int m, int j) {   // each operation rounded (the float results do not depend on contraction)
+    const float d = (float)(j - m);
+    return __fsub_rn(rowf[m], __fmul_rn(__fmul_rn(q2f, d), d));
+  };
   for (int i = threadIdx.x; i < nt; i += blockDim.x) {
-    const int j0 = i / P, part = i % P, j = min(j0, N - 1);
-    auto srcv = [&](int m) { return row[m]; };
-    auto srcfv = [&](int m) { return rowf[m]; };
-    R v;
-    if (shifted) v = lse_window_shift<R, FAST>(srcv, srcfv, N, j, q2, part, P, dst[(long long)j * N + k]);
-    else v = lse_window<R, FAST>(srcv, srcfv, N, j, q2, part, P);
-    __syncwarp();
-    if (part == 0 && j0 < N) {
-      dst[(long long)j * N + k] = v;
-      if (dstf) dstf[(long long)j * N + k] = (float)v;
+    const int t0 = i / P, j = j_lo + min(t0, j_n - 1);
+    R sig = shifted ? dst[(long long)j * N + k] : R(0);
+    float sigf = (float)sig;
+    R acc = R(0);
+    bool todo = shifted ? sigf > -INFINITY && sigf < INFINITY : false;
+    for (int pass = shifted ? 0 : 1; pass < 2; ++pass) {
+      if (pass == 1) {
+        // the maximum, from the block with the largest bound and those that can exceed it
+        const bool again = !todo;
+        float ub = -INFINITY, mx = -INFINITY;
+        int best = 0;
+        for (int b = part; b < nb; b += P) {
+          const float u = bound(b, j);
+          if (u > ub) { ub = u; best = b; }
+        }
+        for (int o = 1; o < P; o <<= 1) {
+          const float u = __shfl_xor_sync(0xffffffffu, ub, o);
+          const int b = __shfl_xor_sync(0xffffffffu, best, o);
+          if (u > ub || (u == ub && b < best)) { ub = u; best = b; }
+        }
+        for (int m = best * kSepBlock + part; m < min(N, (best + 1) * kSepBlock); m += P) mx = fmaxf(mx, term_f(m, j));
+        for (int o = 1; o < P; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        for (int b = part; b < nb; b += P)
+          if (bound(b, j) >= mx)
+            for (int m = b * kSepBlock; m < min(N, (b + 1) * kSepBlock); ++m) mx = fmaxf(mx, term_f(m, j));
+        for (int o = 1; o < P; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        if (again) {
+          sigf = mx;
+          sig = R(mx);
+          acc = mx > -INFINITY ? R(0) : R(1);   // no finite term: the value is the maximum itself
+          todo = mx > -INFINITY;
+        } else {
+          todo = false;   // this target's sum stands; its neighbours' are repeated
+        }
+      }
+      // the window: from the first to the last block that can hold a kept term
+      int lo = N, hi = 0;
+      if (todo)
+        for (int b = part; b < nb; b += P)
+          if (bound(b, j) - sigf > -cutf - 1.0f) {
+            lo = min(lo, b * kSepBlock);
+            hi = max(hi, min(N, (b + 1) * kSepBlock));
+          }
+      for (int o = 1; o < P; o <<= 1) {
+        lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+        hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+      }
+      bool over = false;
+      R a = R(0);
+      for (int m = lo + part; m < hi; m += P) {   // lo is a multiple of 16: residue `part`, ascending
+        const float vf = term(m, j) - sigf;
+        if (vf > -cutf) {
+          over |= vf > 60.0f;
+          if constexpr (DBL) {
+            const int d = abs(j - m);
+            const double2 t = reinterpret_cast<const double2*>(qd)[d];   // q2 d, d
+            const double x = fma(-t.x, t.y, row[m]) - sig;
+            if (FAST) a += widen_pos(dd_ex2(narrow(x)));
+            else a += dd_ex2(x);
+          } else {
+            a += dd_ex2(vf);
+          }
+        }
+      }
+      for (int o = 1; o < P; o <<= 1) {
+        a += __shfl_xor_sync(0xffffffffu, a, o);
+        over |= __shfl_xor_sync(0xffffffffu, (int)over, o) != 0;
+      }
+      if (todo) acc = a;
+      if (pass == 0) {
+        todo = todo && !over && acc >= R(9.313225746154785e-10) && acc <= R(1.152921504606847e18);   // [2^-30, 2^60]
+        if (!__any_sync(0xffffffffu, !todo)) break;
+      }
+    }
+    if (part == 0 && t0 < j_n) {
+      accS[t0] = acc;
+      sigS[t0] = sig;
+    }
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < j_n; t += blockDim.x) {
+    R lg;
+    if constexpr (DBL && FAST) lg = log2(accS[t]);   // a last-bit change here moves float exponents of the mixed mode
+    else lg = dd_lg2(accS[t]);
+    const R v = sigS[t] + lg;
+    const long long o = (long long)(j_lo + t) * N + k;
+    dst[o] = v;
+    if (dstf) dstf[o] = (float)v;
+    if (half.pot) {
+      const double pot = -half.kappa * (double)v * DD_LN2;
+      half.pot[o] = pot;
+      const R in = R(fma(pot, half.inv_eps, half.logm[o])) * R(DD_LOG2E);
+      half.in2[o] = in;
+      if (DBL) half.in2f[o] = (float)in;
     }
   }
 }
@@ -228,7 +320,7 @@ void sk_eval(const double* mu, const double* nu, const double* alpha, const doub
     k_sk_eval<R><<<1, 512, 0, st>>>(mu, nu, alpha, beta, w2, z2, eps, lam, n, d_eval);
   } else {
     k_sk_eval<R><<<G, 512, 0, st>>>(mu, nu, alpha, beta, w2, z2, eps, lam, n, partials);
-    k_sum_partials<<<1, 32, 0, st>>>(partials, G, 6, d_eval);
+    k_sum_partials<<<1, 32 * 6, 0, st>>>(partials, G, 6, d_eval);
   }
 }
 
@@ -258,7 +350,7 @@ void ti_step(const double* mu, const double* nu, double* alpha, const double* be
              double* sums, double* partials, cudaStream_t st) {
   const int G = red_blocks(n, 512, partials);
   k_ti_sums<<<G, 512, 0, st>>>(mu, nu, alpha, beta, lam, n, partials);
-  k_sum_partials<<<1, 32, 0, st>>>(partials, G, 2, sums);
+  k_sum_partials<<<1, 32 * 2, 0, st>>>(partials, G, 2, sums);
   k_ti_apply<<<(n + 255) / 256, 256, 0, st>>>(alpha, sums, lam, n);
 }
 
@@ -268,35 +360,95 @@ struct Work {
   float *in2f, *tmpf;  // float shadows (double precision only)
 };
 
+// One separable pass: a CTA per row, or several where the rows alone are fewer
+// than four per SM of a 152-SM GPU.
+template <typename R, bool FAST>
+cudaError_t sep_pass(const R* in, const float* inf, R* out, float* outf, int N, double q2, int shifted,
+                     const SepHalf<R>& half, cudaStream_t st) {
+  const int gy = std::max(1, std::min((N + 15) / 16, (608 + N - 1) / N));
+  const int per = (N + gy - 1) / gy, thr = std::min(1024, ((per * kSepLanes + 31) / 32) * 32);
+  const int nb = (N + kSepBlock - 1) / kSepBlock;
+  const size_t sm = sizeof(R) * ((size_t)N + 2 * (size_t)per + 1) + (sizeof(R) == 8 ? 20 * (size_t)N : 0) + 4 * (size_t)nb + 16;
+  if (sm > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(k_sep_rows_t<R, FAST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+  }
+  k_sep_rows_t<R, FAST><<<dim3(N, (N + per - 1) / per), thr, sm, st>>>(in, inf, out, outf, N, q2, shifted, per, half);
+  return cudaGetLastError();
+}
+
 // in2f / tmpf: float shadows (required for R = double; ignored for float).
 // use_shift (separable): tmp and out2 hold this evaluation's previous values
 // (tmp: the row pass, transposed) and every target is summed against them in
-// one pass; otherwise max-shifted.
+// one pass; otherwise max-shifted.  half (separable only): see SepHalf.
 template <typename R>
 cudaError_t lse_all(const R* in2, R* tmp, R* out2, int N, double q, int variant, int use_shift, cudaStream_t st,
-                    const float* in2f = nullptr, float* tmpf = nullptr, bool fast = false) {
+                    const float* in2f = nullptr, float* tmpf = nullptr, bool fast = false,
+                    const SepHalf<R>& half = SepHalf<R>{}) {
   if (variant == 1) {
-    const float* inf = sizeof(R) == 8 ? in2f : reinterpret_cast<const float*>(in2);
-    float* tf = sizeof(R) == 8 ? tmpf : nullptr;                       // shadow written by pass 1
-    const float* tfr = sizeof(R) == 8 ? tmpf : reinterpret_cast<const float*>(tmp);
     const double q2 = q * DD_LOG2E;
-    const int thr_rows = min(1024, ((N * kSepLanes + 31) / 32) * 32);
-    const size_t sm = N * (sizeof(R) + sizeof(float));
     // rows, stored transposed; then the rows of that (the original columns), transposed back
     const int sh = use_shift ? 1 : 0;
-    if (fast && sizeof(R) == 8) {
-      k_sep_rows_t<R, true><<<N, thr_rows, sm, st>>>(in2, inf, tmp, tf, N, q2, sh);
-      k_sep_rows_t<R, true><<<N, thr_rows, sm, st>>>(tmp, tfr, out2, nullptr, N, q2, sh);
+    cudaError_t e;
+    if constexpr (sizeof(R) == 8) {
+      if (fast) {
+        e = sep_pass<R, true>(in2, in2f, tmp, tmpf, N, q2, sh, SepHalf<R>{}, st);
+        if (e == cudaSuccess) e = sep_pass<R, true>(tmp, tmpf, out2, nullptr, N, q2, sh, half, st);
+      } else {
+        e = sep_pass<R, false>(in2, in2f, tmp, tmpf, N, q2, sh, SepHalf<R>{}, st);
+        if (e == cudaSuccess) e = sep_pass<R, false>(tmp, tmpf, out2, nullptr, N, q2, sh, half, st);
+      }
     } else {
-      k_sep_rows_t<R, false><<<N, thr_rows, sm, st>>>(in2, inf, tmp, tf, N, q2, sh);
-      k_sep_rows_t<R, false><<<N, thr_rows, sm, st>>>(tmp, tfr, out2, nullptr, N, q2, sh);
+      e = sep_pass<R, false>(in2, nullptr, tmp, nullptr, N, q2, sh, SepHalf<R>{}, st);
+      if (e == cudaSuccess) e = sep_pass<R, false>(tmp, nullptr, out2, nullptr, N, q2, sh, half, st);
     }
-  } else {
-    R q2 = R(q * DD_LOG2E);
-    int n = N * N;
-    k_dense<R><<<(n + 255) / 256, 256, 0, st>>>(in2, out2, N, q2, use_shift);
+    return e;
   }
+  R q2 = R(q * DD_LOG2E);
+  int n = N * N;
+  k_dense<R><<<(n + 255) / 256, 256, 0, st>>>(in2, out2, N, q2, use_shift);
   return cudaGetLastError();
+}
+
+// Iterations of one eps stage of the alternation, from w = the log-sum-exp of
+// beta.  Where no check follows, the second pass of a half-step also writes the
+// potential and the next input (SepHalf).  check(it) is called every check_every
+// iterations and at the last one and returns true to stop.  Returns the
+// iterations made.
+template <typename R, typename Check>
+int sinkhorn_stage(const double* logmu, const double* lognu, double* alpha, double* beta, R* in2, float* in2f, R* tmp,
+                   R* tmpz, float* tmpf, R* w2, R* z2, int N, double e, double kap, int variant, bool fast, int maxit,
+                   int check_every, bool fuse, cudaStream_t st, Check check, void (*after_x)(void*), void* ctx) {
+  const int n = N * N, grid = (n + 255) / 256;
+  const double q = (1.0 / N) * (1.0 / N) / e;
+  k_to_log2<R><<<grid, 256, 0, st>>>(beta, lognu, 1.0 / e, in2, n, in2f);
+  lse_all<R>(in2, tmp, w2, N, q, variant, 0, st, in2f, tmpf, fast);
+  const bool sep = variant == 1;
+  bool ready = false;   // alpha and in2 are those of the coming half-step
+  int it = 0, shift_ok = 0;
+  while (it < maxit) {
+    if (!ready) {
+      k_half<R><<<grid, 256, 0, st>>>(w2, kap, alpha, n);
+      if (after_x) after_x(ctx);
+      k_to_log2<R><<<grid, 256, 0, st>>>(alpha, logmu, 1.0 / e, in2, n, in2f);
+    }
+    if (sep) {
+      lse_all<R>(in2, tmpz, z2, N, q, variant, shift_ok, st, in2f, tmpf, fast,
+                 SepHalf<R>{beta, lognu, in2, in2f, kap, 1.0 / e});
+    } else {
+      lse_all<R>(in2, tmpz, z2, N, q, variant, shift_ok, st, in2f, tmpf, fast);
+      k_half<R><<<grid, 256, 0, st>>>(z2, kap, beta, n);
+      k_to_log2<R><<<grid, 256, 0, st>>>(beta, lognu, 1.0 / e, in2, n, in2f);
+    }
+    shift_ok = 1;
+    ++it;
+    const bool checked = it % check_every == 0 || it == maxit;
+    ready = sep && fuse && !checked;
+    lse_all<R>(in2, tmp, w2, N, q, variant, 1, st, in2f, tmpf, fast,
+               ready ? SepHalf<R>{alpha, logmu, in2, in2f, kap, 1.0 / e} : SepHalf<R>{});
+    if (checked && check(it)) break;
+  }
+  return it;
 }
 
 }  // namespace
@@ -323,7 +475,6 @@ static int full_sinkhorn_impl(const double* mu, const double* nu, const double* 
                               double err, int check_every, double* alpha, double* beta, double* out,
                               double* d_eval, cudaStream_t st, cudaError_t* cerr, bool fast = false) {
   const int n = N * N;
-  const double h = 1.0 / N;
   const bool ti = (variant & DOMDEC_SINKHORN_TI) && std::isfinite(lam);
   variant &= ~DOMDEC_SINKHORN_TI;
   Work<R> w;
@@ -335,46 +486,36 @@ static int full_sinkhorn_impl(const double* mu, const double* nu, const double* 
   w.in2f = reinterpret_cast<float*>(w.tmpz + n);
   w.tmpf = w.in2f + n;
   double* partials = reinterpret_cast<double*>(reinterpret_cast<unsigned char*>(w.in2) + wbytes);
-  const int grid = (n + 255) / 256;
   double evalh[6];
   long long total = 0;
   double gap = INFINITY;
   int rc = 0;
   if (check_every < 1) check_every = 1;
   double e = eps_start > eps ? eps_start : eps;
-  bool first_stage = true;
   for (;;) {
     const double kap = std::isfinite(lam) ? e / (1.0 + e / lam) : e;
-    const double q = h * h / e;
-    // w = LSE_y[beta/e + log nu]
-    k_to_log2<R><<<grid, 256, 0, st>>>(beta, lognu, 1.0 / e, w.in2, n, w.in2f);
-    lse_all<R>(w.in2, w.tmp, w.w2, N, q, variant, 0, st, w.in2f, w.tmpf, fast);
-    int it = 0;
-    bool conv = false;
-    int shift_ok = 0;
-    while (it < maxit) {
-      k_half<R><<<grid, 256, 0, st>>>(w.w2, kap, alpha, n);
-      if (ti) ti_step(mu, nu, alpha, beta, lam, n, d_eval + 6, partials, st);
-      k_to_log2<R><<<grid, 256, 0, st>>>(alpha, logmu, 1.0 / e, w.in2, n, w.in2f);
-      lse_all<R>(w.in2, w.tmpz, w.z2, N, q, variant, shift_ok, st, w.in2f, w.tmpf, fast);
-      k_half<R><<<grid, 256, 0, st>>>(w.z2, kap, beta, n);
-      k_to_log2<R><<<grid, 256, 0, st>>>(beta, lognu, 1.0 / e, w.in2, n, w.in2f);
-      lse_all<R>(w.in2, w.tmp, w.w2, N, q, variant, 1, st, w.in2f, w.tmpf, fast);
-      shift_ok = 1;
-      ++it;
-      if (it % check_every == 0 || it == maxit) {
-        sk_eval<R>(mu, nu, alpha, beta, w.w2, nullptr, e, lam, n, d_eval, partials, st);
-        cudaMemcpyAsync(evalh, d_eval, 6 * sizeof(double), cudaMemcpyDeviceToHost, st);
-        *cerr = cudaStreamSynchronize(st);
-        if (*cerr != cudaSuccess) { cudaFreeAsync(w.in2, st); return -1; }
-        gap = evalh[0];
-        if (err >= 0.0 && gap <= err * evalh[4]) { conv = true; break; }
-        if (!(gap == gap)) break;
-      }
-    }
+    bool conv = false, broke = false;
+    struct Ti { const double *mu, *nu; double *alpha; const double* beta; double lam; int n; double *sums, *part; cudaStream_t st; };
+    Ti tc{mu, nu, alpha, beta, lam, n, d_eval + 6, partials, st};
+    auto ti_run = [](void* p) {
+      Ti* t = static_cast<Ti*>(p);
+      ti_step(t->mu, t->nu, t->alpha, t->beta, t->lam, t->n, t->sums, t->part, t->st);
+    };
+    const int it = sinkhorn_stage<R>(
+        logmu, lognu, alpha, beta, w.in2, w.in2f, w.tmp, w.tmpz, w.tmpf, w.w2, w.z2, N, e, kap, variant, fast, maxit,
+        check_every, !ti, st,
+        [&](int) {
+          sk_eval<R>(mu, nu, alpha, beta, w.w2, nullptr, e, lam, n, d_eval, partials, st);
+          cudaMemcpyAsync(evalh, d_eval, 6 * sizeof(double), cudaMemcpyDeviceToHost, st);
+          *cerr = cudaStreamSynchronize(st);
+          if (*cerr != cudaSuccess) return broke = true;
+          gap = evalh[0];
+          conv = err >= 0.0 && gap <= err * evalh[4];
+          return conv || !(gap == gap);
+        },
+        ti ? +ti_run : nullptr, &tc);
+    if (broke) { cudaFreeAsync(w.in2, st); return -1; }
     total += it;
-    first_stage = false;
-    (void)first_stage;
     if (e <= eps) { rc = conv || err < 0.0 ? 0 : 1; break; }
     e = fmax(eps, 0.5 * e);
   }
@@ -481,7 +622,6 @@ int full_sinkhorn_noalloc_impl(const double* mu, const double* nu, const double*
                                double err, int check_every, double* alpha, double* beta, double* out,
                                double* work, double* d_eval, cudaStream_t st, cudaError_t* cerr) {
   const int n = N * N;
-  const double h = 1.0 / N;
   // five work arrays in double-sized slots (float arrays use the first half of each)
   R* in2 = reinterpret_cast<R*>(work);
   R* tmp = reinterpret_cast<R*>(work + n);
@@ -490,7 +630,6 @@ int full_sinkhorn_noalloc_impl(const double* mu, const double* nu, const double*
   R* tmpz = reinterpret_cast<R*>(work + 4 * (long long)n);
   float* in2f = reinterpret_cast<float*>(work + 5 * (long long)n);
   float* tmpf = in2f + n;
-  const int grid = (n + 255) / 256;
   double evalh[6];
   long long total = 0;
   int rc = 0;
@@ -498,29 +637,20 @@ int full_sinkhorn_noalloc_impl(const double* mu, const double* nu, const double*
   double e = eps_start > eps ? eps_start : eps;
   for (;;) {
     const double kap = std::isfinite(lam) ? e / (1.0 + e / lam) : e;
-    const double q = h * h / e;
-    k_to_log2<R><<<grid, 256, 0, st>>>(beta, lognu, 1.0 / e, in2, n, in2f);
-    lse_all<R>(in2, tmp, w2, N, q, variant, 0, st, in2f, tmpf);
-    int it = 0, shift_ok = 0;
-    bool conv = false;
-    while (it < maxit) {
-      k_half<R><<<grid, 256, 0, st>>>(w2, kap, alpha, n);
-      k_to_log2<R><<<grid, 256, 0, st>>>(alpha, logmu, 1.0 / e, in2, n, in2f);
-      lse_all<R>(in2, tmpz, z2, N, q, variant, shift_ok, st, in2f, tmpf);
-      k_half<R><<<grid, 256, 0, st>>>(z2, kap, beta, n);
-      k_to_log2<R><<<grid, 256, 0, st>>>(beta, lognu, 1.0 / e, in2, n, in2f);
-      lse_all<R>(in2, tmp, w2, N, q, variant, 1, st, in2f, tmpf);
-      shift_ok = 1;
-      ++it;
-      if (it % check_every == 0 || it == maxit) {
-        k_sk_eval<R><<<1, 512, 0, st>>>(mu, nu, alpha, beta, w2, nullptr, e, lam, n, d_eval);
-        cudaMemcpyAsync(evalh, d_eval, 6 * sizeof(double), cudaMemcpyDeviceToHost, st);
-        *cerr = cudaStreamSynchronize(st);
-        if (*cerr != cudaSuccess) return -1;
-        if (err >= 0.0 && evalh[0] <= err * evalh[4]) { conv = true; break; }
-        if (!(evalh[0] == evalh[0])) break;
-      }
-    }
+    bool conv = false, broke = false;
+    const int it = sinkhorn_stage<R>(
+        logmu, lognu, alpha, beta, in2, in2f, tmp, tmpz, tmpf, w2, z2, N, e, kap, variant, false, maxit, check_every,
+        true, st,
+        [&](int) {
+          k_sk_eval<R><<<1, 512, 0, st>>>(mu, nu, alpha, beta, w2, nullptr, e, lam, n, d_eval);
+          cudaMemcpyAsync(evalh, d_eval, 6 * sizeof(double), cudaMemcpyDeviceToHost, st);
+          *cerr = cudaStreamSynchronize(st);
+          if (*cerr != cudaSuccess) return broke = true;
+          conv = err >= 0.0 && evalh[0] <= err * evalh[4];
+          return conv || !(evalh[0] == evalh[0]);
+        },
+        nullptr, nullptr);
+    if (broke) return -1;
     total += it;
     if (e <= eps) { rc = conv || err < 0.0 ? 0 : 1; break; }
     e = fmax(eps, 0.5 * e);
