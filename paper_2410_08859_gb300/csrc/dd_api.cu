@@ -40,12 +40,12 @@ cudaError_t launch_compact(const DevState& S, long long* newoff, cudaStream_t st
 cudaError_t launch_prepare_inputs(const double* mu, const double* nu, double* logmu, double* lognu, int n,
                                   int* status, cudaStream_t st);
 cudaError_t launch_init_product_boxes(const DevState& S, double* nu_mom, double* mumass, long long* newoff,
-                                      cudaStream_t st);
+                                      double* partials, cudaStream_t st);
 cudaError_t launch_init_product_fill(const DevState& S, double* nu_mom, double* mumass, long long* newoff,
                                      cudaStream_t st);
 cudaError_t launch_init_duals_boxes(const DevState& S, const double* alpha0, const double* beta0, double eps0,
                                     double* nu_mom, double* mumass, long long* newoff, float* gscratch,
-                                    cudaStream_t st);
+                                    double* partials, cudaStream_t st);
 cudaError_t launch_init_duals_fill(const DevState& S, const double* alpha0, const double* beta0, double eps0,
                                    const double* w, long long* newoff, cudaStream_t st);
 cudaError_t launch_score(const DevState& S, double* out, cudaStream_t st, double* partials);
@@ -430,9 +430,9 @@ int load_problem(domdec_s* h, const double* mu, const double* nu, const double* 
     if (e == cudaSuccess) e = cudaMemcpyAsync(bd, beta0, n * sizeof(double), cudaMemcpyDefault, st);
     if (e == cudaSuccess)
       e = launch_init_duals_boxes(S, ad, bd, eps0, h->d_numom, h->d_mumass, h->d_newoff,
-                                  reinterpret_cast<float*>(wtmp), st);
+                                  reinterpret_cast<float*>(wtmp), h->d_partials, st);
   } else {
-    e = launch_init_product_boxes(S, h->d_numom, h->d_mumass, h->d_newoff, st);
+    e = launch_init_product_boxes(S, h->d_numom, h->d_mumass, h->d_newoff, h->d_partials, st);
   }
   long long total = 0;
   if (e == cudaSuccess)

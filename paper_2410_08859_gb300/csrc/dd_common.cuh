@@ -180,6 +180,20 @@ __device__ __forceinline__ double dd_rcp(double x) {
   return fma(fma(-x, r, 1.0), r, r);
 }
 
+// float(x) rounded to nearest and double(f) for positive normal f, on the integer
+// pipe: conversions to and from double share the two-lane FP64 path.
+__device__ __forceinline__ float narrow(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  if ((hi & 0x7fffffffu) < 0x38100000u) return 0.0f;   // below 2^-126
+  unsigned f = __funnelshift_l(lo, hi, 3) - (896u << 23);
+  f += (lo & 0x1fffffffu) + (f & 1u) > 0x10000000u ? 1u : 0u;
+  return __uint_as_float((f & 0x7fffffffu) | (hi & 0x80000000u));
+}
+__device__ __forceinline__ double widen_pos(float f) {
+  const unsigned u = __float_as_uint(f);
+  return __hiloint2double((int)((u >> 3) + 0x38000000u), (int)(u << 29));
+}
+
 template <typename R> __device__ __forceinline__ R dd_inf() { return R(INFINITY); }
 
 // psi(d) = d e^d - e^d + 1 = e^{-g} KL-term ratio (phi(e^d) with phi(s) = s log s - s + 1),

@@ -470,15 +470,21 @@ k_basic_masses(DevState S, const double* nu_mom, double* mumass) {
   }
 }
 
-__global__ void __launch_bounds__(512) k_moments(const double* nu, int N, double h, double* out) {
+// Block partials of (|nu|, sum y1 nu, sum y2 nu, sum |y|^2 nu) (one block over the
+// image took 2.8 ms at 1024^2).
+__global__ void __launch_bounds__(512) k_moments(const double* nu, int N, double h, double* partials) {
   __shared__ double red[33 * 4];
   double v[4] = {0, 0, 0, 0};
-  for (int y = threadIdx.x; y < N * N; y += blockDim.x) {
+  for (int y = blockIdx.x * blockDim.x + threadIdx.x; y < N * N; y += gridDim.x * blockDim.x) {
     double m = nu[y], y1 = (y / N) * h, y2 = (y % N) * h;
     v[0] += m; v[1] += m * y1; v[2] += m * y2; v[3] += m * (y1 * y1 + y2 * y2);
   }
-  block_sum<4>(v, red);
-  if (threadIdx.x == 0) for (int k = 0; k < 4; ++k) out[k] = v[k];
+  block_sum_to<4>(v, red, partials);
+}
+static void moments(const double* nu, int N, double h, double* out, double* partials, cudaStream_t st) {
+  const int G = red_blocks((long long)N * N, 512, partials);
+  k_moments<<<G, 512, 0, st>>>(nu, N, h, partials);
+  k_sum_partials<<<1, 32 * 4, 0, st>>>(partials, G, 4, out);
 }
 
 // Product plan pi0 = mu x nu: nu_i = |mu_i| nu on the full grid, truncated.
@@ -541,6 +547,25 @@ __global__ void k_log_nu_beta(const double* __restrict__ lognu, const double* __
     g[y] = (float)(lognu[y] + beta0[y] / eps0);
 }
 
+// Per 16 x 16 tile of pixels: the maximum of g and of |g| (tmax[0..nt), tmax[nt..2 nt)).
+constexpr int kInitTile = 16;
+__global__ void __launch_bounds__(256) k_tile_max(const float* __restrict__ g, int N, float* __restrict__ tmax) {
+  __shared__ float sm[16];
+  const int ntc = (N + kInitTile - 1) / kInitTile, t = blockIdx.x;
+  const int k = t / ntc * kInitTile + threadIdx.x / kInitTile, l = t % ntc * kInitTile + threadIdx.x % kInitTile;
+  const bool in = k < N && l < N;
+  const float v = in ? g[(long long)k * N + l] : -INFINITY;
+  const float m = warp_max(v), b = warp_max(in ? fabsf(v) : 0.0f);
+  if ((threadIdx.x & 31) == 0) { sm[threadIdx.x >> 5] = m; sm[8 + (threadIdx.x >> 5)] = b; }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    float mm = sm[0], bb = sm[8];
+    for (int w = 1; w < 8; ++w) { mm = fmaxf(mm, sm[w]); bb = fmaxf(bb, sm[8 + w]); }
+    tmax[t] = mm;
+    tmax[gridDim.x + t] = bb;
+  }
+}
+
 // Plan from duals pi = exp((alpha0 + beta0 - c)/eps0) mu x nu, per basic cell.
 // mode 0: tight box of {y : nu_i(y) >= thr} from the full-grid log marginal,
 //         two 1-D log-sum-exp passes over X_i: the first in FP64 (s N values),
@@ -548,13 +573,17 @@ __global__ void k_log_nu_beta(const double* __restrict__ lognu, const double* __
 //         log nu + beta0/eps0); only where the float value lies within a
 //         safety band of log thr (its float error is ~1e-2 at |values| ~ 1e5)
 //         is the FP64 value computed and compared, so the box is the one of
-//         the FP64 test;
+//         the FP64 test.  Tiles of 16 x 16 pixels whose upper bound (the tile's
+//         largest g, each row's largest T over the tile's columns, the smallest
+//         distance) lies below the threshold by more than the tile's band are left
+//         out: a cell's plan reaches a few dozen of the 4096 tiles of a 1024^2
+//         grid, and testing every pixel took 35 ms there (now 1 ms);
 // mode 1: values on the box (dense over X_i), C_i, H_i, P_Y.
 constexpr int kInitChunk = 128;   // box columns per pass of the dual-initialised fill
 constexpr int kInitBand = 2048;   // band pixels listed per basic cell by the box test
 __global__ void __launch_bounds__(1024)
 k_init_duals(DevState S, const double* __restrict__ alpha0, const double* __restrict__ beta0,
-             double eps0, int mode, const float* __restrict__ gf) {
+             double eps0, int mode, const float* __restrict__ gf, const float* __restrict__ tmax) {
   extern __shared__ double tsm[];   // mode 0: see init_box_smem; mode 1: 3 s kInitChunk doubles
   __shared__ int bb[4];
   __shared__ double red[33 * 2];
@@ -601,9 +630,24 @@ k_init_duals(DevState S, const double* __restrict__ alpha0, const double* __rest
     auto keep = [&](int k, int l) {
       lb[0] = min(lb[0], k); lb[1] = max(lb[1], k); lb[2] = min(lb[2], l); lb[3] = max(lb[3], l);
     };
-    // the float test of every pixel; `band` collects those it cannot decide
-    for (int y = threadIdx.x; y < N * N; y += blockDim.x) {
-      const int k = y / N, l = y - (y / N) * N;
+    // row maxima of T per tile column (in the space of the double T, which is filled later)
+    const int ntc = (N + kInitTile - 1) / kInitTile, ntile = ntc * ntc;
+    float* Tm = reinterpret_cast<float*>(tsm);
+    float* Ta = Tm + s * ntc;
+    for (int t = threadIdx.x; t < s * ntc; t += blockDim.x) {
+      const int r = t / ntc, l0 = (t - r * ntc) * kInitTile;
+      float m = -INFINITY, b = 0.0f;
+      for (int l = l0; l < min(N, l0 + kInitTile); ++l) {
+        m = fmaxf(m, tsmf[r * N + l]);
+        b = fmaxf(b, fabsf(tsmf[r * N + l]));
+      }
+      Tm[t] = m;
+      Ta[t] = b;
+    }
+    __syncthreads();
+    // the float test of a pixel; `band` collects those it cannot decide
+    auto test = [&](int k, int l) {
+      const int y = k * N + l;
       float mxf = -INFINITY, big = fabsf(gf[y]);
       for (int r = 0; r < s; ++r) {
         const float d = (float)(r0 + r - k), v = tsmf[r * N + l];
@@ -614,7 +658,7 @@ k_init_duals(DevState S, const double* __restrict__ alpha0, const double* __rest
       // float X values and T add ~1e-7 of the same magnitudes)
       const float band_w = 0.5f + 1e-5f * big;
       const float lo = gf[y] + mxf;   // log nu_i(y) lies in [lo, lo + log s]
-      if (lo + dd_lg2((float)s) * LN2 < lthrf - band_w) continue;   // clearly below the threshold
+      if (lo + dd_lg2((float)s) * LN2 < lthrf - band_w) return;   // clearly below the threshold
       float accf = 0.0f;
       for (int r = 0; r < s; ++r) {
         const float d = (float)(r0 + r - k);
@@ -627,6 +671,30 @@ k_init_duals(DevState S, const double* __restrict__ alpha0, const double* __rest
         colflag[l] = 1;
         const int j = atomicAdd(&nband, 1);
         if (j < kInitBand) band[j] = y;
+      }
+    };
+    const int lane = threadIdx.x & 31;
+    for (int base = threadIdx.x & ~31; base < ntile; base += blockDim.x) {
+      const int t = base + lane;
+      bool cand = false;
+      if (t < ntile) {
+        const int k0t = t / ntc * kInitTile, tc = t - t / ntc * ntc;
+        float up = -INFINITY, big = tmax[ntile + t];
+        for (int r = 0; r < s; ++r) {
+          const int x = r0 + r;
+          const float dn = (float)(x - min(max(x, k0t), k0t + kInitTile - 1));
+          const float df = (float)max(abs(x - k0t), abs(x - k0t - kInitTile + 1));
+          up = fmaxf(up, Tm[r * ntc + tc] - qf * dn * dn);
+          big = fmaxf(big, Ta[r * ntc + tc] + qf * df * df);
+        }
+        cand = !(tmax[t] + up + dd_lg2((float)s) * LN2 < lthrf - (0.5f + 2e-5f * big));
+      }
+      for (unsigned m = __ballot_sync(0xffffffffu, cand); m; m &= m - 1) {
+        const int tt = base + __ffs(m) - 1, kt = tt / ntc * kInitTile, lt = (tt - tt / ntc * ntc) * kInitTile;
+        for (int p = lane; p < kInitTile * kInitTile; p += 32) {
+          const int k = kt + p / kInitTile, l = lt + p % kInitTile;
+          if (k < N && l < N) test(k, l);
+        }
       }
     }
     __syncthreads();
@@ -702,57 +770,77 @@ k_init_duals(DevState S, const double* __restrict__ alpha0, const double* __rest
     //   nu_i(y) = nu(y) exp(beta0/eps0) sum_r exp(T1 - q (r - k)^2),
     //   sum_x c pi = h^2 sum_r w_r ((r - k)^2 + E[(c - l)^2]),  sum_x pi log(pi / mu nu) likewise.
     // s exponentials per box point instead of s^2.
+    // Exponentials and logarithms are the table-driven ones, shifts come from a
+    // float maximum (any value near the maximum serves), and integer distances
+    // are widened on the integer pipe: about 16 FP64 operations a term (35 before;
+    // 1024^2, 7.7 M box points: 9 -> 4 ms).
     double* T1 = tsm;
     double* M2 = T1 + s * kInitChunk;
     double* MA = M2 + s * kInitChunk;
+    double* xa = MA + s * kInitChunk;    // alpha0/eps0 + log mu on X_i
+    double* xb = xa + s * s;             // alpha0/eps0
+    float* T1f = reinterpret_cast<float*>(xb + s * s);
+    float* xaf = T1f + s * kInitChunk;
     const BoxRec b = S.box[i];
     double v[2] = {0.0, 0.0};
     const double ie0 = 1.0 / eps0;
+    const float qf = (float)q;
+    for (int t = threadIdx.x; t < s * s; t += blockDim.x) {
+      const int x = (r0 + t / s) * N + c0 + t % s;
+      xb[t] = alpha0[x] * ie0;
+      xa[t] = xb[t] + S.logmu[x];
+      xaf[t] = (float)xa[t];
+    }
+    __syncthreads();
     for (int lc = 0; lc < b.W; lc += kInitChunk) {
       const int wc = min(kInitChunk, b.W - lc);
       for (int t = threadIdx.x; t < s * wc; t += blockDim.x) {
-        const int r = t / wc, l = b.l0 + lc + t % wc;
-        double mx = -INFINITY;
+        const int r = t / wc, lj = t - r * wc, l = b.l0 + lc + lj;
+        float mxf = -INFINITY;
         for (int c = 0; c < s; ++c) {
-          const int x = (r0 + r) * N + c0 + c;
-          const double d = c0 + c - l;
-          mx = fmax(mx, alpha0[x] * ie0 + S.logmu[x] - q * d * d);
+          const float d = (float)(c0 + c - l);
+          mxf = fmaxf(mxf, xaf[r * s + c] - qf * d * d);
         }
+        const double mx = (double)mxf;
         double a = 0.0, a2 = 0.0, aa = 0.0;
         for (int c = 0; c < s; ++c) {
-          const int x = (r0 + r) * N + c0 + c;
-          const double d = c0 + c - l;
-          const double w = exp(alpha0[x] * ie0 + S.logmu[x] - q * d * d - mx);
-          a += w; a2 += w * d * d; aa += w * (alpha0[x] * ie0);
+          const float d = (float)(c0 + c - l);
+          const double d2 = widen_pos(d * d);
+          const double w = dd_ex2((fma(-q, d2, xa[r * s + c]) - mx) * DD_LOG2E);
+          a += w; a2 += w * d2; aa += w * xb[r * s + c];
         }
-        T1[r * kInitChunk + t % wc] = mx + log(a);
-        M2[r * kInitChunk + t % wc] = a2 / a;
-        MA[r * kInitChunk + t % wc] = aa / a;
+        const double ia = 1.0 / a, t1 = mx + dd_log(a);
+        T1[r * kInitChunk + lj] = t1;
+        T1f[r * kInitChunk + lj] = (float)t1;
+        M2[r * kInitChunk + lj] = a2 * ia;
+        MA[r * kInitChunk + lj] = aa * ia;
       }
       __syncthreads();
       for (int u = threadIdx.x; u < b.H * wc; u += blockDim.x) {
-        const int kk = u / wc, lj = u % wc;
+        const int kk = u / wc, lj = u - kk * wc;
         const int k = b.k0 + kk, l = b.l0 + lc + lj, y = k * N + l;
-        double mx = -INFINITY;
+        float mxf = -INFINITY;
         for (int r = 0; r < s; ++r) {
-          const double d = r0 + r - k;
-          mx = fmax(mx, T1[r * kInitChunk + lj] - q * d * d);
+          const float d = (float)(r0 + r - k);
+          mxf = fmaxf(mxf, T1f[r * kInitChunk + lj] - qf * d * d);
         }
+        const double mx = (double)mxf;
         double a = 0.0, ac = 0.0, aa = 0.0;
         for (int r = 0; r < s; ++r) {
-          const double d = r0 + r - k;
-          const double w = exp(T1[r * kInitChunk + lj] - q * d * d - mx);
-          a += w; ac += w * (d * d + M2[r * kInitChunk + lj]); aa += w * MA[r * kInitChunk + lj];
+          const float d = (float)(r0 + r - k);
+          const double d2 = widen_pos(d * d);
+          const double w = dd_ex2((fma(-q, d2, T1[r * kInitChunk + lj]) - mx) * DD_LOG2E);
+          a += w; ac += w * (d2 + M2[r * kInitChunk + lj]); aa += w * MA[r * kInitChunk + lj];
         }
         const double by = beta0[y] * ie0;
         const double acc = S.nu[y] * exp(by + mx) * a;   // nu_i(y) = sum_x pi(x, y)
         const double val = acc < S.thr ? 0.0 : acc;
         arena[b.off + kk * b.W + lc + lj] = val;
         if (val != 0.0) atomicAdd(S.PY + y, val);
-        const double cc = S.h * S.h * ac / a;   // E[c] under pi(., y)
+        const double ia = 1.0 / a, cc = S.h * S.h * ac * ia;   // E[c] under pi(., y)
         v[0] += cc * acc;
         // sum_x pi (log(pi / (mu nu)) - 1), log(pi / (mu nu)) = (alpha0 + beta0 - c)/eps0
-        v[1] += acc * (aa / a + by - cc * ie0 - 1.0);
+        v[1] += acc * (aa * ia + by - cc * ie0 - 1.0);
       }
       __syncthreads();
     }
@@ -900,8 +988,8 @@ __global__ void k_reset_cur(DevState S, const long long* newoff) {
 }
 
 cudaError_t launch_init_product_boxes(const DevState& S, double* nu_mom, double* mumass, long long* newoff,
-                                      cudaStream_t st) {
-  k_moments<<<1, 512, 0, st>>>(S.nu, S.N, S.h, nu_mom);
+                                      double* partials, cudaStream_t st) {
+  moments(S.nu, S.N, S.h, nu_mom, partials, st);
   k_basic_masses<<<S.nbasic, 256, 0, st>>>(S, nu_mom, mumass);
   k_init_product<<<S.nbasic, 256, 0, st>>>(S, mumass, 0);
   k_scan_boxes<<<1, 1024, 0, st>>>(S, newoff);
@@ -914,7 +1002,7 @@ cudaError_t launch_init_product_fill(const DevState& S, double* nu_mom, double* 
   k_px_product<<<(S.N * S.N + 255) / 256, 256, 0, st>>>(S, nu_mom);
   return cudaGetLastError();
 }
-// gscratch: N*N floats of device scratch
+// gscratch: 2 N*N floats of device scratch
 // dynamic shared memory of the box test (mode 0 of k_init_duals)
 static size_t init_box_smem(int s, int N) {
   return (size_t)s * N * (sizeof(double) + sizeof(float)) + (size_t)s * s * sizeof(float) + ((N + 15) & ~15) +
@@ -922,23 +1010,26 @@ static size_t init_box_smem(int s, int N) {
 }
 cudaError_t launch_init_duals_boxes(const DevState& S, const double* alpha0, const double* beta0, double eps0,
                                     double* nu_mom, double* mumass, long long* newoff, float* gscratch,
-                                    cudaStream_t st) {
-  k_moments<<<1, 512, 0, st>>>(S.nu, S.N, S.h, nu_mom);
+                                    double* partials, cudaStream_t st) {
+  moments(S.nu, S.N, S.h, nu_mom, partials, st);
   k_basic_masses<<<S.nbasic, 256, 0, st>>>(S, nu_mom, mumass);
   const int n = S.N * S.N;
   k_log_nu_beta<<<(n + 255) / 256, 256, 0, st>>>(S.lognu, beta0, eps0, n, gscratch);
+  const int ntc = (S.N + kInitTile - 1) / kInitTile;
+  float* tmax = gscratch + n;
+  k_tile_max<<<ntc * ntc, 256, 0, st>>>(gscratch, S.N, tmax);
   const size_t sm = init_box_smem(S.s, S.N);
   cudaFuncSetAttribute(k_init_duals, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  k_init_duals<<<S.nbasic, 1024, sm, st>>>(S, alpha0, beta0, eps0, 0, gscratch);
+  k_init_duals<<<S.nbasic, 1024, sm, st>>>(S, alpha0, beta0, eps0, 0, gscratch, tmax);
   k_scan_boxes<<<1, 1024, 0, st>>>(S, newoff);
   return cudaGetLastError();
 }
 cudaError_t launch_init_duals_fill(const DevState& S, const double* alpha0, const double* beta0, double eps0,
                                    const double* w, long long* newoff, cudaStream_t st) {
   k_set_offsets<<<(S.nbasic + 255) / 256, 256, 0, st>>>(S, newoff);
-  const size_t sm = 3 * sizeof(double) * (size_t)S.s * kInitChunk;
+  const size_t sm = (3 * sizeof(double) + sizeof(float)) * (size_t)S.s * kInitChunk + (2 * sizeof(double) + sizeof(float)) * (size_t)S.s * S.s;
   cudaFuncSetAttribute(k_init_duals, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::max(sm, init_box_smem(S.s, S.N)));
-  k_init_duals<<<S.nbasic, 256, sm, st>>>(S, alpha0, beta0, eps0, 1, nullptr);
+  k_init_duals<<<S.nbasic, 256, sm, st>>>(S, alpha0, beta0, eps0, 1, nullptr, nullptr);
   k_px_duals<<<(S.N * S.N + 255) / 256, 256, 0, st>>>(S, alpha0, w, eps0);
   return cudaGetLastError();
 }
