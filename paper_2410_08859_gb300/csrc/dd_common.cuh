@@ -294,6 +294,30 @@ __device__ __forceinline__ void block_sum(T (&v)[K], T* scratch) {
   __syncthreads();
 }
 
+// block_sum through shared memory: the np first threads store their K values, warp
+// k mod (number of warps) adds value k (np / 32 additions a lane, then five
+// shuffles).  On the two-lane FP64 pipe this is K (np / 32 + 5) warp additions
+// where the shuffles of every warp are 5 K np / 32 (14 values of 512 threads:
+// 18 k clocks; 14 of 128: 2 k).  sm: K * np + K doubles; ends with a barrier.
+template <int K>
+__device__ __forceinline__ void block_sum_wide(double (&v)[K], double* sm, int np) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+  if ((int)threadIdx.x < np)
+#pragma unroll
+    for (int k = 0; k < K; ++k) sm[k * np + threadIdx.x] = v[k];
+  __syncthreads();
+  for (int k = wid; k < K; k += nw) {
+    double a = 0.0;
+    for (int i = lane; i < np; i += 32) a += sm[k * np + i];
+    a = warp_sum(a);
+    if (lane == 0) sm[K * np + k] = a;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < K; ++k) v[k] = sm[K * np + k];
+  __syncthreads();
+}
+
 // block_sum of doubles carried as unevaluated sums of two floats through the warp
 // shuffles (TwoSum, Knuth): 48 bits of the running sum on the FP32 pipe, where
 // the double shuffles of 16 warps take 16 clocks an addition on the FP64 pipe

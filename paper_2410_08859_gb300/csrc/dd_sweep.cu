@@ -24,7 +24,8 @@ __device__ __forceinline__ double kl_term_log(double p, double m, double log_m) 
 // theta = 1/|b|; decision on the device, deterministic fixed-order reductions.
 __device__ __forceinline__ void decide_body(const DevState& S, const CellDesc* __restrict__ cells, int begin,
                                             int nbatch, int bid, int nblk) {
-  __shared__ double red[33 * 5];
+  constexpr int kSumThreads = 128;   // threads of the last block's reduction (its lists are a few hundred long)
+  __shared__ double red[14 * kSumThreads > 5 * 512 ? 14 * kSumThreads + 14 : 5 * 512 + 5];
   __shared__ bool is_last;
   __shared__ unsigned long long smax[2];   // largest iteration count and Y box of the sub-batch
   if (*(volatile int*)S.status & ST_HALT) return;   // halted until the host reruns the sub-batch
@@ -56,7 +57,7 @@ __device__ __forceinline__ void decide_body(const DevState& S, const CellDesc* _
   }
   for (int i = bid * blockDim.x + threadIdx.x; i < S.nbasic; i += nblk * blockDim.x)
     v[4] += S.Cc[i] + eps * S.Hh[i];
-  block_sum<5>(v, red);
+  block_sum_wide<5>(v, red, 512);
   if (threadIdx.x == 0) {
     for (int k = 0; k < 5; ++k) S.red[bid * 5 + k] = v[k];
     __threadfence();
@@ -71,9 +72,10 @@ __device__ __forceinline__ void decide_body(const DevState& S, const CellDesc* _
   // stopped at maxit, exp terms, Y-box points), added to the handle's counters
   // only when the sub-batch goes ahead (a halted one is solved again later)
   double tot[14] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-  for (int b = threadIdx.x; b < nblk; b += blockDim.x)
+  const int t0 = threadIdx.x < kSumThreads ? (int)threadIdx.x : 1 << 30;
+  for (int b = t0; b < nblk; b += kSumThreads)
     for (int k = 0; k < 5; ++k) tot[k] += ((volatile double*)S.red)[b * 5 + k];
-  for (int j = threadIdx.x; j < nbatch; j += blockDim.x) {
+  for (int j = t0; j < nbatch; j += kSumThreads) {
     const CellOut& o = S.cout[j];
     if (o.status == CELL_EMPTY || o.status == CELL_TOOBIG) continue;
     const CellDesc cd = cells[begin + j];
@@ -96,8 +98,7 @@ __device__ __forceinline__ void decide_body(const DevState& S, const CellDesc* _
     atomicMax(&smax[0], (unsigned long long)o.iters);
     atomicMax(&smax[1], (unsigned long long)(o.H * o.W));
   }
-  __shared__ double red14[33 * 14];
-  block_sum<14>(tot, red14);
+  block_sum_wide<14>(tot, red, kSumThreads);
   if (threadIdx.x != 0) return;
   // reserve the arena space of the sub-batch's new boxes before anything changes
   if ((double)*S.head + tot[8] > (double)S.cap) {
@@ -185,46 +186,8 @@ k_decide_multi(const DevState* __restrict__ states, int part, int sub) {
 constexpr int kLineIters = 48;
 constexpr double kLineGtol = 1e-12, kLineXtol = 1e-12, kLinePfloor = 1e-300;
 
-// Block partials of [<d, log(p(z)/m)>, <d^2, 1/p(z)>, <|d log(p(z)/m)|>, <d, log(p(lo)/m)>]
-// at z = 1 (first == 1, also at lo) or at z = S.line[2].
-__global__ void __launch_bounds__(512)
-k_line_eval(DevState S, const CellDesc* __restrict__ cells, int begin, int nbatch, int first, double* partials) {
-  __shared__ double red[33 * 4];
-  if (S.line[5] != 0.0 || (*(volatile int*)S.status & ST_HALT)) return;   // uniform across blocks
-  const double z = first ? 1.0 : S.line[2], lo = S.line[6];
-  double v[4] = {0.0, 0.0, 0.0, 0.0};
-  auto term = [&](double p0, double d, double m) {
-    const double p = fmax(p0 + z * d, kLinePfloor);
-    const double t = d * log(p / m);
-    v[0] += t;
-    v[1] += d * d / p;
-    v[2] += fabs(t);
-    if (first) v[3] += d * log(fmax(p0 + lo * d, kLinePfloor) / m);
-  };
-  const int N = S.N;
-  for (int j = blockIdx.x; j < nbatch; j += gridDim.x) {
-    const CellOut& o = S.cout[j];
-    if (o.status == CELL_EMPTY || o.status == CELL_TOOBIG) continue;
-    const CellDesc cd = cells[begin + j];
-    const int nx = cd.nx1 * cd.nx2;
-    for (int t = threadIdx.x; t < nx; t += blockDim.x) {
-      const int r = t / cd.nx2, c = t - r * cd.nx2;
-      const int x = (cd.i0 + r) * N + cd.j0 + c;
-      const double p0 = S.PX[x], d = S.PXnew[x] - p0;
-      if (d != 0.0) term(p0, d, S.mu[x]);
-    }
-  }
-  const int n = N * N;
-  for (int y = blockIdx.x * blockDim.x + threadIdx.x; y < n; y += gridDim.x * blockDim.x) {
-    const double d = S.dPY[y];
-    if (d != 0.0) term(S.PY[y], d, S.nu[y]);
-  }
-  block_sum_to<4>(v, red, partials);
-}
-
-// One step of the search from the sums of the last evaluation (one thread).
-__global__ void k_line_step(DevState S, int first, int last) {
-  if (threadIdx.x != 0 || S.line[5] != 0.0 || (*(volatile int*)S.status & ST_HALT)) return;
+// One step of the search, from the summed terms of an evaluation (one thread).
+__device__ __forceinline__ void line_step(const DevState& S, int first, int last) {
   double* L = S.line;
   const double lam = S.lam;
   const double g = L[7] + lam * L[12], h = lam * L[13], scale = fabs(L[7]) + lam * L[14];
@@ -252,6 +215,67 @@ __global__ void k_line_step(DevState S, int first, int last) {
   const unsigned long long slot = (*S.slotctr + DD_LOGCAP - 1) % DD_LOGCAP;
   S.declog[4 * slot + 3] = zeta;
   atomicAdd(S.counters + (zeta == 1.0 ? 3 : 4), 1ull);
+}
+
+// One evaluation and step: the terms [<d, log(p(z)/m)>, <d^2, 1/p(z)>,
+// <|d log(p(z)/m)|>, <d, log(p(lo)/m)>] at z = 1 (first == 1, also at lo) or at
+// z = S.line[2]; the block that finishes last adds the block partials in order and
+// makes the step.  (Evaluation, sum and step were three launches of 6.5, 8 and
+// 1.7 us; a launch after the search has stopped returns at once.)
+__global__ void __launch_bounds__(512)
+k_line(DevState S, const CellDesc* __restrict__ cells, int begin, int nbatch, int first, int last, double* partials) {
+  __shared__ double red[4 * 512 + 4];
+  __shared__ bool is_last;
+  if (S.line[5] != 0.0 || (*(volatile int*)S.status & ST_HALT)) return;   // uniform across blocks
+  const double z = first ? 1.0 : S.line[2], lo = S.line[6];
+  double v[4] = {0.0, 0.0, 0.0, 0.0};
+  auto term = [&](double p0, double d, double log_m) {
+    const double p = fmax(p0 + z * d, kLinePfloor);
+    const double t = d * (dd_log(p) - log_m);
+    v[0] += t;
+    v[1] += d * d * dd_rcp(p);
+    v[2] += fabs(t);
+    if (first) v[3] += d * (dd_log(fmax(p0 + lo * d, kLinePfloor)) - log_m);
+  };
+  const int N = S.N;
+  for (int j = blockIdx.x; j < nbatch; j += gridDim.x) {
+    const CellOut& o = S.cout[j];
+    if (o.status == CELL_EMPTY || o.status == CELL_TOOBIG) continue;
+    const CellDesc cd = cells[begin + j];
+    const int nx = cd.nx1 * cd.nx2;
+    for (int t = threadIdx.x; t < nx; t += blockDim.x) {
+      const int r = t / cd.nx2, c = t - r * cd.nx2;
+      const int x = (cd.i0 + r) * N + cd.j0 + c;
+      const double p0 = S.PX[x], d = S.PXnew[x] - p0;
+      if (d != 0.0) term(p0, d, S.logmu[x]);
+    }
+  }
+  const int n = N * N;
+  for (int y = blockIdx.x * blockDim.x + threadIdx.x; y < n; y += gridDim.x * blockDim.x) {
+    const double d = S.dPY[y];
+    if (d != 0.0) term(S.PY[y], d, S.lognu[y]);
+  }
+  block_sum_wide<4>(v, red, 512);
+  if (threadIdx.x == 0) {
+    for (int k = 0; k < 4; ++k) partials[blockIdx.x * 4 + k] = v[k];
+    __threadfence();
+    is_last = atomicAdd(S.red_count, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!is_last) return;
+  __threadfence();
+  const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (k < 4) {
+    double a = 0.0;
+    for (int g = lane; g < (int)gridDim.x; g += 32) a += ((volatile double*)partials)[g * 4 + k];
+    a = warp_sum(a);
+    if (lane == 0) S.line[12 + k] = a;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    *S.red_count = 0u;
+    line_step(S, first, last);
+  }
 }
 
 // ================================================================= apply (a7)
@@ -925,9 +949,7 @@ cudaError_t launch_line_search(const DevState& S, const CellDesc* cells, int beg
   if (G < nbatch) G = nbatch;
   if (G > kRedBlocks) G = kRedBlocks;
   for (int k = 0; k <= kLineIters; ++k) {
-    k_line_eval<<<G, 512, 0, st>>>(S, cells, begin, nbatch, k == 0, partials);
-    k_sum_partials<<<1, 32 * 4, 0, st>>>(partials, G, 4, S.line + 12);
-    k_line_step<<<1, 32, 0, st>>>(S, k == 0, k == kLineIters);
+    k_line<<<G, 512, 0, st>>>(S, cells, begin, nbatch, k == 0, k == kLineIters, partials);
   }
   return cudaGetLastError();
 }
