@@ -584,6 +584,13 @@ int domdec_init(domdec_t* out, const double* mu, const double* nu, int N, const 
   // one CTA per cell with balancing or the translation step
   {
     int C = pin->cell_ctas == 0 ? (h->s <= 8 ? 4 : 8) : pin->cell_ctas;
+    // double cells are bound by the FP64 pipe of their SMs: where a sub-batch has
+    // too few of them to fill the GPU with clusters of four, clusters of eight
+    if (pin->cell_ctas == 0 && pin->precision) {
+      const int nc = N / (2 * h->s) + 1;
+      const bool stag = pin->strategy == DOMDEC_STAGGERED || pin->strategy == DOMDEC_STAGGERED_LINE;
+      if ((stag ? ((nc + 1) / 2) * ((nc + 1) / 2) : nc * nc) * 8 <= 152) C = 8;
+    }
     if (pin->balance || pin->cell_ti) C = 1;
     h->order_mode = pin->cell_ctas == 0 ? 0 : 1;
     const size_t rs = pin->precision ? sizeof(double) : sizeof(float);

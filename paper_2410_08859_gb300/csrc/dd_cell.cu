@@ -369,12 +369,58 @@ __device__ __forceinline__ void run_pass(const float* src, int sl, int sm, const
     pass_tiles<1>(src, sl, sm, prev, ol, oj, L, J, M, off, q2, first, tid, nthr, put);
 }
 
+// ---- double passes: one target on a group of P lanes.  The FP64 pipe gives two
+// lanes a clock, so a term (12 operations) is evaluated only if a float test
+// finds it within 2^-65 of the target's shift (at eps = h^2: 13 of 32 sources);
+// narrowing and widening run on the integer pipe.  A sum below 2^-4 of its
+// shift, and a target without a previous value, is taken against the float
+// maximum, so what is left out is below 32 * 2^-61 = 2^-56 of the sum.
+__device__ __forceinline__ double lse_lanes_f64(const double* row, int sm, int M, int ctr, double q2, double shift,
+                                                bool have, int part, int P) {
+  const float q2f = (float)q2;
+  double acc = 0.0;
+  bool todo = true;
+  for (int pass = have ? 0 : 1; pass < 2; ++pass) {
+    if (pass == 1) {
+      float mx = -INFINITY;
+      for (int m = part; m < M; m += P) {
+        const float d = (float)(m - ctr);
+        mx = fmaxf(mx, fmaf(-q2f * d, d, narrow(row[m * sm])));
+      }
+      for (int o = 1; o < P; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      if (todo) shift = mx > -INFINITY ? (double)mx : 0.0;
+    }
+    const float sf = (float)shift;
+    double a = 0.0;
+    for (int m = part; m < M; m += P) {
+      const float d = (float)(m - ctr);
+      const double v = row[m * sm];
+      if (!(fmaf(-q2f * d, d, narrow(v)) - sf < -65.0f)) a += dd_ex2(fma(-q2, widen_pos(d * d), v) - shift);
+    }
+    for (int o = 1; o < P; o <<= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    if (todo) acc = a;
+    if (pass == 0) {
+      todo = !(acc > 0.0625 && acc < 1e25);
+      if (!__any_sync(0xffffffffu, todo)) break;
+    }
+  }
+  return shift + dd_lg2(acc);
+}
+
 template <typename Put>
 __device__ __forceinline__ void run_pass(const double* src, int sl, int sm, const double* prev, int ol, int oj, int L,
                                          int J, int M, int off, double q2, bool first, int tid, int nthr, Put put,
                                          bool = false) {
-  pass_lanes<double>(src, sl, sm, prev, ol, oj, L, J, M, off, q2, first, lanes_per_target(L * J, M, nthr), tid, nthr,
-                     put);
+  const int nt = L * J, P = lanes_per_target(nt, M, nthr), ni = (nt * P + 31) & ~31, lp = 31 - __clz(P);
+  const float iL = 1.0f / (float)L;
+  for (int i = tid; i < ni; i += nthr) {
+    const int tg0 = i >> lp, part = i & (P - 1), tg = min(tg0, nt - 1);
+    const int j = quot(tg, L, iL), l = tg - j * L;
+    double v[1];
+    v[0] = lse_lanes_f64(src + l * sl, sm, M, j + off, q2, prev[l * ol + j * oj], !first, part, P);
+    __syncwarp();
+    if (part == 0 && tg0 < nt) put(l, j, 1, v);
+  }
 }
 
 // Roots u of g(u) = (1+s) u + c0 + softplus(lr - u) = 0, i.e. of
@@ -455,6 +501,50 @@ __device__ __forceinline__ R newton_rest(R lr, R c0, R u, R s, int steps) {
   return u;
 }
 
+// The root in double.  A float solve gives the start (or the previous root, if it
+// lies within 0.05 of it); double steps with the second-order correction
+// du (1 + du g''/(2 g')) follow, whose error is below |du|^3 / 2, so a step of at
+// most 1e-5 is the last: two steps as a rule (six to eight first-order ones
+// before).  About 40 FP64 operations a step: table-driven 2^x and logarithm, the
+// reciprocal from the float one, one division-free slope.
+__device__ __forceinline__ double newton_f64(double lr, double c0, double uw, double s, double is, double i1s,
+                                             int maxit) {
+  double u = -c0 * i1s;
+  if (!(lr > -dd_inf<double>())) return u;   // rho = 0: closed form (Eq. sinkhorn-iters-ot)
+  if (s > 0.0) u = fmin(u, -(lr + c0) * is);
+  const double bound = u;                    // right of the root
+  const float lrf = (float)lr, c0f = (float)c0, sf = (float)s;
+  float uf = (float)u;
+  {
+    const float w = (float)uw;
+    float du;
+    const float wn = newton_next(lrf, c0f, w, 1.0f + sf, &du);
+    if (wn == wn && wn < uf) uf = wn;
+    for (int it = 0; it < 8; ++it) {
+      uf = newton_next(lrf, c0f, uf, 1.0f + sf, &du);
+      if (fabsf(du) <= 1e-3f * fmaxf(1.0f, fabsf(uf))) break;
+    }
+    if (fabsf(uf) < 1e6f) u = fmin(u, (double)uf);
+    if (fabsf(w - uf) < 0.05f) u = fmin(bound, uw);
+  }
+  const double one_s = 1.0 + s;
+  for (int it = 0; it < maxit; ++it) {
+    const double t = lr - u;
+    const double e = dd_ex2(-fabs(t) * DD_LOG2E), op = 1.0 + e;
+    const double g = fma(one_s, u, c0) + (fmax(t, 0.0) + dd_lg2(op) * DD_LN2);
+    const double den = fma(s, op, t >= 0.0 ? e : 1.0);
+    const double du0 = g * op * dd_rcp(den);
+    // g''/(2 g') in float: it only corrects a small step
+    const float h = 0.5f * narrow(e) * dd_rcp(narrow(op) * narrow(den));
+    const float d0 = narrow(du0);
+    double du = du0;
+    if (fabsf(d0) < 0.1f) du = fma(du0, (double)(h * d0), du0);
+    u = fmin(u - du, bound);
+    if (fabsf(d0) <= 1e-5f) break;
+  }
+  return u;
+}
+
 constexpr int kLock = 4;     // Newton steps made in lock-step by every warp (float cells)
 constexpr int kPend = 512;   // targets listed for the remaining steps (more are finished in place)
 
@@ -504,7 +594,7 @@ __device__ __forceinline__ void cell_sum(double (&v)[K], double* scratch) {
 template <typename R>
 struct CellScalars {
   double A, qD2;   // alpha/eps = A + a + 2 q D.xi; beta/eps = q|D|^2 - A + b - 2 q D.eta
-  R q2, qR, sR, rR, sB, cEta1, cEta2, cA, gA, cD1, cD2, tol;
+  R q2, qR, sR, rR, sB, cEta1, cEta2, cA, gA, cD1, cD2, tol, is, i1s;
   __device__ __forceinline__ void set_A(const DevState& S, double a) {
     A = a;
     sB = R(S.sl * (qD2 - A));   // s B
@@ -517,6 +607,8 @@ struct CellScalars {
     cEta1 = R(S.sl * 2.0 * S.q * D1); cEta2 = R(S.sl * 2.0 * S.q * D2);
     cD1 = R(2.0 * (1.0 - S.rr) * S.q * D1); cD2 = R(2.0 * (1.0 - S.rr) * S.q * D2);
     // gap <= err |mu_J| in the working precision: the largest value not above the bound
+    is = R(1) / sR;
+    i1s = R(1) / (R(1) + sR);
     const double t = S.err * muJ;
     if constexpr (sizeof(R) == 4) tol = __double2float_rd(t);
     else tol = t;
@@ -707,6 +799,9 @@ __device__ __forceinline__ void cell_solve_body(const DevState& S, const CellDes
   // the gap is reduced from per-warp partials after that pass's barrier.
   const R LN2 = R(DD_LN2), L2E = R(DD_LOG2E);
   const bool stops = S.err >= 0.0;
+  const R is = sk.is, i1s = sk.i1s;   // 1/s, 1/(1 + s) (double cells)
+  (void)is;
+  (void)i1s;
   R* gpart = reinterpret_cast<R*>(red) + 32 * 12;   // per-warp gap partials
   R* apart = gpart + 32;                             // per-warp <e^{-alpha/lam}, mu> (translation step)
   R* bpart = gpart + 64;                             // per-warp <e^{-beta/lam}, nu>
@@ -762,7 +857,12 @@ __device__ __forceinline__ void cell_solve_body(const DevState& S, const CellDes
         uw[k] = first ? dd_inf<R>() : bv[v] + Zn[k];
       }
       bool open[B];
-      newton_tile<R, B>(lr, c0, uw, sR, min(S.newton_maxit, lock), root, open);
+      if constexpr (sizeof(R) == 8) {
+        root[0] = newton_f64(lr[0], c0[0], uw[0], sR, is, i1s, S.newton_maxit);
+        open[0] = false;
+      } else {
+        newton_tile<R, B>(lr, c0, uw, sR, min(S.newton_maxit, lock), root, open);
+      }
 #pragma unroll
       for (int k = 0; k < B; ++k) {
         if (k >= n) break;
@@ -1375,6 +1475,9 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
   // ------------------------------------------------------- Sinkhorn loop
   const R LN2 = R(DD_LN2), L2E = R(DD_LOG2E);
   const bool stops = S.err >= 0.0;
+  const R is = sk.is, i1s = sk.i1s;   // 1/s, 1/(1 + s) (double cells)
+  (void)is;
+  (void)i1s;
   int* pend = reinterpret_cast<int*>(red + 256);    // as in cell_solve_body
   const int lock = sizeof(R) == 4 ? kLock : S.newton_maxit;
   int it = 0;
@@ -1415,7 +1518,12 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
         uw[k] = first ? dd_inf<R>() : bv[v] + Zn[k];
       }
       bool open[B];
-      newton_tile<R, B>(lr, c0, uw, sR, min(S.newton_maxit, lock), root, open);
+      if constexpr (sizeof(R) == 8) {
+        root[0] = newton_f64(lr[0], c0[0], uw[0], sR, is, i1s, S.newton_maxit);
+        open[0] = false;
+      } else {
+        newton_tile<R, B>(lr, c0, uw, sR, min(S.newton_maxit, lock), root, open);
+      }
 #pragma unroll
       for (int k = 0; k < B; ++k) {
         if (k >= n) break;
