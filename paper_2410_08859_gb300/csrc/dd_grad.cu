@@ -30,9 +30,17 @@
 // float carries only ~1e-3 absolute.  Each surviving term's exponent
 // f - Q d^2 - max is formed in double (three operations) and only the
 // exponential and the sums run in R: float (ex2.approx) or double.
+//
+// In double, grids of kTileMinN and more use the tile passes of dd_tiles.cuh
+// instead (both stored transposed, so the second runs along the columns): a term
+// takes 2.4 (no moment) to 5 (two moments) FP64 operations there where a term of its own
+// exponential takes 12 to 16.  512 x 512, eps = (2/N)^2, the whole call:
+// 2.63 ms (CUDA exp2) -> 2.02 (table exponential) -> 1.26 (tiles); below
+// kTileMinN the tiles are too few to hide the FP64 latency (N = 150: 32 us a pass
+// against 28).
 #include <cmath>
 
-#include "dd_common.cuh"
+#include "dd_tiles.cuh"
 #include "domdec.h"
 
 namespace {
@@ -138,6 +146,24 @@ struct AdjOut {
   double eps, lam, h;
 };
 
+// The gradient entries of point x from its log2-sum L and the mean displacements.
+template <bool MOM>
+__device__ __forceinline__ void adj_store(const AdjOut& O, long long x, double L, double m1, double m2) {
+  const double eps = O.eps, lam = O.lam;
+  const double pot = O.pot[x], w = O.mu[x];
+  // P(x)/w(x) = exp(pot/eps + L ln 2)
+  const double ratio = exp(pot / eps + L * DD_LN2);
+  const double marg = w * ratio;
+  O.marg[x] = marg;
+  const double other = O.sums[O.side == 0 ? 1 : 0];
+  const double pen = isfinite(lam) ? -lam * (exp(-pot / lam) - 1.0) : pot;
+  O.grad[x] = eps * other - eps * ratio + pen;
+  if (MOM && O.grad_x) {
+    O.grad_x[2 * x] = -2.0 * marg * O.h * m1;
+    O.grad_x[2 * x + 1] = -2.0 * marg * O.h * m2;
+  }
+}
+
 // Pass 2 (block = (column tile, grid row i)) and the gradient epilogue.
 template <typename R, bool MOM>
 __global__ void __launch_bounds__(256) k_adj_cols(AdjBufs<R> B, AdjOut O, int N, double Q) {
@@ -157,20 +183,53 @@ __global__ void __launch_bounds__(256) k_adj_cols(AdjBufs<R> B, AdjOut O, int N,
       },
       N, i, (float)Q, Q, part, P, mo);
   if (part != 0 || j0 >= N) return;
-  const long long x = (long long)i * N + j;
-  const double eps = O.eps, lam = O.lam;
-  const double pot = O.pot[x], w = O.mu[x];
-  // P(x)/w(x) = exp(pot/eps + L ln 2)
-  const double ratio = exp(pot / eps + L * DD_LN2);
-  const double marg = w * ratio;
-  O.marg[x] = marg;
-  const double other = O.sums[O.side == 0 ? 1 : 0];
-  const double pen = isfinite(lam) ? -lam * (exp(-pot / lam) - 1.0) : pot;
-  O.grad[x] = eps * other - eps * ratio + pen;
-  if (MOM && O.grad_x) {
-    O.grad_x[2 * x] = -2.0 * marg * O.h * (double)mo[0];
-    O.grad_x[2 * x + 1] = -2.0 * marg * O.h * (double)mo[1];
-  }
+  adj_store<MOM>(O, (long long)i * N + j, L, (double)mo[0], MOM ? (double)mo[1] : 0.0);
+}
+
+// The tile passes: a[j, k] and, with MOM, m[j, k] (transposed) ...
+template <int P, bool MOM>
+__global__ void __launch_bounds__(512)
+k_adj_first(const double* __restrict__ f, const float* __restrict__ fs, double* __restrict__ a, float* __restrict__ as,
+            double* __restrict__ m, int N, double Q, int per, int D4) {
+  extern __shared__ __align__(16) unsigned char sm[];
+  const int k = blockIdx.x;
+  tile_rows<P, MOM ? 1 : 0>(sm, f, fs, nullptr, N, Q, per, D4, [&](int j, double v, double m1, double) {
+    const long long o = (long long)j * N + k;
+    a[o] = v;
+    as[o] = (float)v;
+    if (MOM) m[o] = m1;
+  });
+}
+
+// ... then along the columns of the grid, with the gradient epilogue.
+template <int P, bool MOM>
+__global__ void __launch_bounds__(512)
+k_adj_second(const double* __restrict__ a, const float* __restrict__ as, const double* __restrict__ m, AdjOut O, int N,
+             double Q, int per, int D4) {
+  extern __shared__ __align__(16) unsigned char sm[];
+  const int j = blockIdx.x;
+  tile_rows<P, MOM ? 2 : 0>(sm, a, as, m, N, Q, per, D4, [&](int i, double L, double m1, double m2) {
+    adj_store<MOM>(O, (long long)i * N + j, L, m1, m2);
+  });
+}
+
+// The two passes of one side.
+template <bool MOM>
+cudaError_t adj_side_tiles(const double* f, const float* fs, double* a, float* as, double* m, const AdjOut& O, int N,
+                           double Q, cudaStream_t st) {
+  auto run = [&](auto kernel, const TileShape& t, auto... args) {
+    if (t.smem > 40 * 1024) {
+      const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)t.smem);
+      if (e != cudaSuccess) return e;
+    }
+    kernel<<<t.grid, t.threads, t.smem, st>>>(args..., N, Q, t.per, t.D4);
+    return cudaGetLastError();
+  };
+  const TileShape t1 = tile_shape(N, Q, MOM ? 1 : 0), t2 = tile_shape(N, Q, MOM ? 2 : 0);
+  cudaError_t e = t1.lanes == 8 ? run(k_adj_first<8, MOM>, t1, f, fs, a, as, m) : run(k_adj_first<4, MOM>, t1, f, fs, a, as, m);
+  if (e == cudaSuccess)
+    e = t2.lanes == 8 ? run(k_adj_second<8, MOM>, t2, a, as, m, O) : run(k_adj_second<4, MOM>, t2, a, as, m, O);
+  return e;
 }
 
 // f = (pot/eps + log w) log2 e and its float shadow; marks a non-positive or
@@ -259,14 +318,28 @@ cudaError_t adjoint_impl(const double* mu, const double* nu, const double* alpha
   k_sum_partials<<<1, 32 * 2, 0, st>>>(partials, G, 2, sums);
   // X side: f = beta/eps + log nu summed over y for every x, with moments.
   k_adj_prep<<<eb, 256, 0, st>>>(beta, nu, 1.0 / eps, f, fs, (int)n, d_bad);
-  k_adj_rows<R, true><<<N, thr_rows, smem_rows, st>>>(B, N, Q);
   AdjOut OX{mu, alpha, grad_mu, grad_x, px, sums, 0, eps, lam, h};
-  k_adj_cols<R, true><<<gcols, 256, 0, st>>>(B, OX, N, Q);
+  const bool tiles = sizeof(R) == 8 && N >= kTileMinN;
+  cudaError_t e = cudaSuccess;
+  if constexpr (sizeof(R) == 8) {
+    if (tiles) e = adj_side_tiles<true>(f, fs, a, as, m, OX, N, Q, st);
+  }
+  if (e != cudaSuccess) return e;
+  if (!tiles) {
+    k_adj_rows<R, true><<<N, thr_rows, smem_rows, st>>>(B, N, Q);
+    k_adj_cols<R, true><<<gcols, 256, 0, st>>>(B, OX, N, Q);
+  }
   // Y side: f = alpha/eps + log mu summed over x for every y.
   k_adj_prep<<<eb, 256, 0, st>>>(alpha, mu, 1.0 / eps, f, fs, (int)n, d_bad);
-  k_adj_rows<R, false><<<N, thr_rows, smem_rows, st>>>(B, N, Q);
   AdjOut OY{nu, beta, grad_nu, nullptr, py, sums, 1, eps, lam, h};
-  k_adj_cols<R, false><<<gcols, 256, 0, st>>>(B, OY, N, Q);
+  if constexpr (sizeof(R) == 8) {
+    if (tiles) e = adj_side_tiles<false>(f, fs, a, as, m, OY, N, Q, st);
+  }
+  if (e != cudaSuccess) return e;
+  if (!tiles) {
+    k_adj_rows<R, false><<<N, thr_rows, smem_rows, st>>>(B, N, Q);
+    k_adj_cols<R, false><<<gcols, 256, 0, st>>>(B, OY, N, Q);
+  }
   k_adj_value<<<G, 512, 0, st>>>(mu, nu, alpha, beta, px, py, lam, (int)n, partials);
   k_sum_partials<<<1, 32 * 4, 0, st>>>(partials, G, 4, sums + 4);
   k_adj_finish<<<1, 32, 0, st>>>(sums, sums + 4, eps, d_out);
