@@ -98,10 +98,12 @@ typedef struct {
                           terms of one iteration, from the box sizes).  A cell may be solved by a whole
                           thread-block cluster, its Y box split by rows over the CTAs (each CTA holds its
                           rows' Y-side arrays; the X-half log-sum-exp is combined from per-CTA parts).
-                          0 = automatic: clusters of 4 CTAs (s <= 8) or 8 (s > 8) for the cells whose
+                          0 = automatic: clusters of 4 CTAs (s <= 8), 8 (s > 8, and FP64 when a
+                          sub-batch's clusters of 8 all fit the GPU at once) for the cells whose
                           work exceeds twice the mean work per CTA or whose box exceeds one CTA's
                           shared memory, one CTA for the others; 1 = one CTA per cell; 2, 4, 8 = every
-                          cell whose box fits the cluster layout on a cluster of that many CTAs.  With
+                          cell whose box fits the cluster layout (or does with its per-y arrays in a
+                          spill slot) on a cluster of that many CTAs.  With
                           balance or cell_ti every cell runs on one CTA. */
   int    cell_ti;      /* 1: after each X-half of a cell solve, shift alpha by the t maximising the cell
                           dual along (alpha + t, beta - t) (closed form; not in the paper: it removes the

@@ -701,7 +701,7 @@ __device__ __forceinline__ void cell_solve_body(const DevState& S, const CellDes
   const int Wo = W | 1, Uo = nx2 | 1;
   // A spilled box keeps T, U and beta + log nu, which the passes read many times,
   // in shared memory if those fit; the arrays that each y touches once an
-  // iteration stay in the slot (143 x 81 at s = 8: 3200 -> 1500 kclk a solve).
+  // iteration stay in the slot (143 x 81 at s = 8: 2.15 -> 1.94 ms a solve).
   const int rsz = 4 * s * S.cap_side + 5 * S.cap_ny;
   const bool hyb = spilled && nx1 * Wo + H * Uo + H * Wo <= rsz && 3 * nx1 * W <= rsz && H * Wo <= N * N;
   const int Wp = hyb || (!spilled && nx1 * Wo <= tsz && H * Wo <= cap_ny && 3 * nx1 * Wo <= rsz) ? Wo : W;
@@ -1281,7 +1281,7 @@ __device__ __forceinline__ bool fits_cluster(const DevState& S, int H, int W, in
 }
 // Whether it does with the per-y arrays in a spill slot: T, U and beta + log nu,
 // and the epilogue's three rows-of-X arrays, share the cluster layout's space.
-// (234 x 257 at s = 16: 4.65 ms on one CTA from its slot, 0.5 ms so on eight.)
+// (234 x 257 at s = 16: 4.65 ms on one CTA from its slot, 0.65 to 0.72 ms so on eight.)
 __device__ __forceinline__ bool fits_hybrid(const DevState& S, int nx1, int nx2, int H, int W, int C) {
   if (C < 2 || C > S.dist_c || H < C || S.spill_slots <= 0) return false;
   const long long Wo = W | 1, Hc = (H + C - 1) / C;

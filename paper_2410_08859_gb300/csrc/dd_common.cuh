@@ -189,6 +189,12 @@ __device__ __forceinline__ float narrow(double x) {
   f += (lo & 0x1fffffffu) + (f & 1u) > 0x10000000u ? 1u : 0u;
   return __uint_as_float((f & 0x7fffffffu) | (hi & 0x80000000u));
 }
+// (float)x for every x (the conversion itself for zeros, subnormals, what exceeds
+// the float range, infinities and NaN).
+__device__ __forceinline__ float narrow_any(double x) {
+  const unsigned a = (unsigned)__double2hiint(x) & 0x7fffffffu;
+  return a - 0x38100000u < 0x47e00000u - 0x38100000u ? narrow(x) : (float)x;
+}
 __device__ __forceinline__ double widen_pos(float f) {
   const unsigned u = __float_as_uint(f);
   return __hiloint2double((int)((u >> 3) + 0x38000000u), (int)(u << 29));
@@ -230,13 +236,18 @@ __device__ __forceinline__ double dd_log(double x) {
     e = -54;
   }
   e += (hi >> 20) - 1023;
-  double m = __hiloint2double((hi & 0x000fffff) | 0x3ff00000, lo);   // [1, 2)
-  if (m >= 1.5) {
-    m *= 0.5;
-    e += 1;
-  }
-  const int j = __double2int_rn((m - 1.0) * 128.0);   // -32..64; m - 1 is exact
-  const double f = m - (1.0 + j * 0.0078125);
+  // m in [1, 2); from 1.5 on the nearest c with spacing 1/64, both halved: index,
+  // c_j and e as a double come from integer operations (conversions to and from
+  // double share the FP64 path)
+  const int mh = hi & 0x000fffff;
+  const double m = __hiloint2double(mh | 0x3ff00000, lo);
+  const bool up = mh >= 0x00080000;
+  const int kk = up ? (mh + 0x2000) >> 14 : (mh + 0x1000) >> 13;
+  double f = m - __hiloint2double(0x3ff00000 + (up ? kk << 14 : kk << 13), 0);   // exact
+  f = up ? 0.5 * f : f;
+  const int j = up ? kk - 64 : kk;   // -32..64
+  e += up ? 1 : 0;
+  const double ed = __hiloint2double(0x43300000, (int)((unsigned)e ^ 0x80000000u)) - 4503601774854144.0;   // 2^52 + 2^31
   const double r = f * kInvC[j + 32];
   double p = fma(r, 1.0 / 7.0, -1.0 / 6.0);
   p = fma(p, r, 0.2);
@@ -244,7 +255,7 @@ __device__ __forceinline__ double dd_log(double x) {
   p = fma(p, r, 1.0 / 3.0);
   p = fma(p, r, -0.5);
   const double l1p = fma(p, r * r, r);
-  return fma((double)e, 0.6931471805599453, kLogC[j + 32] + l1p);
+  return fma(ed, 0.6931471805599453, kLogC[j + 32] + l1p);
 }
 
 // mu phi(p/mu) with phi(s) = s log s - s + 1 (phi(0) = 1), in double.
@@ -321,8 +332,9 @@ __device__ __forceinline__ void block_sum_wide(double (&v)[K], double* sm, int n
 // block_sum of doubles carried as unevaluated sums of two floats through the warp
 // shuffles (TwoSum, Knuth): 48 bits of the running sum on the FP32 pipe, where
 // the double shuffles of 16 warps take 16 clocks an addition on the FP64 pipe
-// (12 values: 27 k clocks before, 4 k now).  For finite values within float range
-// (smaller than 2^-126: flushed).
+// (12 values at the end of a cell: 27 k clocks before, 10 to 16 k now, with the wait
+// for the block's last warp).  For finite values within float range (smaller
+// than 2^-126: flushed).
 template <int K>
 __device__ __forceinline__ void block_sum_ff(double (&v)[K], double* scratch) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;

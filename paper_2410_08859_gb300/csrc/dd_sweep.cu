@@ -6,10 +6,12 @@
 #include "dd_common.cuh"
 
 // ============================================================== decision (a6)
-// mu phi(p/mu) in float (the current score's marginal terms; see k_decide).
+// mu phi(p/mu) in float (the current score's marginal terms; see k_decide).  With
+// the conversions here and in dd_log on the integer pipe a decision at 1024^2
+// takes 142 us (186 before).
 __device__ __forceinline__ float kl_term_f(double p, double m) {
-  if (p <= 0.0) return (float)m;
-  float pf = (float)p, mf = (float)m;
+  const float pf = narrow_any(p), mf = narrow_any(m);
+  if (pf <= 0.0f) return mf;
   return pf * (dd_lg2(pf / mf) * (float)DD_LN2) - pf + mf;
 }
 
@@ -601,7 +603,9 @@ __global__ void __launch_bounds__(256) k_tile_max(const float* __restrict__ g, i
 //         largest g, each row's largest T over the tile's columns, the smallest
 //         distance) lies below the threshold by more than the tile's band are left
 //         out: a cell's plan reaches a few dozen of the 4096 tiles of a 1024^2
-//         grid, and testing every pixel took 35 ms there (now 1 ms);
+//         grid, where testing every pixel and the fill with CUDA's exponentials
+//         took 46 ms (both modes; 17 with tiles and tables, 14 with the table
+//         functions in the double part of the test too);
 // mode 1: values on the box (dense over X_i), C_i, H_i, P_Y.
 constexpr int kInitChunk = 128;   // box columns per pass of the dual-initialised fill
 constexpr int kInitBand = 2048;   // band pixels listed per basic cell by the box test
@@ -726,29 +730,31 @@ k_init_duals(DevState S, const double* __restrict__ alpha0, const double* __rest
     for (int t = threadIdx.x; t < s * N; t += blockDim.x) {
       const int r = t / N, l = t - (t / N) * N;
       if (!colflag[l]) continue;
-      double mx = -INFINITY;
-      for (int c = 0; c < s; ++c) {
-        const int x = (r0 + r) * N + c0 + c;
-        const double d = c0 + c - l;
-        mx = fmax(mx, alpha0[x] * ie0 + S.logmu[x] - q * d * d);
-      }
+      const double mx = (double)tsmf[t];   // the float value is a good enough shift
       double acc = 0.0;
       for (int c = 0; c < s; ++c) {
         const int x = (r0 + r) * N + c0 + c;
-        const double d = c0 + c - l;
-        acc += exp(alpha0[x] * ie0 + S.logmu[x] - q * d * d - mx);
+        const float d = (float)(c0 + c - l);
+        acc += dd_ex2((fma(-q, widen_pos(d * d), alpha0[x] * ie0 + S.logmu[x]) - mx) * DD_LOG2E);
       }
-      tsm[t] = mx + log(acc);
+      tsm[t] = mx + dd_log(acc);
     }
     __syncthreads();
     // the double test of the band pixels (rescanning all pixels if the list overflowed)
     auto dtest = [&](int y) {
       const int k = y / N, l = y - (y / N) * N;
-      double mx = -INFINITY;
-      for (int r = 0; r < s; ++r) { const double d = r0 + r - k; mx = fmax(mx, tsm[r * N + l] - q * d * d); }
+      float mxf = -INFINITY;
+      for (int r = 0; r < s; ++r) {
+        const float d = (float)(r0 + r - k);
+        mxf = fmaxf(mxf, tsmf[r * N + l] - qf * d * d);
+      }
+      const double mx = (double)mxf;
       double acc = 0.0;
-      for (int r = 0; r < s; ++r) { const double d = r0 + r - k; acc += exp(tsm[r * N + l] - q * d * d - mx); }
-      if (S.lognu[y] + beta0[y] * ie0 + mx + log(acc) >= lthr) keep(k, l);
+      for (int r = 0; r < s; ++r) {
+        const float d = (float)(r0 + r - k);
+        acc += dd_ex2((fma(-q, widen_pos(d * d), tsm[r * N + l]) - mx) * DD_LOG2E);
+      }
+      if (S.lognu[y] + beta0[y] * ie0 + mx + dd_log(acc) >= lthr) keep(k, l);
     };
     const int nb = nband;
     if (nb <= kInitBand) {
@@ -796,8 +802,7 @@ k_init_duals(DevState S, const double* __restrict__ alpha0, const double* __rest
     // s exponentials per box point instead of s^2.
     // Exponentials and logarithms are the table-driven ones, shifts come from a
     // float maximum (any value near the maximum serves), and integer distances
-    // are widened on the integer pipe: about 16 FP64 operations a term (35 before;
-    // 1024^2, 7.7 M box points: 9 -> 4 ms).
+    // are widened on the integer pipe: about 16 FP64 operations a term (35 before).
     double* T1 = tsm;
     double* M2 = T1 + s * kInitChunk;
     double* MA = M2 + s * kInitChunk;

@@ -23,9 +23,10 @@ constexpr int kTileMinN = 192;   // smallest grid of the tile passes (few tiles 
 // instead of 12.  Only sources within 2^-65 of some target's shift are used
 // (maxima of blocks of 16, then a float test).  The powers cover
 // |n| <= D4 and 2^{+-400}, so that G stays a normal number for every term that
-// counts; a tile whose window is wider, and a target whose
-// sum leaves [2^-29, 2^59] of its float maximum, is summed term by term.  The rounding of a power's exponent (|2 q2 n| <= 400: below
-// 1e-13) is that of f - q2 d^2 itself at |f| ~ 1000.
+// counts; a tile whose window is wider, and a target whose sum leaves
+// [2^-29, 2^59] of its float maximum, is summed term by term.  The rounding of a
+// power's exponent (|2 q2 n| <= 400: below 1e-13) is that of f - q2 d^2 itself at
+// |f| ~ 1000.
 // MOM >= 1 also carries the mean of m - j under the terms, MOM == 2 that of mom(k, m):
 // one and two more multiply-adds a term.
 // out(j, L, mean1, mean2) is called once per target by consecutive threads.
