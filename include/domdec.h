@@ -104,7 +104,7 @@ typedef struct {
                           shared memory, one CTA for the others; 1 = one CTA per cell; 2, 4, 8 = every
                           cell whose box fits the cluster layout (or does with its per-y arrays in a
                           spill slot) on a cluster of that many CTAs.  With
-                          balance or cell_ti every cell runs on one CTA. */
+                          balance every cell runs on one CTA. */
   int    cell_ti;      /* 1: after each X-half of a cell solve, shift alpha by the t maximising the cell
                           dual along (alpha + t, beta - t) (closed form; not in the paper: it removes the
                           slow total-mass mode of the alternation when eps << lam, same fixed point);

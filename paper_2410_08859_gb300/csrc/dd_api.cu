@@ -581,7 +581,7 @@ int domdec_init(domdec_t* out, const double* mu, const double* nu, int N, const 
     return DOMDEC_EINVAL;
   }
   // clusters for the largest cells: automatic 4 CTAs (s <= 8) or 8 (larger cells);
-  // one CTA per cell with balancing or the translation step
+  // one CTA per cell with balancing
   {
     int C = pin->cell_ctas == 0 ? (h->s <= 8 ? 4 : 8) : pin->cell_ctas;
     // double cells are bound by the FP64 pipe of their SMs: where a sub-batch has
@@ -591,7 +591,7 @@ int domdec_init(domdec_t* out, const double* mu, const double* nu, int N, const 
       const bool stag = pin->strategy == DOMDEC_STAGGERED || pin->strategy == DOMDEC_STAGGERED_LINE;
       if ((stag ? ((nc + 1) / 2) * ((nc + 1) / 2) : nc * nc) * 8 <= 152) C = 8;
     }
-    if (pin->balance || pin->cell_ti) C = 1;
+    if (pin->balance) C = 1;
     h->order_mode = pin->cell_ctas == 0 ? 0 : 1;
     const size_t rs = pin->precision ? sizeof(double) : sizeof(float);
     size_t smem = cell_smem_bytes(h->s, cap_side, cap_ny, pin->precision);

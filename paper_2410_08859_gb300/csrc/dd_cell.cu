@@ -601,6 +601,12 @@ struct CellScalars {
     cA = R(-(1.0 - S.rr) * A);
     gA = R(-S.sl * A);          // -s A: the A part of -alpha/lam
   }
+  // translation step: alpha += t*, e^{t*/lam} = (a + sqrt(a^2 + 4 A_s B_s)) / (2 B_s) with A_s =
+  // <e^{-alpha/lam}, mu_J>, B_s = <e^{-beta/lam}, nu>, a = |nu_{-J}|; it moves A by t*/eps
+  __device__ __forceinline__ void translate(const DevState& S, double a0, double a, double As, double Bs) {
+    const double uu = (a + sqrt(a * a + 4.0 * As * Bs)) / (2.0 * Bs);
+    if (uu > 0.0 && uu < INFINITY) set_A(S, a0 + log(uu) / S.sl);
+  }
   __device__ __forceinline__ void set(const DevState& S, int D1, int D2, double a, double muJ) {
     qD2 = S.q * (double)(D1 * D1 + D2 * D2);
     q2 = R(S.q * DD_LOG2E); qR = R(S.q); sR = R(S.sl); rR = R(S.rr);
@@ -961,8 +967,7 @@ __device__ __forceinline__ void cell_solve_body(const DevState& S, const CellDes
           As += (double)apart[w];
           Bs += (double)bpart[w];
         }
-        const double uu = (a_tot + sqrt(a_tot * a_tot + 4.0 * As * Bs)) / (2.0 * Bs);
-        if (uu > 0.0 && uu < INFINITY) sk.set_A(S, A + log(uu) / sl);
+        sk.translate(S, A, a_tot, As, Bs);
       }
       __syncthreads();
       A = sk.A; sB = sk.sB; cA = sk.cA; gA = sk.gA;
@@ -1407,8 +1412,9 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
   // rho = max(0, P_Y - nu_J)/nu and log nu; the barycentre of nu_J (the Y frame
   // origin) is summed over the whole box from every CTA's part
   int c1, c2;
+  double a_tot = 0.0;   // |nu_{-J}| on B_J (translation step)
   {
-    double m3[3] = {0.0, 0.0, 0.0};
+    double m3[4] = {0.0, 0.0, 0.0, 0.0};
     for (int ul = tid; ul < nyl; ul += nthr) {
       const int kl = quot(ul, W, iW), ll = ul - kl * W, kk = kb + kl, v = kl * Wp + ll;
       const int y1 = k0 + kk, y2 = l0 + ll, y = y1 * N + y2;
@@ -1420,16 +1426,17 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
       lrho[v] = rho > R(0) ? dd_lg2(rho) * R(DD_LN2) : -dd_inf<R>();
       lnu[v] = R(S.lognu[y]);
       m3[0] += nuJ; m3[1] += nuJ * kk; m3[2] += nuJ * ll;
+      if (S.ti) m3[3] += num;
     }
-    cell_sum<R, 3>(m3, red);
+    cell_sum<R, 4>(m3, red);
     if (tid == 0)
       for (int r = 0; r < C; ++r) {
         double* px = cl.map_shared_rank(dx, r);
-        for (int k = 0; k < 3; ++k) px[crank * 16 + k] = m3[k];
+        for (int k = 0; k < 4; ++k) px[crank * 16 + k] = m3[k];
       }
     csync();
     double t0 = 0.0, t1 = 0.0, t2 = 0.0;
-    for (int r = 0; r < C; ++r) { t0 += dx[r * 16]; t1 += dx[r * 16 + 1]; t2 += dx[r * 16 + 2]; }
+    for (int r = 0; r < C; ++r) { t0 += dx[r * 16]; t1 += dx[r * 16 + 1]; t2 += dx[r * 16 + 2]; a_tot += dx[r * 16 + 3]; }
     c1 = H / 2; c2 = W / 2;
     if (t0 > 0.0) {
       c1 = min(H - 1, max(0, (int)lrint(t1 / t0)));
@@ -1455,9 +1462,10 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
   block_sum<2>(acc2, red);
   if (tid == 0) sk.set(S, D1, D2, acc2[0] / nx, acc2[1]);
   __syncthreads();
-  const double A = sk.A;
-  const R q2 = sk.q2, qR = sk.qR, sR = sk.sR, rR = sk.rR, sB = sk.sB, cEta1 = sk.cEta1, cEta2 = sk.cEta2, cA = sk.cA,
-          gA = sk.gA, cD1 = sk.cD1, cD2 = sk.cD2, tol = sk.tol;
+  double A = sk.A;
+  R sB = sk.sB, cA = sk.cA, gA = sk.gA;   // they move with A (translation step)
+  const R q2 = sk.q2, qR = sk.qR, sR = sk.sR, rR = sk.rR, cEta1 = sk.cEta1, cEta2 = sk.cEta2, cD1 = sk.cD1,
+          cD2 = sk.cD2, tol = sk.tol;
   for (int t = tid; t < nx; t += nthr) {
     const int r = quot(t, nx2, inx2), c = t - r * nx2;
     const int x = (cd.i0 + r) * N + cd.j0 + c;
@@ -1479,6 +1487,20 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
   (void)is;
   (void)i1s;
   int* pend = reinterpret_cast<int*>(red + 256);    // as in cell_solve_body
+  // translation step, as in cell_solve_body: nu e^{-beta/lam} of the own rows in the
+  // cell's buffer of new marginals, every CTA's sum in dx[16 rk + 4] of all CTAs.  It
+  // travels with the parts of W, so it adds no cluster barrier (such cells ran on one
+  // CTA before: 256 x 256, s = 8, largest box 11 583 points 1.94 -> 0.70 ms).
+  const bool ti = S.ti && sl > 0.0;
+  R* apart = reinterpret_cast<R*>(red) + 32;
+  R* bpart = apart + 32;
+  R* tib;
+  {
+    CellOut tmp;
+    tmp.slot = slot;
+    int st;
+    tib = reinterpret_cast<R*>(cell_nut(S, tmp, cidx, &st)) + kb * W;
+  }
   const int lock = sizeof(R) == 4 ? kLock : S.newton_maxit;
   int it = 0;
   R gap = R(0);
@@ -1498,11 +1520,12 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
     csync();
     // Y-half on the own rows: Z(kk, ll) = log2 sum_r 2^{T(r,ll) - q2 (r - kk - offr)^2}, Newton (a3)
     const bool fused_y = sizeof(R) == 4 && nyl * 2 > nthr;
-    auto y_store = [&](int v, R u, R Zx) {   // as in cell_solve_body
+    auto y_store = [&](int v, int y, R u, R Zx, R c0) {   // as in cell_solve_body
       const R b = fused_y ? u - Zx : fma(-Zx, LN2, u);
       Zv[v] = fused_y ? mul_rn(Zx, L2E) : Zx;
       bv[v] = b;
       bl[v] = (b + lnu[v]) * L2E;
+      if (ti) tib[y] = dd_ex2((lnu[v] - sR * u - c0) * L2E);
     };
     auto y_root = [&](int ll, int kl, int n, const auto& Z2) {
       constexpr int B = sizeof(Z2) / sizeof(R);
@@ -1537,7 +1560,7 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
           }
           root[k] = newton_rest(lr[k], c0[k], root[k], sR, S.newton_maxit - lock);
         }
-        y_store((kl + k) * Wp + ll, root[k], fused_y ? Zn[k] : Z2[k]);
+        y_store((kl + k) * Wp + ll, (kl + k) * W + ll, root[k], fused_y ? Zn[k] : Z2[k], c0[k]);
       }
     };
     if constexpr (sizeof(R) == 4) {
@@ -1550,7 +1573,7 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
         const R Zx = Zv[v], Zn = fused_y ? Zx : mul_rn(Zx, LN2);
         const R eta1 = R(k0 + kb + kl - yc1), eta2 = R(l0 + ll - yc2);
         const R c0 = sB - cEta1 * eta1 - cEta2 * eta2 - sR * Zn;
-        y_store(v, newton_rest(lrho[v], c0, bv[v], sR, S.newton_maxit - lock), Zx);
+        y_store(v, kl * W + ll, newton_rest(lrho[v], c0, bv[v], sR, S.newton_maxit - lock), Zx, c0);
       }
     } else {
       run_pass(T, 1, Wp, Zv, 1, Wp, W, Hl, nx1, offr + kb, q2, first, tid, nthr,
@@ -1562,7 +1585,19 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
         y_root(ll, kl, 1, z);
       }
     }
+    if (ti) {
+      __syncthreads();
+      R bsum = R(0);
+      for (int ul = tid; ul < nyl; ul += nthr) bsum += tib[ul];
+      bsum = warp_sum(bsum);
+      if ((tid & 31) == 0) bpart[tid >> 5] = bsum;
+    }
     __syncthreads();
+    if (ti && tid == 0) {
+      double bs = 0.0;
+      for (int w = 0; w < (nthr >> 5); ++w) bs += (double)bpart[w];
+      for (int rk = 0; rk < C; ++rk) cl.map_shared_rank(dx, rk)[crank * 16 + 4] = bs;
+    }
     // X-half on the own rows: U(kl, c) = log2 sum_ll 2^{bl(kl,ll) - q2 (ll - (c - offc))^2}
     run_pass(bl, Wp, 1, U, Up, 1, Hl, nx2, W, -offc, q2, first, tid, nthr, [&](int kl, int c, int n, const auto& v) {
       for (int k = 0; k < n; ++k) U[kl * Up + c + k] = v[k];
@@ -1584,7 +1619,7 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
     }
     csync();
     // combine the parts (rank order: every CTA gets the same W), gap terms (a4), next alpha (a2)
-    R gl = R(0);
+    R gl = R(0), asum = R(0);
     for (int t = tid; t < nx; t += nthr) {
       R mx = -dd_inf<R>();
       for (int rk = 0; rk < C; ++rk) mx = max(mx, Wx[rk * cap_nx + t]);
@@ -1604,18 +1639,33 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
       const R an = cA - rR * W2 * LN2 - cD1 * xi1 - cD2 * xi2;
       av_n[t] = an;
       xa_n[r * xp + c] = (an + lm[t]) * L2E;
+      if (ti) asum += dd_ex2((lm[t] + gA + g0[t] - sR * an) * L2E);   // mu e^{-alpha_new/lam}
     }
     {
       // every CTA adds the same values in the same order
       R* gpart = reinterpret_cast<R*>(red);
       gl = warp_sum(gl);
       if ((tid & 31) == 0) gpart[tid >> 5] = gl;
+      if (ti) {
+        asum = warp_sum(asum);
+        if ((tid & 31) == 0) apart[tid >> 5] = asum;
+      }
       __syncthreads();
       gap = R(0);
       for (int w = 0; w < (nthr >> 5); ++w) gap += gpart[w];
     }
     first = false;
     if ((stops && gap <= tol) || it >= S.maxit || !(gap == gap)) break;
+    if (ti) {   // every CTA the same step
+      if (tid == 0) {
+        double As = 0.0, Bs = 0.0;
+        for (int w = 0; w < (nthr >> 5); ++w) As += (double)apart[w];
+        for (int rk = 0; rk < C; ++rk) Bs += dx[rk * 16 + 4];
+        sk.translate(S, A, a_tot, As, Bs);
+      }
+      __syncthreads();
+      A = sk.A; sB = sk.sB; cA = sk.cA; gA = sk.gA;
+    }
     R* tp = av_c; av_c = av_n; av_n = tp;
     tp = xa_c; xa_c = xa_n; xa_n = tp;
   }

@@ -177,3 +177,25 @@ def test_boxes_beyond_shared_memory(env, ctas, precision="fp64", tol=1e-11):
     for k in range(2):
         assert np.abs(got[k] - ref[k]).sum() <= tol * np.abs(ref[k]).sum()
     assert np.abs(got[2] - ref[2]).max() <= tol * (1 + np.abs(ref[2]).max())
+
+
+@pytest.mark.parametrize("ctas", [2, 4, 8])
+@pytest.mark.parametrize("N,s", [(48, 4), (96, 8), (160, 16)])
+def test_translation_step_on_clusters(env, N, s, ctas):
+    """Cells with the translation step on a cluster against one CTA each, two sweeps (the
+    second with the ragged boundary cells) of a fixed number of iterations.  In double the sums
+    in another order differ by ~1e-16; t*/eps = log(u)/s amplifies that by 1/s (here up to 6.4e3)."""
+    torch, dd = env
+    mu, nu = inputs.mixture_blobs(N=N, seed=11)
+    eps = 4.0 / N ** 2
+    out = []
+    for c in (1, ctas):
+        with dd.DomDec(mu, nu, eps, 1.0, s, precision="fp64", cell_ctas=c, cell_ti=1, err=-1.0, maxit=4,
+                       strategy="safe", spill_slots=100) as g:
+            g.iterate(2)
+            g.sync()
+            out.append((*g.marginals(), g.duals()))
+    ref, got = out
+    for k in range(2):
+        assert np.abs(got[k] - ref[k]).sum() <= 1e-11 * np.abs(ref[k]).sum()
+    assert np.abs(got[2] - ref[2]).max() <= 1e-11 * (1 + np.abs(ref[2]).max())
