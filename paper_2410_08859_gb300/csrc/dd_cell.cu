@@ -1932,7 +1932,9 @@ __global__ void __launch_bounds__(1024) k_cell_order(DevState S, int part, int m
       const unsigned int cost = cell_cost(S, cells[begin + i], &H, &W);
       const bool fits_one = H <= S.cap_side && W <= S.cap_side && H * W <= S.cap_ny;
       const CellDesc& cd = cells[begin + i];
-      const bool fits_dist = fits_cluster(S, H, W, C) || (!fits_one && fits_hybrid(S, cd.nx1, cd.nx2, H, W, C));
+      // a box that a larger cluster holds without a slot is regrouped, not spilled
+      const bool fits_dist = fits_cluster(S, H, W, C) ||
+                             (!fits_one && !fits_layout(S, H, W) && fits_hybrid(S, cd.nx1, cd.nx2, H, W, C));
       const bool big = mode != 2 && fits_dist && (mode == 1 || !fits_one || (double)cost > thr);
       if (!fits_one && !big && fits_layout(S, H, W) && (mode == 2 || C < S.dist_c)) atomicOr(S.status, ST_REGROUP);
       k = ((unsigned long long)big << 62) | ((unsigned long long)cost << 30) | (0x3fffffffu - (unsigned)i);
@@ -2066,7 +2068,9 @@ k_ref_order(const DevState* __restrict__ states, const CellRef* __restrict__ ref
       const unsigned int cost = cell_cost(S, S.cells[part][rf.cell], &H, &W);
       const bool fits_one = H <= S.cap_side && W <= S.cap_side && H * W <= S.cap_ny;
       const CellDesc& cd = S.cells[part][rf.cell];
-      const bool fits_dist = fits_cluster(S, H, W, C) || (!fits_one && fits_hybrid(S, cd.nx1, cd.nx2, H, W, C));
+      // a box that a larger cluster holds without a slot is regrouped, not spilled
+      const bool fits_dist = fits_cluster(S, H, W, C) ||
+                             (!fits_one && !fits_layout(S, H, W) && fits_hybrid(S, cd.nx1, cd.nx2, H, W, C));
       const bool big = fits_dist && (!fits_one || (double)cost > thr);
       if (!fits_one && !big && fits_layout(S, H, W) && C < S.dist_c) atomicOr(S.status, ST_REGROUP);
       k = ((unsigned long long)big << 62) | ((unsigned long long)cost << 30) | (0x3fffffffu - (unsigned)i);

@@ -199,3 +199,19 @@ def test_translation_step_on_clusters(env, N, s, ctas):
     for k in range(2):
         assert np.abs(got[k] - ref[k]).sum() <= 1e-11 * np.abs(ref[k]).sum()
     assert np.abs(got[2] - ref[2]).max() <= 1e-11 * (1 + np.abs(ref[2]).max())
+
+
+def test_boxes_that_a_larger_cluster_holds_take_no_slot(env):
+    """176 x 176 boxes fit the shared memory of four CTAs but not of two: with a launch on two and a
+    single spill slot for many cells the sweep regroups to four."""
+    torch, dd = env
+    N, s = 176, 8
+    mu, nu = inputs.mixture_blobs(N=N, seed=12)
+    with dd.DomDec(mu, nu, 16.0 / N ** 2, 1.0, s, precision="fp32", err=-1.0, maxit=2, strategy="staggered",
+                   spill_slots=1) as g:
+        assert g.set_launch(2, 2.0) == 2
+        g.iterate(1)
+        g.sync()
+        assert g.stats()["cluster_regroups"] >= 1
+        PX, PY = g.marginals()
+    assert abs(PX.sum() - PY.sum()) <= 1e-5 * PX.sum()
