@@ -1653,6 +1653,9 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
       __syncthreads();
       gap = R(0);
       for (int w = 0; w < (nthr >> 5); ++w) gap += gpart[w];
+      // the epilogue's sums use the same scratch: no warp may get there while another still
+      // adds the parts (it would see another gap and miss the cluster's barriers)
+      __syncthreads();
     }
     first = false;
     if ((stops && gap <= tol) || it >= S.maxit || !(gap == gap)) break;
