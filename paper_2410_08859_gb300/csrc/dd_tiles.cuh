@@ -55,13 +55,15 @@ __device__ __forceinline__ void tile_rows(unsigned char* sm, const double* __res
     if (MOM == 2) momr[l] = mom[(long long)k * N + l];
   }
   for (int l = threadIdx.x; l < N + kTile; l += blockDim.x) qd[l] = make_double2(q2 * (double)l, (double)l);
+  const int na = D4 / 16 + 1;
   if (D4 <= 128) {
     for (int i = threadIdx.x; i < 2 * D4 + 1; i += blockDim.x) pw[i] = dd_ex2(2.0 * q2 * (double)(i - D4));
   } else {   // products of a coarse and a fine power (D4 <= 4095; 2 q2 (D4 + 32) < 1022)
-    const int na = D4 / 16 + 1;
     for (int i = threadIdx.x; i < 2 * na + 1; i += blockDim.x) pa[i] = dd_ex2(2.0 * q2 * (double)(16 * (i - na)));
     for (int i = threadIdx.x; i < 16; i += blockDim.x) pb[i] = dd_ex2(2.0 * q2 * (double)i);
-    __syncthreads();
+  }
+  __syncthreads();   // the line (block maxima) and the coarse and fine powers
+  if (D4 > 128) {
     for (int i = threadIdx.x; i < 2 * D4 + 1; i += blockDim.x) {
       const int n = i - D4 + 16 * na;                    // >= 0
       pw[i] = pa[n >> 4] * pb[n & 15];

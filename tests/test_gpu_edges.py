@@ -55,3 +55,53 @@ def test_stop_on_a_tolerance_on_clusters(env, N, s, ctas, precision):
             assert np.abs(got[k] - one[k]).sum() <= 1e-9 * np.abs(one[k]).sum()
     else:   # each side's P_X is within sqrt(2 gap |mu|) of its cells' limit (Pinsker), in both sweeps
         assert np.abs(got[1] - one[1]).sum() <= 4.0 * np.sqrt(2.0 * err) * mu.sum()
+
+
+# ------------------------------------------------------ adjoint at very small eps
+def lse(torch, f, q):
+    """log sum_y exp(f(y) - q |x - y|^2), f: N x N."""
+    N = f.shape[0]
+    t = torch.arange(N, device=f.device, dtype=torch.float64)
+    K = -q * (t[:, None] - t[None, :]) ** 2
+    for _ in range(2):
+        f = torch.cat([torch.logsumexp(f[i:i + 64, None, :] + K[None], 2) for i in range(0, N, 64)]).T
+    return f
+
+
+@pytest.mark.parametrize("N", [192, 259])
+@pytest.mark.parametrize("eps_px", [0.005, 0.1, 0.5, 0.9, 0.95])
+@pytest.mark.parametrize("rows", [0.0, 60.0])
+@pytest.mark.parametrize("half", ["x", "y"])
+def test_adjoint_windows_at_small_eps(env, N, eps_px, rows, half):
+    """The double tile passes below eps = 0.93 h^2, where the table of powers is short, at
+    potentials that jump by `rows` units of eps from row to row (every line's block maxima are
+    its own).  One potential is the closed-form half of the other, so the ratio P/w that the
+    gradient carries is e^{-pot/lam} in every pixel of that side."""
+    torch, dd = env
+    rng = np.random.default_rng(N)
+    eps = eps_px / N ** 2
+    lam = 500.0 * eps
+    mu, nu = (torch.from_numpy(np.ascontiguousarray(x)).cuda() for x in inputs.mixture_blobs(N=N, seed=12))
+    t = np.arange(N) / N
+    rough = torch.from_numpy(2.0 * eps * (np.sin(7 * t[:, None] + 2 * t[None, :]) + rng.normal(size=(N, N)))
+                             + eps * rows * rng.uniform(-1, 1, size=(N, 1))).cuda()
+    q, kap = 1.0 / (N * N * eps), eps / (1 + eps / lam)
+    if half == "y":
+        alpha = rough
+        beta = -kap * lse(torch, alpha / eps + mu.log(), q)
+    else:
+        beta = rough
+        alpha = -kap * lse(torch, beta / eps + nu.log(), q)
+    flat = [x.reshape(-1).contiguous() for x in (mu, nu, alpha, beta)]
+    g = [torch.empty(N * N, dtype=torch.float64, device="cuda") for _ in range(2)]
+    dd.domdec_uot_gradients(*flat, N, eps, lam, precision=dd.FP64, grad_mu=g[0], grad_nu=g[1])
+    ry = (beta / eps + lse(torch, alpha / eps + mu.log(), q)).exp()
+    rx = (alpha / eps + lse(torch, beta / eps + nu.log(), q)).exp()
+    # exponents of magnitude f = pot/eps: one rounding of them in each pass
+    tol = 1e-12 + 1e-15 * float(max(alpha.abs().max(), beta.abs().max())) / eps
+    if half == "y":
+        ref, r, got = eps * mu.sum() - eps * ry - lam * torch.expm1(-beta / lam), ry, g[1]
+    else:
+        ref, r, got = eps * nu.sum() - eps * rx - lam * torch.expm1(-alpha / lam), rx, g[0]
+    err = (got.view(N, N) - ref).abs()
+    assert float((err / (ref.abs() + eps * r + eps)).max()) <= tol
