@@ -217,6 +217,7 @@ __device__ __forceinline__ void tile_rows(unsigned char* sm, const double* __res
       }
     for (int o = 1; o < P; o <<= 1) bad |= __shfl_xor_sync(0xffffffffu, (int)bad, o) != 0;
     if (__any_sync(0xffffffffu, bad)) {
+      __syncwarp();   // lane 0 of a group replaces what the group's lanes have stored above
       // term by term against each target's maximum
       for (int e = 0; e < kTile; ++e) {
         const int j = min(j0 + e, N - 1);

@@ -105,3 +105,32 @@ def test_adjoint_windows_at_small_eps(env, N, eps_px, rows, half):
         ref, r, got = eps * nu.sum() - eps * rx - lam * torch.expm1(-alpha / lam), rx, g[0]
     err = (got.view(N, N) - ref).abs()
     assert float((err / (ref.abs() + eps * r + eps)).max()) <= tol
+
+
+@pytest.mark.parametrize("N", [200, 409])
+def test_adjoint_tiles_summed_term_by_term(env, N):
+    """Single pixels that stand 300 units of eps above their line: the sums of the tile's other
+    targets leave the accepted range and are repeated term by term, by one lane of the group for
+    all of its targets.  Equal in repeated calls and equal to plain torch."""
+    torch, dd = env
+    rng = np.random.default_rng(N)
+    eps = 4.0 / N ** 2
+    lam = 500.0 * eps
+    mu, nu = (torch.from_numpy(np.ascontiguousarray(x)).cuda() for x in inputs.mixture_blobs(N=N, seed=13))
+    a = eps * rng.normal(size=(N, N))
+    a[rng.integers(0, N, 40), rng.integers(0, N, 40)] += 300.0 * eps
+    a[rng.integers(0, N, 40), rng.integers(0, N, 40)] -= 300.0 * eps
+    alpha = torch.from_numpy(a).cuda()
+    q = 1.0 / (N * N * eps)
+    beta = -eps / (1 + eps / lam) * lse(torch, alpha / eps + mu.log(), q)
+    flat = [x.reshape(-1).contiguous() for x in (mu, nu, alpha, beta)]
+    out = []
+    for _ in range(3):
+        g = torch.empty(N * N, dtype=torch.float64, device="cuda")
+        dd.domdec_uot_gradients(*flat, N, eps, lam, precision=dd.FP64, grad_nu=g)
+        out.append(g.view(N, N))
+    assert torch.equal(out[0], out[1]) and torch.equal(out[0], out[2])
+    ry = (beta / eps + lse(torch, alpha / eps + mu.log(), q)).exp()
+    ref = eps * mu.sum() - eps * ry - lam * torch.expm1(-beta / lam)
+    tol = 1e-12 + 1e-15 * float(max(alpha.abs().max(), beta.abs().max())) / eps
+    assert float(((out[0] - ref).abs() / (ref.abs() + eps * ry + eps)).max()) <= tol
