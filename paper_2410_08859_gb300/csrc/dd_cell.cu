@@ -594,6 +594,7 @@ __device__ __forceinline__ void cell_sum(double (&v)[K], double* scratch) {
 template <typename R>
 struct CellScalars {
   double A, qD2;   // alpha/eps = A + a + 2 q D.xi; beta/eps = q|D|^2 - A + b - 2 q D.eta
+  double bound;    // err |mu_J|
   R q2, qR, sR, rR, sB, cEta1, cEta2, cA, gA, cD1, cD2, tol, is, i1s;
   __device__ __forceinline__ void set_A(const DevState& S, double a) {
     A = a;
@@ -615,9 +616,9 @@ struct CellScalars {
     // gap <= err |mu_J| in the working precision: the largest value not above the bound
     is = R(1) / sR;
     i1s = R(1) / (R(1) + sR);
-    const double t = S.err * muJ;
-    if constexpr (sizeof(R) == 4) tol = __double2float_rd(t);
-    else tol = t;
+    bound = S.err * muJ;
+    if constexpr (sizeof(R) == 4) tol = __double2float_rd(bound);
+    else tol = bound;
     set_A(S, a);
   }
 };
@@ -1305,6 +1306,7 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
   __shared__ BoxRec dbox[4];
   __shared__ int dgeo[8];
   __shared__ int npend;
+  __shared__ bool stop;
   __shared__ CellScalars<R> sk;
   __shared__ double dx[kDistMaxC * 16];                 // partial sums of every CTA of the cluster
   CellOut* out = S.cout + cidx;
@@ -1465,7 +1467,7 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
   double A = sk.A;
   R sB = sk.sB, cA = sk.cA, gA = sk.gA;   // they move with A (translation step)
   const R q2 = sk.q2, qR = sk.qR, sR = sk.sR, rR = sk.rR, cEta1 = sk.cEta1, cEta2 = sk.cEta2, cD1 = sk.cD1,
-          cD2 = sk.cD2, tol = sk.tol;
+          cD2 = sk.cD2;
   for (int t = tid; t < nx; t += nthr) {
     const int r = quot(t, nx2, inx2), c = t - r * nx2;
     const int x = (cd.i0 + r) * N + cd.j0 + c;
@@ -1482,7 +1484,6 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
 
   // ------------------------------------------------------- Sinkhorn loop
   const R LN2 = R(DD_LN2), L2E = R(DD_LOG2E);
-  const bool stops = S.err >= 0.0;
   const R is = sk.is, i1s = sk.i1s;   // 1/s, 1/(1 + s) (double cells)
   (void)is;
   (void)i1s;
@@ -1503,7 +1504,7 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
   }
   const int lock = sizeof(R) == 4 ? kLock : S.newton_maxit;
   int it = 0;
-  R gap = R(0);
+  double gap = 0.0;   // of thread 0
   bool first = true;
   R *xa_c = xa, *av_c = av, *xa_n = xa_nx, *av_n = av_nx;
   for (;;) {
@@ -1619,7 +1620,8 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
     }
     csync();
     // combine the parts (rank order: every CTA gets the same W), gap terms (a4), next alpha (a2)
-    R gl = R(0), asum = R(0);
+    double gl = 0.0;
+    R asum = R(0);
     for (int t = tid; t < nx; t += nthr) {
       R mx = -dd_inf<R>();
       for (int rk = 0; rk < C; ++rk) mx = max(mx, Wx[rk * cap_nx + t]);
@@ -1634,7 +1636,7 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
       const R a = av_c[t];
       const R tt = a + W2 * LN2;         // log(P_X pi / mu)
       const R g = gA + g0[t] - sR * a;   // -alpha/lam
-      gl += dd_ex2((lm[t] + g) * L2E) * dd_psi<R>(tt - g);
+      gl += (double)(dd_ex2((lm[t] + g) * L2E) * dd_psi<R>(tt - g));
       const R xi1 = R(cd.i0 + r - xc1), xi2 = R(cd.j0 + c - xc2);
       const R an = cA - rR * W2 * LN2 - cD1 * xi1 - cD2 * xi2;
       av_n[t] = an;
@@ -1642,23 +1644,28 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
       if (ti) asum += dd_ex2((lm[t] + gA + g0[t] - sR * an) * L2E);   // mu e^{-alpha_new/lam}
     }
     {
-      // every CTA adds the same values in the same order
-      R* gpart = reinterpret_cast<R*>(red);
-      gl = warp_sum(gl);
-      if ((tid & 31) == 0) gpart[tid >> 5] = gl;
+      // The gap in double, as its terms decide when a cell stops: every CTA adds the same
+      // values in the same order (the warps that hold any, then warp 0 over the warps), and one
+      // thread of each decides, so no two threads can disagree.  The parts lie clear of
+      // the scratch of the epilogue's first sum, which a warp may reach before another
+      // has read the decision.
+      double* gpart = red + 384;
+      const int nw = nthr >> 5, wid = tid >> 5, lane = tid & 31;
+      if (32 * wid < nx) gl = warp_sum(gl);
+      if (lane == 0) gpart[wid] = gl;
       if (ti) {
         asum = warp_sum(asum);
-        if ((tid & 31) == 0) apart[tid >> 5] = asum;
+        if (lane == 0) apart[wid] = asum;
       }
       __syncthreads();
-      gap = R(0);
-      for (int w = 0; w < (nthr >> 5); ++w) gap += gpart[w];
-      // the epilogue's sums use the same scratch: no warp may get there while another still
-      // adds the parts (it would see another gap and miss the cluster's barriers)
+      if (wid == 0) {
+        gap = warp_sum(lane < nw ? gpart[lane] : 0.0);
+        if (lane == 0) stop = (S.err >= 0.0 && gap <= sk.bound) || it >= S.maxit || !(gap == gap);
+      }
       __syncthreads();
     }
     first = false;
-    if ((stops && gap <= tol) || it >= S.maxit || !(gap == gap)) break;
+    if (stop) break;
     if (ti) {   // every CTA the same step
       if (tid == 0) {
         double As = 0.0, Bs = 0.0;
@@ -1672,7 +1679,6 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
     R* tp = av_c; av_c = av_n; av_n = tp;
     tp = xa_c; xa_c = xa_n; xa_n = tp;
   }
-  const bool nonfinite = !(gap == gap);
 
   // ------------------------------------------------------- epilogue (a5)
   const double th_s = 1.0 / nbatch;
@@ -1788,11 +1794,11 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
   CellOut o;
   o.k0 = k0; o.l0 = l0; o.H = H; o.W = W;
   o.iters = it;
-  o.status = nonfinite ? CELL_NONFINITE : (stops && gap > tol ? CELL_MAXIT : CELL_OK);
+  o.status = !(gap == gap) ? CELL_NONFINITE : (S.err >= 0.0 && gap > sk.bound ? CELL_MAXIT : CELL_OK);
   o.D1 = D1; o.D2 = D2;
   o.slot = slot;
   o.usec = (int)min((dd_global_ns() - t_start) / 1000ull, 2147483647ull);
-  o.gap = (double)gap;
+  o.gap = gap;
   o.dKX[0] = dk[0]; o.dKX[1] = dk[1];
   for (int q4 = 0; q4 < 4; ++q4) {
     const int bi = cd.mem[q4];
@@ -1801,7 +1807,7 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
     o.Ht[q4] = bi >= 0 ? hsd[q4] - hsd[8 + q4] + S.muinu[bi] : 0.0;
   }
   *out = o;   // the decision kernel adds the sub-batch's counters
-  if (nonfinite) atomicOr(S.status, ST_NONFINITE);
+  if (!(gap == gap)) atomicOr(S.status, ST_NONFINITE);
 }
 
 // One sub-batch, persistent grid over the resident CTAs in clusters of
