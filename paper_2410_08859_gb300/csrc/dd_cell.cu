@@ -580,10 +580,10 @@ __device__ __forceinline__ double box_value(const BoxRec& b, const double* arena
 
 }  // namespace
 
-// Block sums of a cell: doubles for the double cells, pairs of floats for the float ones.
+// Block sums of a cell (in double; the orders of the double cells' sums are those of block_sum).
 template <typename R, int K>
 __device__ __forceinline__ void cell_sum(double (&v)[K], double* scratch) {
-  if constexpr (sizeof(R) == 4) block_sum_ff<K>(v, scratch);
+  if constexpr (sizeof(R) == 4) block_sum_split<K>(v, scratch);
   else block_sum<K>(v, scratch);
 }
 

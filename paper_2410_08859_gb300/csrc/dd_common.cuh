@@ -329,28 +329,32 @@ __device__ __forceinline__ void block_sum_wide(double (&v)[K], double* sm, int n
   __syncthreads();
 }
 
-// block_sum of doubles carried as unevaluated sums of two floats through the warp
-// shuffles (TwoSum, Knuth): 48 bits of the running sum on the FP32 pipe, where
-// the double shuffles of 16 warps take 16 clocks an addition on the FP64 pipe
-// (12 values at the end of a cell: 27 k clocks before, 10 to 16 k now, with the wait
-// for the block's last warp).  For finite values within float range (smaller
-// than 2^-126: flushed).
+// block_sum of K doubles whose warp sums split the values over the lanes: at the
+// first steps a lane passes half of its values on and keeps the sums of the other
+// half, so K values take about K + 4 shuffled additions a warp where K warp sums take
+// 5 K (K = 12: 16 against 60; the FP64 pipe gives two lanes a clock, so 16 warps
+// of 60 additions are 15 k clocks).  Same precision: every addition is a double one.
+// scratch: 33 K doubles.
 template <int K>
-__device__ __forceinline__ void block_sum_ff(double (&v)[K], double* scratch) {
+__device__ __forceinline__ void block_sum_split(double (&v)[K], double* scratch) {
+  constexpr int KP = K > 16 ? 32 : K > 8 ? 16 : K > 4 ? 8 : K > 2 ? 4 : K;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+  double u[KP];
 #pragma unroll
-  for (int k = 0; k < K; ++k) {
-    float hi = (float)v[k], lo = (float)(v[k] - (double)hi);
+  for (int k = 0; k < KP; ++k) u[k] = k < K ? v[k] : 0.0;
+  int idx = 0, o = 1;   // the value that the lane ends with
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float h2 = __shfl_xor_sync(0xffffffffu, hi, o), l2 = __shfl_xor_sync(0xffffffffu, lo, o);
-      const float s = __fadd_rn(hi, h2), b = __fsub_rn(s, hi);
-      const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(h2, b));
-      lo = __fadd_rn(__fadd_rn(lo, l2), e);
-      hi = s;
+  for (int h = KP / 2; h > 0; h >>= 1, o <<= 1) {
+    const bool up = lane & o;
+    idx += up ? h : 0;
+#pragma unroll
+    for (int k = 0; k < h; ++k) {
+      const double give = up ? u[k] : u[k + h], keep = up ? u[k + h] : u[k];
+      u[k] = keep + __shfl_xor_sync(0xffffffffu, give, o);
     }
-    if (lane == 0) scratch[wid * K + k] = (double)hi + (double)lo;
   }
+  for (; o < 32; o <<= 1) u[0] += __shfl_xor_sync(0xffffffffu, u[0], o);
+  if (lane < KP && idx < K) scratch[wid * K + idx] = u[0];
   __syncthreads();
   for (int k = wid; k < K; k += nw) {
     double a = lane < nw ? scratch[lane * K + k] : 0.0;
