@@ -385,7 +385,7 @@ __device__ __forceinline__ double lse_lanes_f64(const double* row, int sm, int M
       float mx = -INFINITY;
       for (int m = part; m < M; m += P) {
         const float d = (float)(m - ctr);
-        mx = fmaxf(mx, fmaf(-q2f * d, d, narrow(row[m * sm])));
+        mx = fmaxf(mx, fmaf(-q2f * d, d, narrow_any(row[m * sm])));
       }
       for (int o = 1; o < P; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
       if (todo) shift = mx > -INFINITY ? (double)mx : 0.0;
@@ -395,7 +395,7 @@ __device__ __forceinline__ double lse_lanes_f64(const double* row, int sm, int M
     for (int m = part; m < M; m += P) {
       const float d = (float)(m - ctr);
       const double v = row[m * sm];
-      if (!(fmaf(-q2f * d, d, narrow(v)) - sf < -65.0f)) a += dd_ex2(fma(-q2, widen_pos(d * d), v) - shift);
+      if (!(fmaf(-q2f * d, d, narrow_any(v)) - sf < -65.0f)) a += dd_ex2(fma(-q2, widen_pos(d * d), v) - shift);
     }
     for (int o = 1; o < P; o <<= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
     if (todo) acc = a;

@@ -180,8 +180,8 @@ __device__ __forceinline__ double dd_rcp(double x) {
   return fma(fma(-x, r, 1.0), r, r);
 }
 
-// float(x) rounded to nearest and double(f) for positive normal f, on the integer
-// pipe: conversions to and from double share the two-lane FP64 path.
+// float(x) rounded to nearest, for finite |x| < 2^128 (what is below 2^-126 gives 0), on
+// the integer pipe: conversions to and from double share the two-lane FP64 path.
 __device__ __forceinline__ float narrow(double x) {
   const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
   if ((hi & 0x7fffffffu) < 0x38100000u) return 0.0f;   // below 2^-126
@@ -195,6 +195,8 @@ __device__ __forceinline__ float narrow_any(double x) {
   const unsigned a = (unsigned)__double2hiint(x) & 0x7fffffffu;
   return a - 0x38100000u < 0x47e00000u - 0x38100000u ? narrow(x) : (float)x;
 }
+// double(f) for positive normal f.  0 gives 2^-127, which changes no exponent that a
+// squared distance of 0 is multiplied into.
 __device__ __forceinline__ double widen_pos(float f) {
   const unsigned u = __float_as_uint(f);
   return __hiloint2double((int)((u >> 3) + 0x38000000u), (int)(u << 29));
