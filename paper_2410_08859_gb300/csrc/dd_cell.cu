@@ -372,9 +372,13 @@ __device__ __forceinline__ void run_pass(const float* src, int sl, int sm, const
 // ---- double passes: one target on a group of P lanes.  The FP64 pipe gives two
 // lanes a clock, so a term (12 operations) is evaluated only if a float test
 // finds it within 2^-65 of the target's shift (at eps = h^2: 13 of 32 sources);
-// narrowing and widening run on the integer pipe.  A sum below 2^-4 of its
-// shift, and a target without a previous value, is taken against the float
-// maximum, so what is left out is below 32 * 2^-61 = 2^-56 of the sum.
+// narrowing and widening run on the integer pipe.  The test allows for its own
+// rounding: a term that counts is formed from magnitudes below |source| + |shift| + 65,
+// so its float value errs by less than 4e-7 (|source| + |shift|) + 0.001.  A sum below 2^-4
+// of its shift, and a target without a previous value, is taken against its
+// maximum, so what is left out is below M 2^-61 of the sum.  The maximum is the float
+// one (any value near it serves) unless it or a source is beyond 1e6, where a float
+// one could be off by more than a unit (eps below about 1e-3 h^2).
 __device__ __forceinline__ double lse_lanes_f64(const double* row, int sm, int M, int ctr, double q2, double shift,
                                                 bool have, int part, int P) {
   const float q2f = (float)q2;
@@ -382,20 +386,35 @@ __device__ __forceinline__ double lse_lanes_f64(const double* row, int sm, int M
   bool todo = true;
   for (int pass = have ? 0 : 1; pass < 2; ++pass) {
     if (pass == 1) {
-      float mx = -INFINITY;
+      float mx = -INFINITY, big = 0.0f;
       for (int m = part; m < M; m += P) {
-        const float d = (float)(m - ctr);
-        mx = fmaxf(mx, fmaf(-q2f * d, d, narrow_any(row[m * sm])));
+        const float d = (float)(m - ctr), v = narrow_any(row[m * sm]);
+        mx = fmaxf(mx, fmaf(-q2f * d, d, v));
+        big = fmaxf(big, fabsf(v));
       }
-      for (int o = 1; o < P; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      if (todo) shift = mx > -INFINITY ? (double)mx : 0.0;
+      for (int o = 1; o < P; o <<= 1) {
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        big = fmaxf(big, __shfl_xor_sync(0xffffffffu, big, o));
+      }
+      double mxd = (double)mx;
+      if (__any_sync(0xffffffffu, big > 1e6f || (mx < -1e6f && mx > -INFINITY))) {
+        mxd = -INFINITY;
+        for (int m = part; m < M; m += P) {
+          const double d = (double)(m - ctr);
+          mxd = fmax(mxd, fma(-q2, d * d, row[m * sm]));
+        }
+        for (int o = 1; o < P; o <<= 1) mxd = fmax(mxd, __shfl_xor_sync(0xffffffffu, mxd, o));
+      }
+      if (todo) shift = mxd > -INFINITY ? mxd : 0.0;
     }
-    const float sf = (float)shift;
+    const float sf = (float)shift, lo = fmaf(-4e-7f, fabsf(sf), -65.001f);
     double a = 0.0;
     for (int m = part; m < M; m += P) {
       const float d = (float)(m - ctr);
       const double v = row[m * sm];
-      if (!(fmaf(-q2f * d, d, narrow_any(v)) - sf < -65.0f)) a += dd_ex2(fma(-q2, widen_pos(d * d), v) - shift);
+      const float vf = narrow_any(v);
+      if (!(fmaf(-q2f * d, d, vf) - sf < fmaf(-4e-7f, fabsf(vf), lo)))
+        a += dd_ex2(fma(-q2, widen_pos(d * d), v) - shift);
     }
     for (int o = 1; o < P; o <<= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
     if (todo) acc = a;

@@ -199,3 +199,21 @@ def test_lse_of_double_cells_with_special_sources(env):
         f[9] = np.nan
         for prev in (None, np.full(32, base), np.full(32, np.nan)):
             assert np.isnan(lse_dev(env, f, 1.0, 32, 4, prev)).all()
+
+
+@pytest.mark.parametrize("M", [1, 7, 32, 200])
+@pytest.mark.parametrize("P", [1, 4, 32])
+@pytest.mark.parametrize("q2", [1e-3, 1.0, 1e4, 1e8, 1e11])
+def test_lse_of_double_cells(env, M, P, q2):
+    """Sources from moderate to far larger than a float resolves (eps down to 1e-11 h^2), without a
+    previous value, with the value itself, with one that is off by up to 40, and with a useless one.
+    Each exponent carries two roundings of the magnitudes it is formed from."""
+    rng = np.random.default_rng(M + P)
+    n = 45
+    for scale in (1.0, 100.0, 5.0 * q2):
+        f = scale * rng.normal(size=M)
+        ref, _ = lse_ref(f, q2, n)
+        tol = 4 * 2.0 ** -53 * (np.abs(f).max() + np.abs(ref) + 70) + 1e-15
+        for prev in (None, ref, ref + rng.uniform(-40, 40, n), ref + 1e4, np.full(n, -np.inf), np.full(n, np.nan)):
+            got = lse_dev(env, f, q2, n, P, prev)
+            assert (np.abs(got - ref) <= tol).all(), (scale, np.abs(got - ref).max())
