@@ -607,6 +607,16 @@ __global__ void __launch_bounds__(256) k_tile_max(const float* __restrict__ g, i
 //         took 46 ms (both modes; 17 with tiles and tables, 14 with the table
 //         functions in the double part of the test too);
 // mode 1: values on the box (dense over X_i), C_i, H_i, P_Y.
+// A shift for the exponentials of n terms: their float maximum mxf, formed of values of
+// magnitude at most `big`, unless those exceed 1e8 -- beyond (potentials above 1e8 eps0) its
+// rounding could leave the exponentials' range, and the maximum is taken in double.
+template <typename F>
+__device__ __forceinline__ double init_shift(float mxf, float big, int n, F term) {
+  if (fmaxf(fabsf(mxf), big) < 1e8f) return (double)mxf;
+  double mx = -INFINITY;
+  for (int k = 0; k < n; ++k) mx = fmax(mx, term(k));
+  return mx;
+}
 constexpr int kInitChunk = 128;   // box columns per pass of the dual-initialised fill
 constexpr int kInitBand = 2048;   // band pixels listed per basic cell by the box test
 __global__ void __launch_bounds__(1024)
@@ -730,30 +740,35 @@ k_init_duals(DevState S, const double* __restrict__ alpha0, const double* __rest
     for (int t = threadIdx.x; t < s * N; t += blockDim.x) {
       const int r = t / N, l = t - (t / N) * N;
       if (!colflag[l]) continue;
-      const double mx = (double)tsmf[t];   // the float value is a good enough shift
-      double acc = 0.0;
-      for (int c = 0; c < s; ++c) {
+      float big = 0.0f;
+      for (int c = 0; c < s; ++c) big = fmaxf(big, fabsf(xvf[r * s + c]));
+      auto term = [&](int c) {
         const int x = (r0 + r) * N + c0 + c;
         const float d = (float)(c0 + c - l);
-        acc += dd_ex2((fma(-q, widen_pos(d * d), alpha0[x] * ie0 + S.logmu[x]) - mx) * DD_LOG2E);
-      }
+        return fma(-q, widen_pos(d * d), alpha0[x] * ie0 + S.logmu[x]);
+      };
+      const double mx = init_shift(tsmf[t], big, s, term);
+      double acc = 0.0;
+      for (int c = 0; c < s; ++c) acc += dd_ex2((term(c) - mx) * DD_LOG2E);
       tsm[t] = mx + dd_log(acc);
     }
     __syncthreads();
     // the double test of the band pixels (rescanning all pixels if the list overflowed)
     auto dtest = [&](int y) {
       const int k = y / N, l = y - (y / N) * N;
-      float mxf = -INFINITY;
+      float mxf = -INFINITY, big = 0.0f;
       for (int r = 0; r < s; ++r) {
-        const float d = (float)(r0 + r - k);
-        mxf = fmaxf(mxf, tsmf[r * N + l] - qf * d * d);
+        const float d = (float)(r0 + r - k), v = tsmf[r * N + l];
+        mxf = fmaxf(mxf, v - qf * d * d);
+        big = fmaxf(big, fabsf(v));
       }
-      const double mx = (double)mxf;
+      auto term = [&](int r) {
+        const float d = (float)(r0 + r - k);
+        return fma(-q, widen_pos(d * d), tsm[r * N + l]);
+      };
+      const double mx = init_shift(mxf, big, s, term);
       double acc = 0.0;
-      for (int r = 0; r < s; ++r) {
-        const float d = (float)(r0 + r - k);
-        acc += dd_ex2((fma(-q, widen_pos(d * d), tsm[r * N + l]) - mx) * DD_LOG2E);
-      }
+      for (int r = 0; r < s; ++r) acc += dd_ex2((term(r) - mx) * DD_LOG2E);
       if (S.lognu[y] + beta0[y] * ie0 + mx + dd_log(acc) >= lthr) keep(k, l);
     };
     const int nb = nband;
@@ -825,12 +840,16 @@ k_init_duals(DevState S, const double* __restrict__ alpha0, const double* __rest
       const int wc = min(kInitChunk, b.W - lc);
       for (int t = threadIdx.x; t < s * wc; t += blockDim.x) {
         const int r = t / wc, lj = t - r * wc, l = b.l0 + lc + lj;
-        float mxf = -INFINITY;
+        float mxf = -INFINITY, big = 0.0f;
         for (int c = 0; c < s; ++c) {
-          const float d = (float)(c0 + c - l);
-          mxf = fmaxf(mxf, xaf[r * s + c] - qf * d * d);
+          const float d = (float)(c0 + c - l), x = xaf[r * s + c];
+          mxf = fmaxf(mxf, x - qf * d * d);
+          big = fmaxf(big, fabsf(x));
         }
-        const double mx = (double)mxf;
+        const double mx = init_shift(mxf, big, s, [&](int c) {
+          const double d = (double)(c0 + c - l);
+          return fma(-q, d * d, xa[r * s + c]);
+        });
         double a = 0.0, a2 = 0.0, aa = 0.0;
         for (int c = 0; c < s; ++c) {
           const float d = (float)(c0 + c - l);
@@ -848,12 +867,16 @@ k_init_duals(DevState S, const double* __restrict__ alpha0, const double* __rest
       for (int u = threadIdx.x; u < b.H * wc; u += blockDim.x) {
         const int kk = u / wc, lj = u - kk * wc;
         const int k = b.k0 + kk, l = b.l0 + lc + lj, y = k * N + l;
-        float mxf = -INFINITY;
+        float mxf = -INFINITY, big = 0.0f;
         for (int r = 0; r < s; ++r) {
-          const float d = (float)(r0 + r - k);
-          mxf = fmaxf(mxf, T1f[r * kInitChunk + lj] - qf * d * d);
+          const float d = (float)(r0 + r - k), t1 = T1f[r * kInitChunk + lj];
+          mxf = fmaxf(mxf, t1 - qf * d * d);
+          big = fmaxf(big, fabsf(t1));
         }
-        const double mx = (double)mxf;
+        const double mx = init_shift(mxf, big, s, [&](int r) {
+          const double d = (double)(r0 + r - k);
+          return fma(-q, d * d, T1[r * kInitChunk + lj]);
+        });
         double a = 0.0, ac = 0.0, aa = 0.0;
         for (int r = 0; r < s; ++r) {
           const float d = (float)(r0 + r - k);

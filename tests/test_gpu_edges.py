@@ -131,3 +131,23 @@ def test_adjoint_tiles_summed_term_by_term(env, N):
     ref = eps * mu.sum() - eps * ry - lam * torch.expm1(-beta / lam)
     tol = 1e-12 + 1e-15 * float(max(alpha.abs().max(), beta.abs().max())) / eps
     assert float(((out[0] - ref).abs() / (ref.abs() + eps * ry + eps)).max()) <= tol
+
+
+# ------------------------------------------------------ potentials of any magnitude
+@pytest.mark.parametrize("shift", [1e3, 2e10])
+def test_dual_initialised_plan_of_shifted_potentials(env, shift):
+    """alpha0 + K, beta0 - K is the same plan for every K; K = shift eps costs it the roundings of
+    exponents of that size (two in each of the sums over rows and columns)."""
+    torch, dd = env
+    N, s = 24, 3
+    mu, nu = inputs.mixture_blobs(N=N, seed=9)
+    eps = 1.5 / N ** 2
+    a, b = np.empty((N, N)), np.empty((N, N))
+    dd.domdec_full_sinkhorn(mu, nu, N, 2 * eps, 1.0, eps_start=1.0, maxit=20, err=-1.0, alpha=a, beta=b)
+    out = []
+    for k in (0.0, shift * 2 * eps):
+        with dd.DomDec(mu, nu, eps, 1.0, s, alpha0=a + k, beta0=b - k, eps_init=2 * eps, precision="fp64") as g:
+            out.append((*g.marginals(), g.basic_costs()[0]))
+    tol = 8 * 2.0 ** -52 * shift + 1e-12
+    for ref, got in zip(*out):
+        assert np.abs(got - ref).sum() <= tol * np.abs(ref).sum()
