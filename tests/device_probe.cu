@@ -18,6 +18,11 @@ __global__ void k_unary(int kind, const double* x, double* y, int n) {
   }
 }
 
+__global__ void k_binary(int kind, const double* a, const double* b, double* y, int n) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) y[i] = kind == 0 ? dd_log_quotient(a[i], b[i]) : dd_div(a[i], b[i]);
+}
+
 __global__ void k_newton(const double* lr, const double* c0, const double* uw, double s, int maxit, double* u, int n) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) u[i] = newton_f64(lr[i], c0[i], uw[i], s, 1.0 / s, 1.0 / (1.0 + s), maxit);
@@ -51,6 +56,10 @@ int done() { return cudaGetLastError() != cudaSuccess || cudaDeviceSynchronize()
 extern "C" {
 int probe_unary(int kind, const double* x, double* y, int n) {
   k_unary<<<(n + 255) / 256, 256>>>(kind, x, y, n);
+  return done();
+}
+int probe_binary(int kind, const double* a, const double* b, double* y, int n) {
+  k_binary<<<(n + 255) / 256, 256>>>(kind, a, b, y, n);
   return done();
 }
 int probe_newton(const double* lr, const double* c0, const double* uw, double s, int maxit, double* u, int n) {

@@ -124,6 +124,41 @@ def test_conversions(env):
     assert unary(env, 5, np.zeros(1))[0] == 2.0 ** -127
 
 
+# ------------------------------------------- logarithm of a quotient (the line search)
+def test_log_of_a_quotient(env):
+    """Half a unit in the last place of the result and two roundings of a table value (6e-17); next to
+    a = b, where there is no table value, three units and the correction's 2^-44 x 2^-23."""
+    torch, lib = env
+    rng = np.random.default_rng(4)
+    n = 100000
+
+    def run(kind, a, b):
+        y = torch.empty(a.size, dtype=torch.float64, device="cuda")
+        assert lib.probe_binary(kind, ptr(dev(torch, a)), ptr(dev(torch, b)), ptr(y), a.size) == 0
+        return y.cpu().numpy()
+
+    for ratio in (1 + rng.choice([-1, 1], n) * 10 ** rng.uniform(-12, -1, n), rng.uniform(0.5, 2, n),
+                  10 ** rng.uniform(-6, 6, n), 10 ** rng.uniform(-25, 20, n)):
+        b = 10 ** rng.uniform(-9, -3, n)
+        a = b * ratio
+        A, B = a.astype(np.longdouble), b.astype(np.longdouble)
+        ref = np.log1p((A - B) / B)
+        size = np.abs(ref).astype(np.float64)
+        tol = np.where(size > 1 / 257, 0.55 * np.spacing(size) + 6e-17, 3 * np.spacing(size) + 2e-20)
+        assert float((np.abs(run(0, a, b) - ref) / tol).max()) <= 1.0
+        d = (a - b) ** 2
+        q = d.astype(np.longdouble) / A
+        assert (np.abs(run(1, d, a) - q) <= 0.5001 * np.spacing(q.astype(np.float64))).all()
+    # outside the fast path's range: as CUDA's
+    a = np.array([1e-300, 1e-300, 1e300, 1e-40, 3.0, np.inf, np.nan])
+    b = np.array([1e-5, 1e-200, 1e-5, 1e-310, 1e-310, 1e-3, 1.0])
+    with np.errstate(over="ignore"):
+        ref = np.log(a / b)
+    got = run(0, a, b)
+    assert np.allclose(got, ref, rtol=4e-16, atol=0, equal_nan=True)
+    assert np.array_equal(run(1, np.array([0.0, 1e-320, 1e300]), np.array([2.0, 1e-5, 1e-60])), [0.0, 1e-320 / 1e-5, np.inf])
+
+
 # --------------------------------------------------------- the root of a double cell
 @pytest.mark.parametrize("s", [1e-6, 1e-3, 0.3, 20.0])
 @pytest.mark.parametrize("scale", [1.0, 30.0, 1e4, 1e8])
