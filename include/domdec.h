@@ -99,7 +99,7 @@ typedef struct {
                           thread-block cluster, its Y box split by rows over the CTAs (each CTA holds its
                           rows' Y-side arrays; the X-half log-sum-exp is combined from per-CTA parts).
                           0 = automatic: clusters of 4 CTAs (s <= 8), 8 (s > 8, and FP64 when a
-                          sub-batch's clusters of 8 all fit the GPU at once) for the cells whose
+                          sub-batch has at most one cell per 8 SMs) for the cells whose
                           work exceeds twice the mean work per CTA or whose box exceeds one CTA's
                           shared memory, one CTA for the others; 1 = one CTA per cell; 2, 4, 8 = every
                           cell whose box fits the cluster layout (or does with its per-y arrays in a

@@ -560,8 +560,9 @@ int domdec_init(domdec_t* out, const double* mu, const double* nu, int N, const 
   S.margin = pin->box_margin;
   set_eps_scalars(S, pin->eps);
   // shared-memory capacity of the cell kernel
-  int dev = 0, smem_optin = 0;
+  int dev = 0, smem_optin = 0, nsm = 0;
   cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   // dynamic shared memory left beside the kernels' static shared memory
   const int smem_budget = smem_optin - cell_static_smem(pin->precision) - 64;
@@ -584,12 +585,16 @@ int domdec_init(domdec_t* out, const double* mu, const double* nu, int N, const 
   // one CTA per cell with balancing
   {
     int C = pin->cell_ctas == 0 ? (h->s <= 8 ? 4 : 8) : pin->cell_ctas;
-    // double cells are bound by the FP64 pipe of their SMs: where a sub-batch has
-    // too few of them to fill the GPU with clusters of four, clusters of eight
+    // Double cells are bound by the FP64 pipe of their SMs: clusters of eight while a
+    // sub-batch has at most one cell per eight SMs (19).  They need not all be resident
+    // at once (15 are): only the cells above the split threshold take a cluster, the
+    // others run on the SMs that the clusters leave.  Two sweeps of 60 iterations, product plan,
+    // eight against four: 9 cells (N = 32, s = 4) 19.5 | 24.3 ms, 16 cells (N = 48, s = 4) 27.8 | 43.2,
+    // (96, 8) 108 | 177; 25 cells (64, 4) 63.5 | 57.0, (32, 2) 31.9 | 20.6; 36 cells (80, 4) 97.9 | 83.6.
     if (pin->cell_ctas == 0 && pin->precision) {
       const int nc = N / (2 * h->s) + 1;
       const bool stag = pin->strategy == DOMDEC_STAGGERED || pin->strategy == DOMDEC_STAGGERED_LINE;
-      if ((stag ? ((nc + 1) / 2) * ((nc + 1) / 2) : nc * nc) * 8 <= 152) C = 8;
+      if ((stag ? ((nc + 1) / 2) * ((nc + 1) / 2) : nc * nc) * 8 <= nsm) C = 8;
     }
     if (pin->balance) C = 1;
     h->order_mode = pin->cell_ctas == 0 ? 0 : 1;

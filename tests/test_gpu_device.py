@@ -252,3 +252,21 @@ def test_lse_of_double_cells(env, M, P, q2):
         for prev in (None, ref, ref + rng.uniform(-40, 40, n), ref + 1e4, np.full(n, -np.inf), np.full(n, np.nan)):
             got = lse_dev(env, f, q2, n, P, prev)
             assert (np.abs(got - ref) <= tol).all(), (scale, np.abs(got - ref).max())
+
+
+# ------------------------------------------------------- cluster size of double cells
+@pytest.mark.parametrize("N", [12, 20, 28, 32, 40, 48])
+@pytest.mark.parametrize("strategy", ["staggered", "safe"])
+def test_clusters_of_eight_for_few_double_cells(env, N, strategy):
+    """Clusters of eight while the largest sub-batch has at most one cell per eight SMs."""
+    torch, _ = env
+    from paper_2410_08859_gb300 import domdec as dd
+    from paper_2410_08859_gb300 import inputs
+    s, nc = 2, N // 4 + 1
+    cells = ((nc + 1) // 2) ** 2 if strategy == "staggered" else nc ** 2
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    mu, nu = inputs.mixture_small(N=N, seed=5)
+    with dd.DomDec(mu, nu, 1.0 / N ** 2, 1.0, s, precision="fp64", strategy=strategy) as g:
+        got = g.set_launch(8, 2.0)
+    # a layout that a box of few rows cannot use falls back to smaller clusters
+    assert got == (8 if 8 * cells <= sms else 1) or (got == 1 and N < 16)
