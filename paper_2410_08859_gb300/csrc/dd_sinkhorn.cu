@@ -57,11 +57,10 @@ constexpr int kSepBlock = 16;   // sources per block maximum
 // then run over nearly the same window, where a test of every source held all of
 // them for any one's term; the products q2 d come from a table and the
 // logarithms are taken by full warps at the end.  Measured, before -> now:
-// 256 x 256 FAST at eps = 8 h^2 71 -> 33 us, 32 h^2 103 -> 47; float 12.5 -> 9.5 (128 h^2) and
-// 12.7 -> 14.8 (8192 h^2: every source kept); 1024 x 1024 FAST 802 -> 317 (2 h^2), float
+// 256 x 256 FAST at eps = 8 h^2 71 -> 33 us, 32 h^2 103 -> 47; float 12.5 -> 9.5 (128 h^2); 1024 x 1024 FAST 802 -> 317 (2 h^2), float
 // 542 -> 127 (128 h^2); 64 x 64 double 27 -> 12 (the rows split over several CTAs
-// to reach all SMs).
-template <typename R, bool FAST>
+// to reach all SMs).  WIDE: no windows, every source tested (see sep_pass).
+template <typename R, bool FAST, bool WIDE>
 __global__ void __launch_bounds__(1024)
 k_sep_rows_t(const R* __restrict__ src, const float* __restrict__ srcf, R* dst, float* __restrict__ dstf, int N,
              double q2, int shifted, int per, SepHalf<R> half) {
@@ -83,12 +82,14 @@ k_sep_rows_t(const R* __restrict__ src, const float* __restrict__ srcf, R* dst, 
     }
   }
   __syncthreads();
-  for (int b = threadIdx.x; b < nb; b += blockDim.x) {
-    float m = -INFINITY;
-    for (int l = b * kSepBlock; l < min(N, (b + 1) * kSepBlock); ++l) m = fmaxf(m, rowf[l]);
-    bm[b] = m;
+  if (!WIDE) {
+    for (int b = threadIdx.x; b < nb; b += blockDim.x) {
+      float m = -INFINITY;
+      for (int l = b * kSepBlock; l < min(N, (b + 1) * kSepBlock); ++l) m = fmaxf(m, rowf[l]);
+      bm[b] = m;
+    }
+    __syncthreads();
   }
-  __syncthreads();
   const float q2f = (float)q2, cutf = (float)cut_log2<R>() + 1.0f;
   const int P = kSepLanes, part = threadIdx.x & (P - 1), nt = (j_n * P + 31) & ~31;
   // upper bound of the terms of block b at target j (a few ulp are added for the rounding)
@@ -116,21 +117,25 @@ k_sep_rows_t(const R* __restrict__ src, const float* __restrict__ srcf, R* dst, 
         // the maximum, from the block with the largest bound and those that can exceed it
         const bool again = !todo;
         float ub = -INFINITY, mx = -INFINITY;
-        int best = 0;
-        for (int b = part; b < nb; b += P) {
-          const float u = bound(b, j);
-          if (u > ub) { ub = u; best = b; }
+        if (WIDE) {
+          for (int m = part; m < N; m += P) mx = fmaxf(mx, term_f(m, j));
+        } else {
+          int best = 0;
+          for (int b = part; b < nb; b += P) {
+            const float u = bound(b, j);
+            if (u > ub) { ub = u; best = b; }
+          }
+          for (int o = 1; o < P; o <<= 1) {
+            const float u = __shfl_xor_sync(0xffffffffu, ub, o);
+            const int b = __shfl_xor_sync(0xffffffffu, best, o);
+            if (u > ub || (u == ub && b < best)) { ub = u; best = b; }
+          }
+          for (int m = best * kSepBlock + part; m < min(N, (best + 1) * kSepBlock); m += P) mx = fmaxf(mx, term_f(m, j));
+          for (int o = 1; o < P; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+          for (int b = part; b < nb; b += P)
+            if (bound(b, j) >= mx)
+              for (int m = b * kSepBlock; m < min(N, (b + 1) * kSepBlock); ++m) mx = fmaxf(mx, term_f(m, j));
         }
-        for (int o = 1; o < P; o <<= 1) {
-          const float u = __shfl_xor_sync(0xffffffffu, ub, o);
-          const int b = __shfl_xor_sync(0xffffffffu, best, o);
-          if (u > ub || (u == ub && b < best)) { ub = u; best = b; }
-        }
-        for (int m = best * kSepBlock + part; m < min(N, (best + 1) * kSepBlock); m += P) mx = fmaxf(mx, term_f(m, j));
-        for (int o = 1; o < P; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        for (int b = part; b < nb; b += P)
-          if (bound(b, j) >= mx)
-            for (int m = b * kSepBlock; m < min(N, (b + 1) * kSepBlock); ++m) mx = fmaxf(mx, term_f(m, j));
         for (int o = 1; o < P; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         if (again) {
           sigf = mx;
@@ -143,15 +148,19 @@ k_sep_rows_t(const R* __restrict__ src, const float* __restrict__ srcf, R* dst, 
       }
       // the window: from the first to the last block that can hold a kept term
       int lo = N, hi = 0;
-      if (todo)
-        for (int b = part; b < nb; b += P)
-          if (bound(b, j) - sigf > -cutf - 1.0f) {
-            lo = min(lo, b * kSepBlock);
-            hi = max(hi, min(N, (b + 1) * kSepBlock));
-          }
-      for (int o = 1; o < P; o <<= 1) {
-        lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-        hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+      if (WIDE) {
+        if (todo) { lo = 0; hi = N; }
+      } else {
+        if (todo)
+          for (int b = part; b < nb; b += P)
+            if (bound(b, j) - sigf > -cutf - 1.0f) {
+              lo = min(lo, b * kSepBlock);
+              hi = max(hi, min(N, (b + 1) * kSepBlock));
+            }
+        for (int o = 1; o < P; o <<= 1) {
+          lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+          hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+        }
       }
       bool over = false;
       R a = R(0);
@@ -355,11 +364,18 @@ cudaError_t sep_pass(const R* in, const float* inf, R* out, float* outf, int N, 
   const int per = (N + gy - 1) / gy, thr = std::min(1024, ((per * kSepLanes + 31) / 32) * 32);
   const int nb = (N + kSepBlock - 1) / kSepBlock;
   const size_t sm = sizeof(R) * ((size_t)N + 2 * (size_t)per + 1) + (sizeof(R) == 8 ? 20 * (size_t)N : 0) + 4 * (size_t)nb + 16;
+  // Where the distances alone leave no term out (q2 (N - 1)^2 within the cut and a moderate
+  // range of the sources) the windows are whole rows, and looking for them only costs: float,
+  // us a pass with all its kernels, windows | without: N = 256 at q2 (N - 1)^2 = 11 16.4 | 14.4,
+  // 46 16.0 | 14.4, 183 13.5 | 14.4, 1466 10.7 | 14.4; N = 1024 at 46 518 | 493, 184 369 | 491;
+  // N = 64 at 11 4.9 | 4.1; double N = 64 at 45 14.4 | 13.3, N = 256 at 46 467 | 467.
+  const bool wide = q2 * (double)(N - 1) * (double)(N - 1) <= 64.0;
+  auto kernel = wide ? k_sep_rows_t<R, FAST, true> : k_sep_rows_t<R, FAST, false>;
   if (sm > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(k_sep_rows_t<R, FAST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
   }
-  k_sep_rows_t<R, FAST><<<dim3(N, (N + per - 1) / per), thr, sm, st>>>(in, inf, out, outf, N, q2, shifted, per, half);
+  kernel<<<dim3(N, (N + per - 1) / per), thr, sm, st>>>(in, inf, out, outf, N, q2, shifted, per, half);
   return cudaGetLastError();
 }
 

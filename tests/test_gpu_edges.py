@@ -151,3 +151,32 @@ def test_dual_initialised_plan_of_shifted_potentials(env, shift):
     tol = 8 * 2.0 ** -52 * shift + 1e-12
     for ref, got in zip(*out):
         assert np.abs(got - ref).sum() <= tol * np.abs(ref).sum()
+
+
+# --------------------------------------------- separable passes with and without windows
+@pytest.mark.parametrize("N", [16, 31, 200])
+@pytest.mark.parametrize("reach", [5.0, 63.9, 64.1, 300.0])
+@pytest.mark.parametrize("precision,tol", [(0, 5e-6), (1, 1e-12)])
+def test_separable_passes_around_whole_rows(env, N, reach, precision, tol):
+    """q2 (N - 1)^2 on both sides of 64, where the search for windows starts; beta = 0, and in double
+    also a start whose exponents range over 200 (a potential is within one rounding of its
+    exponents a pass; single precision accepts a previous value that the sum has left by up to
+    2^30 as its shift, so its first iterations after such a start are coarse)."""
+    torch, dd = env
+    q2 = reach / (N - 1) ** 2
+    q = q2 * np.log(2.0)
+    eps, lam = 1.0 / (N * N * q), 0.8
+    mu, nu = (torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in inputs.mixture_blobs(N=N, seed=7))
+    t = torch.arange(N, device="cuda", dtype=torch.float64) / N
+    for start in (None, eps * 200.0 * (t[:, None] * t[None, :] - 0.5).contiguous())[:1 + precision]:
+        a, b = torch.empty_like(mu), torch.empty_like(mu)
+        dd.domdec_full_sinkhorn(mu, nu, N, eps, lam, eps_start=eps, precision=precision, maxit=3, err=-1.0,
+                                check_every=2, beta_in=start, alpha=a, beta=b)
+        kap = eps / (1 + eps / lam)
+        beta = torch.zeros_like(mu) if start is None else start
+        for _ in range(3):
+            alpha = -kap * lse(torch, beta / eps + nu.log(), q)
+            beta = -kap * lse(torch, alpha / eps + mu.log(), q)
+        for got, ref in ((a, alpha), (b, beta)):
+            scale = float(ref.abs().max()) + (0.0 if start is None else float(start.abs().max()))
+            assert float((got - ref).abs().max()) <= tol * (scale + eps)
