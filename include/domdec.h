@@ -329,7 +329,8 @@ const char* domdec_error_string(int code);
  * (NULL: 0), alpha/beta (out) the final duals if non-NULL.
  * out[0] total iterations, out[1] last PD/lam, out[2] primal E (= D + PD),
  * out[3] dual D.  Synchronises.  Returns DOMDEC_WNOTCONV if the last stage hit
- * maxit. */
+ * maxit, DOMDEC_ECUDA if a pass cannot be launched (separable: a row must fit
+ * shared memory, N <= 8200 in double and 54000 in float on GB300). */
 #define DOMDEC_SINKHORN_DENSE     0
 #define DOMDEC_SINKHORN_SEPARABLE 1
 #define DOMDEC_SINKHORN_TI        4  /* or-ed into `variant`: translation step after each X-half (not in the

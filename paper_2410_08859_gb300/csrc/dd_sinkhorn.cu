@@ -356,14 +356,24 @@ struct Work {
 };
 
 // One separable pass: a CTA per row, or several where the rows alone are fewer
-// than four per SM of a 152-SM GPU.
+// than four per SM of a 152-SM GPU or where the targets' values do not fit beside the row
+// (double: N > 5250; the row alone fits up to N = 8200 in double, 54000 in float).
 template <typename R, bool FAST>
 cudaError_t sep_pass(const R* in, const float* inf, R* out, float* outf, int N, double q2, int shifted,
                      const SepHalf<R>& half, cudaStream_t st) {
   const int gy = std::max(1, std::min((N + 15) / 16, (608 + N - 1) / N));
-  const int per = (N + gy - 1) / gy, thr = std::min(1024, ((per * kSepLanes + 31) / 32) * 32);
   const int nb = (N + kSepBlock - 1) / kSepBlock;
-  const size_t sm = sizeof(R) * ((size_t)N + 2 * (size_t)per + 1) + (sizeof(R) == 8 ? 20 * (size_t)N : 0) + 4 * (size_t)nb + 16;
+  const size_t rowb = sizeof(R) * ((size_t)N + 1) + (sizeof(R) == 8 ? 20 * (size_t)N : 0) + 4 * (size_t)nb + 16;
+  int per = (N + gy - 1) / gy;
+  if (rowb + 2 * sizeof(R) * (size_t)per > 48 * 1024) {
+    int dev = 0, optin = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (rowb + 2 * sizeof(R) * 16 > (size_t)optin) return cudaErrorInvalidConfiguration;
+    per = (int)std::min<size_t>(per, (optin - rowb) / (2 * sizeof(R)));
+  }
+  const int thr = std::min(1024, ((per * kSepLanes + 31) / 32) * 32);
+  const size_t sm = rowb + 2 * sizeof(R) * (size_t)per;
   // Where the distances alone leave no term out (q2 (N - 1)^2 within the cut and a moderate
   // range of the sources) the windows are whole rows, and looking for them only costs: float,
   // us a pass with all its kernels, windows | without: N = 256 at q2 (N - 1)^2 = 11 16.4 | 14.4,
@@ -373,7 +383,10 @@ cudaError_t sep_pass(const R* in, const float* inf, R* out, float* outf, int N, 
   auto kernel = wide ? k_sep_rows_t<R, FAST, true> : k_sep_rows_t<R, FAST, false>;
   if (sm > 48 * 1024) {
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      return e;
+    }
   }
   kernel<<<dim3(N, (N + per - 1) / per), thr, sm, st>>>(in, inf, out, outf, N, q2, shifted, per, half);
   return cudaGetLastError();
@@ -416,15 +429,15 @@ cudaError_t lse_all(const R* in2, R* tmp, R* out2, int N, double q, int variant,
 // beta.  Where no check follows, the second pass of a half-step also writes the
 // potential and the next input (SepHalf).  check(it) is called every check_every
 // iterations and at the last one and returns true to stop.  Returns the
-// iterations made.
+// iterations made, or -1 with the error in *cerr when a pass could not be launched.
 template <typename R, typename Check>
 int sinkhorn_stage(const double* logmu, const double* lognu, double* alpha, double* beta, R* in2, float* in2f, R* tmp,
                    R* tmpz, float* tmpf, R* w2, R* z2, int N, double e, double kap, int variant, bool fast, int maxit,
-                   int check_every, bool fuse, cudaStream_t st, Check check, void (*after_x)(void*), void* ctx) {
+                   int check_every, bool fuse, cudaStream_t st, Check check, void (*after_x)(void*), void* ctx, cudaError_t* cerr) {
   const int n = N * N, grid = (n + 255) / 256;
   const double q = (1.0 / N) * (1.0 / N) / e;
   k_to_log2<R><<<grid, 256, 0, st>>>(beta, lognu, 1.0 / e, in2, n, in2f);
-  lse_all<R>(in2, tmp, w2, N, q, variant, 0, st, in2f, tmpf, fast);
+  if ((*cerr = lse_all<R>(in2, tmp, w2, N, q, variant, 0, st, in2f, tmpf, fast)) != cudaSuccess) return -1;
   const bool sep = variant == 1;
   bool ready = false;   // alpha and in2 are those of the coming half-step
   int it = 0, shift_ok = 0;
@@ -435,19 +448,21 @@ int sinkhorn_stage(const double* logmu, const double* lognu, double* alpha, doub
       k_to_log2<R><<<grid, 256, 0, st>>>(alpha, logmu, 1.0 / e, in2, n, in2f);
     }
     if (sep) {
-      lse_all<R>(in2, tmpz, z2, N, q, variant, shift_ok, st, in2f, tmpf, fast,
-                 SepHalf<R>{beta, lognu, in2, in2f, kap, 1.0 / e});
+      *cerr = lse_all<R>(in2, tmpz, z2, N, q, variant, shift_ok, st, in2f, tmpf, fast,
+                         SepHalf<R>{beta, lognu, in2, in2f, kap, 1.0 / e});
     } else {
-      lse_all<R>(in2, tmpz, z2, N, q, variant, shift_ok, st, in2f, tmpf, fast);
+      *cerr = lse_all<R>(in2, tmpz, z2, N, q, variant, shift_ok, st, in2f, tmpf, fast);
       k_half<R><<<grid, 256, 0, st>>>(z2, kap, beta, n);
       k_to_log2<R><<<grid, 256, 0, st>>>(beta, lognu, 1.0 / e, in2, n, in2f);
     }
+    if (*cerr != cudaSuccess) return -1;
     shift_ok = 1;
     ++it;
     const bool checked = it % check_every == 0 || it == maxit;
     ready = sep && fuse && !checked;
-    lse_all<R>(in2, tmp, w2, N, q, variant, 1, st, in2f, tmpf, fast,
-               ready ? SepHalf<R>{alpha, logmu, in2, in2f, kap, 1.0 / e} : SepHalf<R>{});
+    *cerr = lse_all<R>(in2, tmp, w2, N, q, variant, 1, st, in2f, tmpf, fast,
+                       ready ? SepHalf<R>{alpha, logmu, in2, in2f, kap, 1.0 / e} : SepHalf<R>{});
+    if (*cerr != cudaSuccess) return -1;
     if (checked && check(it)) break;
   }
   return it;
@@ -464,7 +479,8 @@ cudaError_t global_lse64(const double* pot, const double* logm, double eps, doub
   float* sh_in = reinterpret_cast<float*>(buf_c);
   float* sh_tmp = sh_in + n;
   k_to_log2<double><<<(n + 255) / 256, 256, 0, st>>>(pot, logm, 1.0 / eps, buf_a, n, sh_in);
-  lse_all<double>(buf_a, buf_b, buf_a, N, h * h / eps, 1, 0, st, sh_in, sh_tmp);
+  const cudaError_t e = lse_all<double>(buf_a, buf_b, buf_a, N, h * h / eps, 1, 0, st, sh_in, sh_tmp);
+  if (e != cudaSuccess) return e;
   k_to_nat<double><<<(n + 255) / 256, 256, 0, st>>>(buf_a, out, n);
   return cudaGetLastError();
 }
@@ -515,8 +531,8 @@ static int full_sinkhorn_impl(const double* mu, const double* nu, const double* 
           conv = err >= 0.0 && gap <= err * evalh[4];
           return conv || !(gap == gap);
         },
-        ti ? +ti_run : nullptr, &tc);
-    if (broke) { cudaFreeAsync(w.in2, st); return -1; }
+        ti ? +ti_run : nullptr, &tc, cerr);
+    if (broke || it < 0) { cudaFreeAsync(w.in2, st); return -1; }
     total += it;
     if (e <= eps) { rc = conv || err < 0.0 ? 0 : 1; break; }
     e = fmax(eps, 0.5 * e);
@@ -651,8 +667,8 @@ int full_sinkhorn_noalloc_impl(const double* mu, const double* nu, const double*
           conv = err >= 0.0 && evalh[0] <= err * evalh[4];
           return conv || !(evalh[0] == evalh[0]);
         },
-        nullptr, nullptr);
-    if (broke) return -1;
+        nullptr, nullptr, cerr);
+    if (broke || it < 0) return -1;
     total += it;
     if (e <= eps) { rc = conv || err < 0.0 ? 0 : 1; break; }
     e = fmax(eps, 0.5 * e);

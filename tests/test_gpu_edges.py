@@ -180,3 +180,46 @@ def test_separable_passes_around_whole_rows(env, N, reach, precision, tol):
         for got, ref in ((a, alpha), (b, beta)):
             scale = float(ref.abs().max()) + (0.0 if start is None else float(start.abs().max()))
             assert float((got - ref).abs().max()) <= tol * (scale + eps)
+
+
+# ------------------------------------------------------------------- large grids
+@pytest.mark.parametrize("N,precision,tol", [(5600, 1, 1e-12), (8000, 1, 1e-12), (5600, 2, 1e-6), (8000, 0, 1e-6)])
+def test_separable_sinkhorn_on_large_grids(env, N, precision, tol):
+    """Rows that leave no room for a whole row of results: alpha of the first half-step at sampled
+    pixels, from the sources within e^-60 of them (the tolerances are relative to the largest
+    exponent, log nu)."""
+    torch, dd = env
+    free, _ = torch.cuda.mem_get_info()
+    if free < 30 * N * N * 8:
+        pytest.skip("not enough device memory")
+    g = torch.Generator(device="cuda").manual_seed(N)
+    mu = torch.rand(N, N, generator=g, device="cuda", dtype=torch.float64) + 0.5
+    nu = torch.rand(N, N, generator=g, device="cuda", dtype=torch.float64) + 0.5
+    mu, nu = mu / mu.sum(), nu / nu.sum()
+    eps_px = 100.0 if precision == 0 else 4.0
+    eps, lam = eps_px / N ** 2, 1.0
+    a = torch.zeros_like(mu)
+    dd.domdec_full_sinkhorn(mu, nu, N, eps, lam, eps_start=eps, precision=precision, maxit=1, err=-1.0, alpha=a)
+    rng, w = np.random.default_rng(N), int((60 * eps_px) ** 0.5) + 1
+    for i, j in [(0, 0), (N - 1, N - 1), (N // 2, N - 1)] + [tuple(rng.integers(0, N, 2)) for _ in range(60)]:
+        i0, i1, j0, j1 = max(0, i - w), min(N, i + w + 1), max(0, j - w), min(N, j + w + 1)
+        I = torch.arange(i0, i1, device="cuda", dtype=torch.float64)[:, None] - int(i)
+        J = torch.arange(j0, j1, device="cuda", dtype=torch.float64)[None, :] - int(j)
+        ref = -eps / (1 + eps / lam) * torch.logsumexp((nu[i0:i1, j0:j1].log() - (I * I + J * J) / eps_px).reshape(-1), 0)
+        assert abs(float(a[i, j]) - float(ref)) <= tol * 20 * eps
+
+
+def test_separable_sinkhorn_reports_rows_that_do_not_fit(env):
+    """A row of 8300 doubles with its tables is beyond shared memory: an error, not untouched output;
+    the library goes on working."""
+    torch, dd = env
+    N = 8300
+    free, _ = torch.cuda.mem_get_info()
+    if free < 30 * N * N * 8:
+        pytest.skip("not enough device memory")
+    mu = torch.full((N * N,), 1.0 / N ** 2, dtype=torch.float64, device="cuda")
+    with pytest.raises(dd.DomDecError) as e:
+        dd.domdec_full_sinkhorn(mu, mu, N, 4.0 / N ** 2, 1.0, precision=1, maxit=1, err=-1.0)
+    assert e.value.code == dd.DOMDEC_ECUDA
+    m = torch.full((1024,), 1.0 / 1024, dtype=torch.float64, device="cuda")
+    assert dd.domdec_full_sinkhorn(m, m, 32, 0.01, 1.0, precision=1, maxit=5, err=-1.0)[0] == 5
