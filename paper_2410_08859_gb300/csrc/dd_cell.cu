@@ -2174,12 +2174,7 @@ int cell_resident_ctas(size_t smem, int C, int precision) {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   cudaError_t e;
-  if (precision) e = cudaFuncSetAttribute(k_cell_solve<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  else e = cudaFuncSetAttribute(k_cell_solve<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
+  if (smem > (precision ? allow_smem(k_cell_solve<double, false>) : allow_smem(k_cell_solve<float, false>))) return 0;
   if (C <= 1) {
     int per = 0;
     e = precision ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_cell_solve<double, false>, kCellThreads, smem)
@@ -2231,7 +2226,7 @@ cudaError_t launch_cell_solve(const DevState& S, const CellDesc* cells, const in
   cfg.attrs = attr;
   cfg.numAttrs = C > 1 ? 1 : 0;
   auto run = [&](auto kernel) {
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem(kernel);
     return cudaLaunchKernelEx(&cfg, kernel, S, cells, order, nbig_p, begin, nbatch, crun, C);
   };
   if (S.balance) return precision ? run(k_cell_solve<double, true>) : run(k_cell_solve<float, true>);
@@ -2248,7 +2243,7 @@ cudaError_t launch_cell_solve_multi(const DevState* states, const CellRef* refs,
   int P = 1;
   while (P < nref) P <<= 1;
   const size_t osm = (size_t)std::min(P, kRefOrderMax) * sizeof(unsigned long long);
-  cudaFuncSetAttribute(k_ref_order, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)osm);
+  allow_smem(k_ref_order);
   k_ref_order<<<1, 1024, osm, st>>>(states, refs, nref, part, C, factor, nctas, order, nbig);
   cudaMemsetAsync(queue, 0, 2 * sizeof(unsigned int), st);
   cudaLaunchConfig_t cfg = {};
@@ -2264,11 +2259,11 @@ cudaError_t launch_cell_solve_multi(const DevState* states, const CellRef* refs,
   cfg.attrs = attr;
   cfg.numAttrs = C > 1 ? 1 : 0;
   if (precision) {
-    cudaFuncSetAttribute(k_cell_solve_multi<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem(k_cell_solve_multi<double>);
     return cudaLaunchKernelEx(&cfg, k_cell_solve_multi<double>, states, refs, (const int*)order, (const int*)nbig,
                               nref, part, queue, C);
   }
-  cudaFuncSetAttribute(k_cell_solve_multi<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_smem(k_cell_solve_multi<float>);
   return cudaLaunchKernelEx(&cfg, k_cell_solve_multi<float>, states, refs, (const int*)order, (const int*)nbig, nref,
                             part, queue, C);
 }
@@ -2278,15 +2273,8 @@ int cell_multi_resident_ctas(size_t smem, int C, int precision) {
   int dev = 0, nsm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  cudaError_t e = precision
-                      ? cudaFuncSetAttribute(k_cell_solve_multi<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem)
-                      : cudaFuncSetAttribute(k_cell_solve_multi<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
+  if (smem > (precision ? allow_smem(k_cell_solve_multi<double>) : allow_smem(k_cell_solve_multi<float>))) return 0;
+  cudaError_t e;
   if (C <= 1) {
     int per = 0;
     e = precision ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_cell_solve_multi<double>, kCellThreads, smem)

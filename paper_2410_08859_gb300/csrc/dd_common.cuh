@@ -302,6 +302,29 @@ __device__ __forceinline__ double dd_kl_term(double p, double m) {
   return p * log(p / m) - p + m;
 }
 
+// Allows a kernel all the dynamic shared memory that the device has beside the kernel's
+// static one, and returns how much that is (0: an error).  Always that much, never one
+// call's need: the limit belongs to the function, and another host thread may be between its
+// own call of this and its launch.
+inline size_t allow_smem_of(const void* kernel) {
+  int dev = 0, optin = 0;
+  cudaFuncAttributes a;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, kernel);
+  const int room = e == cudaSuccess ? optin - (int)a.sharedSizeBytes : 0;
+  if (e == cudaSuccess && a.maxDynamicSharedSizeBytes < room)
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, room);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return (size_t)room;
+}
+template <typename... A> inline size_t allow_smem(void (*kernel)(A...)) {
+  return allow_smem_of(reinterpret_cast<const void*>(kernel));
+}
+
 // ------------------------------------------------------------- reductions
 template <typename T> __device__ __forceinline__ T warp_sum(T v) {
 #pragma unroll

@@ -218,10 +218,7 @@ template <bool MOM>
 cudaError_t adj_side_tiles(const double* f, const float* fs, double* a, float* as, double* m, const AdjOut& O, int N,
                            double Q, cudaStream_t st) {
   auto run = [&](auto kernel, const TileShape& t, auto... args) {
-    if (t.smem > 40 * 1024) {
-      const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)t.smem);
-      if (e != cudaSuccess) return e;
-    }
+    if (t.smem > 40 * 1024 && t.smem > allow_smem(kernel)) return cudaErrorInvalidConfiguration;
     kernel<<<t.grid, t.threads, t.smem, st>>>(args..., N, Q, t.per, t.D4);
     return cudaGetLastError();
   };

@@ -381,13 +381,7 @@ cudaError_t sep_pass(const R* in, const float* inf, R* out, float* outf, int N, 
   // N = 64 at 11 4.9 | 4.1; double N = 64 at 45 14.4 | 13.3, N = 256 at 46 467 | 467.
   const bool wide = q2 * (double)(N - 1) * (double)(N - 1) <= 64.0;
   auto kernel = wide ? k_sep_rows_t<R, FAST, true> : k_sep_rows_t<R, FAST, false>;
-  if (sm > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) {
-      cudaGetLastError();
-      return e;
-    }
-  }
+  if (sm > 48 * 1024 && sm > allow_smem(kernel)) return cudaErrorInvalidConfiguration;
   kernel<<<dim3(N, (N + per - 1) / per), thr, sm, st>>>(in, inf, out, outf, N, q2, shifted, per, half);
   return cudaGetLastError();
 }

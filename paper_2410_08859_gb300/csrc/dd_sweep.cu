@@ -1069,7 +1069,7 @@ cudaError_t launch_init_duals_boxes(const DevState& S, const double* alpha0, con
   float* tmax = gscratch + n;
   k_tile_max<<<ntc * ntc, 256, 0, st>>>(gscratch, S.N, tmax);
   const size_t sm = init_box_smem(S.s, S.N);
-  cudaFuncSetAttribute(k_init_duals, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  allow_smem(k_init_duals);   // a need beyond the device's limit fails at the launch
   k_init_duals<<<S.nbasic, 1024, sm, st>>>(S, alpha0, beta0, eps0, 0, gscratch, tmax);
   k_scan_boxes<<<1, 1024, 0, st>>>(S, newoff);
   return cudaGetLastError();
@@ -1078,7 +1078,7 @@ cudaError_t launch_init_duals_fill(const DevState& S, const double* alpha0, cons
                                    const double* w, long long* newoff, cudaStream_t st) {
   k_set_offsets<<<(S.nbasic + 255) / 256, 256, 0, st>>>(S, newoff);
   const size_t sm = (3 * sizeof(double) + sizeof(float)) * (size_t)S.s * kInitChunk + (2 * sizeof(double) + sizeof(float)) * (size_t)S.s * S.s;
-  cudaFuncSetAttribute(k_init_duals, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::max(sm, init_box_smem(S.s, S.N)));
+  allow_smem(k_init_duals);
   k_init_duals<<<S.nbasic, 256, sm, st>>>(S, alpha0, beta0, eps0, 1, nullptr, nullptr);
   k_px_duals<<<(S.N * S.N + 255) / 256, 256, 0, st>>>(S, alpha0, w, eps0);
   return cudaGetLastError();

@@ -223,3 +223,52 @@ def test_separable_sinkhorn_reports_rows_that_do_not_fit(env):
     assert e.value.code == dd.DOMDEC_ECUDA
     m = torch.full((1024,), 1.0 / 1024, dtype=torch.float64, device="cuda")
     assert dd.domdec_full_sinkhorn(m, m, 32, 0.01, 1.0, precision=1, maxit=5, err=-1.0)[0] == 5
+
+
+# ------------------------------------------------------------------ several host threads
+def test_threads_with_grids_of_different_sizes(env):
+    """The same kernels launched from threads whose calls need different amounts of shared memory, each
+    on its own stream: what one thread asks for must not shrink what another is about to
+    launch with.  Every result equals the one of a thread alone."""
+    import threading
+    torch, dd = env
+    jobs = []
+    for N, prec in ((1200, dd.FP64), (2000, dd.FP64), (1600, dd.FP64), (1200, dd.MIXED)):
+        g = torch.Generator(device="cuda").manual_seed(N)
+        mu = torch.rand(N * N, generator=g, device="cuda", dtype=torch.float64) + 0.5
+        mu /= mu.sum()
+        jobs.append([N, prec, mu, torch.empty_like(mu), torch.empty_like(mu), torch.empty_like(mu), torch.empty_like(mu)])
+
+    def solve(N, prec, mu, a, b, gm, gx, stream=None):
+        eps = 4.0 / N ** 2
+        dd.domdec_full_sinkhorn(mu, mu, N, eps, 1.0, eps_start=eps, precision=prec, maxit=4, err=-1.0, check_every=2,
+                                alpha=a, beta=b, stream=stream)
+        dd.domdec_uot_gradients(mu, mu, a, b, N, eps, 1.0, grad_mu=gm, grad_nu=gx, stream=stream)
+
+    ref = []
+    for j in jobs:
+        solve(*j)
+        ref.append([t.clone() for t in j[3:]])
+        for t in j[3:]:
+            t.zero_()
+    torch.cuda.synchronize()
+    errors = []
+
+    def work(k):
+        try:
+            st = torch.cuda.Stream()
+            for _ in range(6):
+                solve(*jobs[k], stream=st)
+        except Exception as e:   # noqa: BLE001
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(len(jobs))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not errors, errors
+    for j, r in zip(jobs, ref):
+        for got, want in zip(j[3:], r):
+            assert torch.equal(got, want)
