@@ -832,7 +832,6 @@ __device__ __forceinline__ void cell_solve_body(const DevState& S, const CellDes
   R* apart = gpart + 32;                             // per-warp <e^{-alpha/lam}, mu> (translation step)
   R* bpart = gpart + 64;                             // per-warp <e^{-beta/lam}, nu>
   int* pend = reinterpret_cast<int*>(red + 256);    // kPend list entries (the last 2 KB of red)
-  const int lock = sizeof(R) == 4 ? kLock : S.newton_maxit;
   const bool ti = S.ti && sl > 0.0;
   const int lane = tid & 31, wid = tid >> 5, nwarp = nthr >> 5;
   int it = 0;
@@ -885,22 +884,23 @@ __device__ __forceinline__ void cell_solve_body(const DevState& S, const CellDes
       bool open[B];
       if constexpr (sizeof(R) == 8) {
         root[0] = newton_f64(lr[0], c0[0], uw[0], sR, is, i1s, S.newton_maxit);
-        open[0] = false;
       } else {
-        newton_tile<R, B>(lr, c0, uw, sR, min(S.newton_maxit, lock), root, open);
+        newton_tile<R, B>(lr, c0, uw, sR, min(S.newton_maxit, kLock), root, open);
       }
 #pragma unroll
       for (int k = 0; k < B; ++k) {
         if (k >= n) break;
-        if (lock < S.newton_maxit && open[k]) {
-          const int v = (kk + k) * Wp + ll, e = atomicAdd(&npend, 1);
-          if (e < kPend) {   // finished below from the list
-            pend[e] = v;
-            bv[v] = root[k];
-            Zv[v] = fused_y ? Zn[k] : Z2[k];
-            continue;
+        if constexpr (sizeof(R) == 4) {
+          if (kLock < S.newton_maxit && open[k]) {
+            const int v = (kk + k) * Wp + ll, e = atomicAdd(&npend, 1);
+            if (e < kPend) {   // finished below from the list
+              pend[e] = v;
+              bv[v] = root[k];
+              Zv[v] = fused_y ? Zn[k] : Z2[k];
+              continue;
+            }
+            root[k] = newton_rest(lr[k], c0[k], root[k], sR, S.newton_maxit - kLock);
           }
-          root[k] = newton_rest(lr[k], c0[k], root[k], sR, S.newton_maxit - lock);
         }
         y_store((kk + k) * Wp + ll, (kk + k) * W + ll, root[k], fused_y ? Zn[k] : Z2[k], Zn[k], c0[k]);
       }
@@ -915,7 +915,7 @@ __device__ __forceinline__ void cell_solve_body(const DevState& S, const CellDes
         const R Zx = Zv[v], Zn = fused_y ? Zx : mul_rn(Zx, LN2);
         const R eta1 = R(k0 + kk - yc1), eta2 = R(l0 + ll - yc2);
         const R c0 = sB - cEta1 * eta1 - cEta2 * eta2 - sR * Zn;
-        y_store(v, kk * W + ll, newton_rest(lrho[v], c0, bv[v], sR, S.newton_maxit - lock), Zx, Zn, c0);
+        y_store(v, kk * W + ll, newton_rest(lrho[v], c0, bv[v], sR, S.newton_maxit - kLock), Zx, Zn, c0);
       }
     } else {
       run_pass(T, 1, Wp, Zv, 1, Wp, W, H, nx1, offr, q2, first, tid, nthr,
@@ -1521,7 +1521,6 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
     int st;
     tib = reinterpret_cast<R*>(cell_nut(S, tmp, cidx, &st)) + kb * W;
   }
-  const int lock = sizeof(R) == 4 ? kLock : S.newton_maxit;
   int it = 0;
   double gap = 0.0;   // of thread 0
   bool first = true;
@@ -1563,22 +1562,23 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
       bool open[B];
       if constexpr (sizeof(R) == 8) {
         root[0] = newton_f64(lr[0], c0[0], uw[0], sR, is, i1s, S.newton_maxit);
-        open[0] = false;
       } else {
-        newton_tile<R, B>(lr, c0, uw, sR, min(S.newton_maxit, lock), root, open);
+        newton_tile<R, B>(lr, c0, uw, sR, min(S.newton_maxit, kLock), root, open);
       }
 #pragma unroll
       for (int k = 0; k < B; ++k) {
         if (k >= n) break;
-        if (lock < S.newton_maxit && open[k]) {
-          const int v = (kl + k) * Wp + ll, e = atomicAdd(&npend, 1);
-          if (e < kPend) {   // finished below from the list
-            pend[e] = v;
-            bv[v] = root[k];
-            Zv[v] = fused_y ? Zn[k] : Z2[k];
-            continue;
+        if constexpr (sizeof(R) == 4) {
+          if (kLock < S.newton_maxit && open[k]) {
+            const int v = (kl + k) * Wp + ll, e = atomicAdd(&npend, 1);
+            if (e < kPend) {   // finished below from the list
+              pend[e] = v;
+              bv[v] = root[k];
+              Zv[v] = fused_y ? Zn[k] : Z2[k];
+              continue;
+            }
+            root[k] = newton_rest(lr[k], c0[k], root[k], sR, S.newton_maxit - kLock);
           }
-          root[k] = newton_rest(lr[k], c0[k], root[k], sR, S.newton_maxit - lock);
         }
         y_store((kl + k) * Wp + ll, (kl + k) * W + ll, root[k], fused_y ? Zn[k] : Z2[k], c0[k]);
       }
@@ -1593,7 +1593,7 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
         const R Zx = Zv[v], Zn = fused_y ? Zx : mul_rn(Zx, LN2);
         const R eta1 = R(k0 + kb + kl - yc1), eta2 = R(l0 + ll - yc2);
         const R c0 = sB - cEta1 * eta1 - cEta2 * eta2 - sR * Zn;
-        y_store(v, kl * W + ll, newton_rest(lrho[v], c0, bv[v], sR, S.newton_maxit - lock), Zx, c0);
+        y_store(v, kl * W + ll, newton_rest(lrho[v], c0, bv[v], sR, S.newton_maxit - kLock), Zx, c0);
       }
     } else {
       run_pass(T, 1, Wp, Zv, 1, Wp, W, Hl, nx1, offr + kb, q2, first, tid, nthr,

@@ -164,13 +164,11 @@ __device__ __forceinline__ void tile_rows(unsigned char* sm, const double* __res
       if (MOM >= 1) a1[e] = 0.0;
       if (MOM == 2) a2[e] = 0.0;
     }
-    bool over = false;
     if (usable)
       for (int m = lo + part; m < hi; m += P) {
-        float v = -INFINITY;
+        float v = -INFINITY;   // S holds the maxima of these terms: v <= 0
 #pragma unroll
         for (int e = 0; e < kTile; ++e) v = fmaxf(v, term_f(m, j0 + e) - S[e]);
-        over |= v > 60.0f;
         if (v > -cutf) {
           const double2 t = qd[abs(m - a)];
           const double G = dd_ex2(fma(-t.x, t.y, row[m]) - sref);
@@ -195,9 +193,8 @@ __device__ __forceinline__ void tile_rows(unsigned char* sm, const double* __res
         if (MOM >= 1) a1[e] += __shfl_xor_sync(0xffffffffu, a1[e], o);
         if (MOM == 2) a2[e] += __shfl_xor_sync(0xffffffffu, a2[e], o);
       }
-    for (int o = 1; o < P; o <<= 1) over |= __shfl_xor_sync(0xffffffffu, (int)over, o) != 0;
     // lane `part` keeps targets part, part + P, ...
-    bool bad = !usable || over;
+    bool bad = !usable;
 #pragma unroll
     for (int e = 0; e < kTile; ++e)
       if (e < n && (e & (P - 1)) == part) {
