@@ -272,3 +272,72 @@ def test_threads_with_grids_of_different_sizes(env):
     for j, r in zip(jobs, ref):
         for got, want in zip(j[3:], r):
             assert torch.equal(got, want)
+
+
+# ------------------------------------------- single-precision cells beyond shared memory
+# eps/lam = 1/4, so a root amplifies a rounding four times at most; an exponent of magnitude
+# below 50 costs 3e-6 a pass, and there are four passes in each of three iterations
+FP32_TOL = 1e-4
+
+
+def test_fp32_boxes_beyond_shared_memory(env):
+    """192 x 192 boxes of a product plan in single precision: the list of slow roots, the tiles and
+    the odd pitches with per-y arrays in a slot, on one CTA and on clusters, against double cells."""
+    torch, dd = env
+    N, s = 192, 8
+    mu, nu = inputs.mixture_blobs(N=N, seed=10)
+    eps = 16.0 / N ** 2
+    out = []
+    for precision, c in (("fp64", 8), ("fp32", 1), ("fp32", 2), ("fp32", 4), ("fp32", 8)):
+        with dd.DomDec(mu, nu, eps, 4 * eps, s, precision=precision, cell_ctas=c, err=-1.0, maxit=3, strategy="safe",
+                       spill_slots=144) as g:
+            g.iterate(1)
+            g.sync()
+            out.append((*g.marginals(), g.duals(), g.cell_log()))
+    ref = out[0]
+    assert (out[1][3][:, 7] >= 0).any()   # cells with a slot
+    for got in out[1:]:
+        for k in range(2):
+            assert np.abs(got[k] - ref[k]).sum() <= FP32_TOL * np.abs(ref[k]).sum()
+        assert np.abs(got[2] - ref[2]).max() <= FP32_TOL * np.abs(ref[2]).max()
+
+
+def test_fp32_regrouped_sweep_is_that_of_the_larger_cluster(env):
+    """A sweep that regroups from clusters of two to four ends where one started on four does."""
+    torch, dd = env
+    N, s = 176, 8
+    mu, nu = inputs.mixture_blobs(N=N, seed=12)
+    eps = 16.0 / N ** 2
+    out = []
+    for first in (4, 2):
+        with dd.DomDec(mu, nu, eps, 4 * eps, s, precision="fp32", err=-1.0, maxit=3, strategy="staggered",
+                       spill_slots=1) as g:
+            assert g.set_launch(first, 2.0) == first
+            g.iterate(1)
+            g.sync()
+            assert (g.stats()["cluster_regroups"] >= 1) == (first == 2)
+            out.append((*g.marginals(), g.duals()))
+    for k in range(2):
+        assert np.abs(out[1][k] - out[0][k]).sum() <= FP32_TOL * np.abs(out[0][k]).sum()
+    assert np.abs(out[1][2] - out[0][2]).max() <= FP32_TOL * np.abs(out[0][2]).max()
+
+
+@pytest.mark.parametrize("N,s", [(32, 4), (64, 8), (64, 16)])
+@pytest.mark.parametrize("ctas", [2, 8])
+def test_translation_step_stops_alike_on_clusters(env, N, s, ctas):
+    """Double cells with the translation step that stop on a tolerance: the same iterations and
+    marginals on clusters as on one CTA each (t*/eps amplifies a rounding by lam/eps = 100)."""
+    torch, dd = env
+    mu, nu = inputs.mixture_blobs(N=N, seed=22)
+    eps = 4.0 / N ** 2
+    out = []
+    for c in (1, ctas):
+        with dd.DomDec(mu, nu, eps, 100 * eps, s, precision="fp64", cell_ctas=c, cell_ti=1, err=1e-4, maxit=3000,
+                       strategy="safe", spill_slots=100) as g:
+            g.iterate(2)
+            g.sync()
+            out.append((g.cell_log(), *g.marginals()))
+    one, got = out
+    assert (got[0][:, 5] == 0).all() and np.array_equal(got[0][:, :5], one[0][:, :5])
+    for k in (1, 2):
+        assert np.abs(got[k] - one[k]).sum() <= 1e-9 * np.abs(one[k]).sum()
