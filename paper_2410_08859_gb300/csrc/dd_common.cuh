@@ -270,13 +270,13 @@ __device__ __forceinline__ double rcp_short(double b) {
   const double r = widen_pos(dd_rcp(narrow(b)));
   return fma(fma(-b, r, 1.0), r, r);
 }
-__device__ __forceinline__ bool mid_range(double x) {   // 2^-120 <= x < 2^121
-  return ((unsigned)__double2hiint(x) >> 20) - (1023u - 120u) <= 240u;
+__device__ __forceinline__ bool mid_range(double x, unsigned e = 120u) {   // 2^-e <= x < 2^(e + 1)
+  return ((unsigned)__double2hiint(x) >> 20) - (1023u - e) <= 2u * e;
 }
 // a/b for a >= 0, b > 0: q = a (1/b), corrected by its remainder a - q b (q and 1/b are
 // short of their values by 2^-44, so what the correction leaves is 2^-88: a rounding).
 __device__ __forceinline__ double dd_div(double a, double b) {
-  if (!mid_range(b) || !(a >= 0x1p-800 && a < 0x1p800)) return a / b;
+  if (!mid_range(b) || !mid_range(a, 800u)) return a / b;
   const double r = rcp_short(b), q = a * r;
   return fma(fma(-q, b, a), r, q);
 }
@@ -285,7 +285,7 @@ __device__ __forceinline__ double dd_div(double a, double b) {
 // log(a/b) near a = b, drops out; the second part of log 2 leaves one rounding of the
 // result and two of the table's value.  Largest error against long arithmetic (a/b in
 // 1 +- 0.1 | 0.5..2 | 1e-6..1e6): 1.4e-17 | 8.2e-17 | 9.4e-16; CUDA's log of CUDA's quotient 1.1e-16 |
-// 1.6e-16 | 9.8e-16, at 9.53 against 9.16 ms for a 256 x 256 solve with line searches (log a - log b:
+// 1.6e-16 | 9.8e-16, at 9.53 against 9.11 ms for a 256 x 256 solve with line searches (log a - log b:
 // 4e-15 in all three, 8.97).
 __device__ __forceinline__ double dd_log_quotient(double a, double b) {
   if (!mid_range(a) || !mid_range(b)) return log(a / b);
