@@ -642,19 +642,31 @@ struct CellScalars {
   }
 };
 
+// What a CTA shares of the cell it works on, one object for both ways of solving it (a
+// cell's barriers end before the next one's begin): static shared memory is taken from
+// the Y-box capacity.
+template <typename R>
+struct CellShared {
+  CellScalars<R> sk;
+  BoxRec box[4];
+  int geo[8];
+  int npend;
+  bool stop;
+};
+
 // One composite cell on one CTA: cell `cd` at position `cidx` of a sub-batch
 // of `nbatch` cells.
 // BAL: with the balancing step (an instance of its own: its registers cost the plain
 // solve spills).
 template <typename R, bool BAL>
 __device__ __forceinline__ void cell_solve_body(const DevState& S, const CellDesc cd, int cidx, int nbatch,
-                                                unsigned char* smem_raw) {
+                                                CellShared<R>& sh, unsigned char* smem_raw) {
   namespace cg = cooperative_groups;
   double* red = reinterpret_cast<double*>(smem_raw);  // 32 * 16 doubles (block reductions)
-  __shared__ BoxRec sbox[4];
-  __shared__ int sgeo[8];
-  __shared__ CellScalars<R> sk;
-  __shared__ int npend;
+  BoxRec* sbox = sh.box;
+  int* sgeo = sh.geo;
+  CellScalars<R>& sk = sh.sk;
+  int& npend = sh.npend;
   CellOut* out = S.cout + cidx;
   const unsigned long long t_start = dd_global_ns();
   const double* __restrict__ arena = S.arena[*S.cur];
@@ -881,7 +893,7 @@ __device__ __forceinline__ void cell_solve_body(const DevState& S, const CellDes
         lr[k] = lrho[v];
         uw[k] = first ? dd_inf<R>() : bv[v] + Zn[k];
       }
-      bool open[B];
+      [[maybe_unused]] bool open[B];
       if constexpr (sizeof(R) == 8) {
         root[0] = newton_f64(lr[0], c0[0], uw[0], sR, is, i1s, S.newton_maxit);
       } else {
@@ -1314,20 +1326,26 @@ __device__ __forceinline__ bool fits_hybrid(const DevState& S, int nx1, int nx2,
   return nx1 * Wo + Hc * (nx2 | 1) + Hc * Wo <= room && 3LL * nx1 * W <= room && H * Wo <= (long long)S.N * S.N;
 }
 
-constexpr int kDistMaxC = 8;
+constexpr int kDistMaxC = 8, kDx = 12;
 
 template <typename R>
 __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDesc cd, int cidx, int nbatch,
-                                                int crank, int C, unsigned char* smem_raw) {
+                                                int crank, int C, CellShared<R>& sh, unsigned char* smem_raw) {
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
   double* red = reinterpret_cast<double*>(smem_raw);   // 32 * 16 doubles (block reductions)
-  __shared__ BoxRec dbox[4];
-  __shared__ int dgeo[8];
-  __shared__ int npend;
-  __shared__ bool stop;
-  __shared__ CellScalars<R> sk;
-  __shared__ double dx[kDistMaxC * 16];                 // partial sums of every CTA of the cluster
+  BoxRec* dbox = sh.box;
+  int* dgeo = sh.geo;
+  CellScalars<R>& sk = sh.sk;
+  int& npend = sh.npend;
+  bool& stop = sh.stop;
+  // partial sums of every CTA of the cluster, kDx each: in double at the end of the reductions'
+  // space, beyond the largest sum's 396 values and the gap's parts; the float cells' list lies there
+  double* dx = red + 400;
+  if constexpr (sizeof(R) == 4) {
+    __shared__ double dx_own[kDistMaxC * kDx];
+    dx = dx_own;
+  }
   CellOut* out = S.cout + cidx;
   const unsigned long long t_start = dd_global_ns();
   const double* __restrict__ arena = S.arena[*S.cur];
@@ -1453,11 +1471,11 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
     if (tid == 0)
       for (int r = 0; r < C; ++r) {
         double* px = cl.map_shared_rank(dx, r);
-        for (int k = 0; k < 4; ++k) px[crank * 16 + k] = m3[k];
+        for (int k = 0; k < 4; ++k) px[crank * kDx + k] = m3[k];
       }
     csync();
     double t0 = 0.0, t1 = 0.0, t2 = 0.0;
-    for (int r = 0; r < C; ++r) { t0 += dx[r * 16]; t1 += dx[r * 16 + 1]; t2 += dx[r * 16 + 2]; a_tot += dx[r * 16 + 3]; }
+    for (int r = 0; r < C; ++r) { t0 += dx[r * kDx]; t1 += dx[r * kDx + 1]; t2 += dx[r * kDx + 2]; a_tot += dx[r * kDx + 3]; }
     c1 = H / 2; c2 = W / 2;
     if (t0 > 0.0) {
       c1 = min(H - 1, max(0, (int)lrint(t1 / t0)));
@@ -1508,7 +1526,7 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
   (void)i1s;
   int* pend = reinterpret_cast<int*>(red + 256);    // as in cell_solve_body
   // translation step, as in cell_solve_body: nu e^{-beta/lam} of the own rows in the
-  // cell's buffer of new marginals, every CTA's sum in dx[16 rk + 4] of all CTAs.  It
+  // cell's buffer of new marginals, every CTA's sum in dx[kDx rk + 4] of all CTAs.  It
   // travels with the parts of W, so it adds no cluster barrier (such cells ran on one
   // CTA before: 256 x 256, s = 8, largest box 11 583 points 1.94 -> 0.70 ms).
   const bool ti = S.ti && sl > 0.0;
@@ -1559,7 +1577,7 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
         lr[k] = lrho[v];
         uw[k] = first ? dd_inf<R>() : bv[v] + Zn[k];
       }
-      bool open[B];
+      [[maybe_unused]] bool open[B];
       if constexpr (sizeof(R) == 8) {
         root[0] = newton_f64(lr[0], c0[0], uw[0], sR, is, i1s, S.newton_maxit);
       } else {
@@ -1616,7 +1634,7 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
     if (ti && tid == 0) {
       double bs = 0.0;
       for (int w = 0; w < (nthr >> 5); ++w) bs += (double)bpart[w];
-      for (int rk = 0; rk < C; ++rk) cl.map_shared_rank(dx, rk)[crank * 16 + 4] = bs;
+      for (int rk = 0; rk < C; ++rk) cl.map_shared_rank(dx, rk)[crank * kDx + 4] = bs;
     }
     // X-half on the own rows: U(kl, c) = log2 sum_ll 2^{bl(kl,ll) - q2 (ll - (c - offc))^2}
     run_pass(bl, Wp, 1, U, Up, 1, Hl, nx2, W, -offc, q2, first, tid, nthr, [&](int kl, int c, int n, const auto& v) {
@@ -1689,7 +1707,7 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
       if (tid == 0) {
         double As = 0.0, Bs = 0.0;
         for (int w = 0; w < (nthr >> 5); ++w) As += (double)apart[w];
-        for (int rk = 0; rk < C; ++rk) Bs += dx[rk * 16 + 4];
+        for (int rk = 0; rk < C; ++rk) Bs += dx[rk * kDx + 4];
         sk.translate(S, A, a_tot, As, Bs);
       }
       __syncthreads();
@@ -1801,13 +1819,13 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
   cell_sum<R, 12>(hsd, red);
   if (tid == 0) {
     double* p0 = cl.map_shared_rank(dx, 0);
-    for (int k = 0; k < 12; ++k) p0[crank * 16 + k] = hsd[k];
+    for (int k = 0; k < 12; ++k) p0[crank * kDx + k] = hsd[k];
   }
   csync();
   if (crank != 0 || tid != 0) return;
   for (int k = 0; k < 12; ++k) {
     double a = 0.0;
-    for (int r = 0; r < C; ++r) a += dx[r * 16 + k];
+    for (int r = 0; r < C; ++r) a += dx[r * kDx + k];
     hsd[k] = a;
   }
   CellOut o;
@@ -1846,6 +1864,7 @@ k_cell_solve(DevState S, const CellDesc* __restrict__ cells, const int* __restri
              const int* __restrict__ nbig_p, int begin, int nbatch, int crun, int cluster) {
   namespace cg = cooperative_groups;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ CellShared<R> sh;
   __shared__ int sj;
   if (*(volatile int*)S.status & ST_HALT) {   // halted until the host reruns the sub-batch
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < nbatch; j += gridDim.x * blockDim.x)
@@ -1867,7 +1886,7 @@ k_cell_solve(DevState S, const CellDesc* __restrict__ cells, const int* __restri
       const int j = sj;
       if (j >= nbig) break;
       const int cidx = order[begin + j];
-      cell_solve_dist<R>(S, cells[begin + cidx], cidx, nbatch, crank, C, smem_raw);
+      cell_solve_dist<R>(S, cells[begin + cidx], cidx, nbatch, crank, C, sh, smem_raw);
       cg::this_cluster().sync();
     }
   }
@@ -1879,7 +1898,7 @@ k_cell_solve(DevState S, const CellDesc* __restrict__ cells, const int* __restri
     const int j = nbig + sj;
     if (j >= nbatch) break;
     const int cidx = order ? order[begin + j] : j;
-    cell_solve_body<R, BAL>(S, cells[begin + cidx], cidx, nbatch, smem_raw);
+    cell_solve_body<R, BAL>(S, cells[begin + cidx], cidx, nbatch, sh, smem_raw);
   }
 }
 
@@ -2013,6 +2032,7 @@ k_cell_solve_multi(const DevState* __restrict__ states, const CellRef* __restric
   namespace cg = cooperative_groups;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ DevState sS;
+  __shared__ CellShared<R> sh;
   __shared__ int sj;
   auto load_state = [&](int inst) {
     const int* src = reinterpret_cast<const int*>(states + inst);
@@ -2043,7 +2063,7 @@ k_cell_solve_multi(const DevState* __restrict__ states, const CellRef* __restric
       if (j >= nbig) break;
       const CellRef rf = refs[order[j]];
       load_state(rf.inst);
-      if (!halted(rf)) cell_solve_dist<R>(sS, sS.cells[part][rf.cell], rf.pos, rf.nbatch, crank, C, smem_raw);
+      if (!halted(rf)) cell_solve_dist<R>(sS, sS.cells[part][rf.cell], rf.pos, rf.nbatch, crank, C, sh, smem_raw);
       cg::this_cluster().sync();
     }
   }
@@ -2056,7 +2076,7 @@ k_cell_solve_multi(const DevState* __restrict__ states, const CellRef* __restric
     if (j >= nref) break;
     const CellRef rf = refs[order ? order[j] : j];
     load_state(rf.inst);
-    if (!halted(rf)) cell_solve_body<R, false>(sS, sS.cells[part][rf.cell], rf.pos, rf.nbatch, smem_raw);
+    if (!halted(rf)) cell_solve_body<R, false>(sS, sS.cells[part][rf.cell], rf.pos, rf.nbatch, sh, smem_raw);
   }
 }
 

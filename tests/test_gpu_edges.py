@@ -341,3 +341,23 @@ def test_translation_step_stops_alike_on_clusters(env, N, s, ctas):
     assert (got[0][:, 5] == 0).all() and np.array_equal(got[0][:, :5], one[0][:, :5])
     for k in (1, 2):
         assert np.abs(got[k] - one[k]).sum() <= 1e-9 * np.abs(one[k]).sum()
+
+
+# --------------------------------------------------------------- capacity of a Y-box
+@pytest.mark.parametrize("ctas", [0, 8])
+def test_largest_boxes_without_spill_slots(env, ctas):
+    """96 x 96 boxes of double cells at s = 16 fill the shared memory of eight CTAs to the last
+    32 points: they run without a spill slot."""
+    torch, dd = env
+    N, s = 96, 16
+    mu, nu = inputs.mixture_blobs(N=N, seed=23)
+    eps = 16.0 / N ** 2
+    out = []
+    for slots in (16, -1):
+        with dd.DomDec(mu, nu, eps, 1.0, s, precision="fp64", cell_ctas=ctas, err=-1.0, maxit=2, strategy="safe",
+                       spill_slots=slots) as g:
+            g.iterate(1)
+            assert g.sync() == 0
+            out.append(g.marginals())
+    for k in range(2):
+        assert np.abs(out[1][k] - out[0][k]).sum() <= 1e-11 * np.abs(out[0][k]).sum()
