@@ -36,8 +36,8 @@
 // takes 2.4 (no moment) to 5 (two moments) FP64 operations there where a term of its own
 // exponential takes 12 to 16.  512 x 512, eps = (2/N)^2, the whole call:
 // 2.63 ms (CUDA exp2) -> 2.02 (table exponential) -> 1.26 (tiles); below
-// kTileMinN the tiles are too few to hide the FP64 latency (N = 150: 32 us a pass
-// against 28).
+// kTileMinN the tiles are too few to hide the FP64 latency (N = 150, eight lanes a
+// tile: 32 us a pass against 28).
 #include <cmath>
 
 #include "dd_tiles.cuh"
@@ -187,13 +187,13 @@ __global__ void __launch_bounds__(256) k_adj_cols(AdjBufs<R> B, AdjOut O, int N,
 }
 
 // The tile passes: a[j, k] and, with MOM, m[j, k] (transposed) ...
-template <int P, bool MOM>
+template <bool MOM>
 __global__ void __launch_bounds__(512)
 k_adj_first(const double* __restrict__ f, const float* __restrict__ fs, double* __restrict__ a, float* __restrict__ as,
             double* __restrict__ m, int N, double Q, int per, int D4) {
   extern __shared__ __align__(16) unsigned char sm[];
   const int k = blockIdx.x;
-  tile_rows<P, MOM ? 1 : 0>(sm, f, fs, nullptr, N, Q, per, D4, [&](int j, double v, double m1, double) {
+  tile_rows<MOM ? 1 : 0>(sm, f, fs, nullptr, N, Q, per, D4, [&](int j, double v, double m1, double) {
     const long long o = (long long)j * N + k;
     a[o] = v;
     as[o] = (float)v;
@@ -202,13 +202,13 @@ k_adj_first(const double* __restrict__ f, const float* __restrict__ fs, double* 
 }
 
 // ... then along the columns of the grid, with the gradient epilogue.
-template <int P, bool MOM>
+template <bool MOM>
 __global__ void __launch_bounds__(512)
 k_adj_second(const double* __restrict__ a, const float* __restrict__ as, const double* __restrict__ m, AdjOut O, int N,
              double Q, int per, int D4) {
   extern __shared__ __align__(16) unsigned char sm[];
   const int j = blockIdx.x;
-  tile_rows<P, MOM ? 2 : 0>(sm, a, as, m, N, Q, per, D4, [&](int i, double L, double m1, double m2) {
+  tile_rows<MOM ? 2 : 0>(sm, a, as, m, N, Q, per, D4, [&](int i, double L, double m1, double m2) {
     adj_store<MOM>(O, (long long)i * N + j, L, m1, m2);
   });
 }
@@ -223,9 +223,9 @@ cudaError_t adj_side_tiles(const double* f, const float* fs, double* a, float* a
     return cudaGetLastError();
   };
   const TileShape t1 = tile_shape(N, Q, MOM ? 1 : 0), t2 = tile_shape(N, Q, MOM ? 2 : 0);
-  cudaError_t e = t1.lanes == 8 ? run(k_adj_first<8, MOM>, t1, f, fs, a, as, m) : run(k_adj_first<4, MOM>, t1, f, fs, a, as, m);
+  cudaError_t e = run(k_adj_first<MOM>, t1, f, fs, a, as, m);
   if (e == cudaSuccess)
-    e = t2.lanes == 8 ? run(k_adj_second<8, MOM>, t2, a, as, m, O) : run(k_adj_second<4, MOM>, t2, a, as, m, O);
+    e = run(k_adj_second<MOM>, t2, a, as, m, O);
   return e;
 }
 

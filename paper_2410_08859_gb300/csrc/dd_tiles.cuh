@@ -9,11 +9,15 @@ namespace {
 
 constexpr int kSepBlock = 16;    // sources per block maximum
 constexpr int kTile = 8;         // consecutive targets of one line per group of lanes
+// Four lanes: the whole adjoint at eps = 4 h^2, four | eight lanes: N = 192 467 | 469 us, 256 576 | 587,
+// 320 655 | 686, 384 730 | 815, 512 964 | 1102, 1024 3151 | 3750 (eight halve a lane's share of a window
+// but double the searches for maxima).
+constexpr int kTileLanes = 4;
 constexpr int kTileMinN = 192;   // smallest grid of the tile passes (few tiles below: their FP64 latency shows)
 
 // One row pass in double: line k = blockIdx.x, L(j) = log2 sum_m 2^{f(k, m) - q2 (j - m)^2}
 // for the targets blockIdx.y * per + [0, per), a tile of kTile consecutive targets
-// per group of P lanes.
+// per group of kTileLanes lanes.
 // With the tile's anchor a and a centre c of its sources,
 //   2^{f(m) - q2 (m - a - k)^2} = G(m) 2^{2 q2 (m - c) k} 2^{2 q2 (c - a) k - q2 k^2},
 //   G(m) = 2^{f(m) - q2 (m - a)^2}:
@@ -32,7 +36,7 @@ constexpr int kTileMinN = 192;   // smallest grid of the tile passes (few tiles 
 // out(j, L, mean1, mean2) is called once per target by consecutive threads.
 // One pass without moments at eps = 4 h^2, against one exponential per term (12
 // operations): 1024 x 1024 1093 -> 344 us, 512 x 512 283 -> 96, 256 x 256 81 -> 43.
-template <int P, int MOM, typename Out>
+template <int MOM, typename Out>
 __device__ __forceinline__ void tile_rows(unsigned char* sm, const double* __restrict__ src,
                                           const float* __restrict__ srcf, const double* __restrict__ mom,
                                           int N, double q2, int per, int D4, Out out) {
@@ -85,7 +89,8 @@ __device__ __forceinline__ void tile_rows(unsigned char* sm, const double* __res
     const float d = (float)(j - m);
     return fmaf(-(q2f * d), d, rowf[m]);
   };
-  // the largest float term of target j (P lanes)
+  // the largest float term of target j (the lanes of a group)
+  constexpr int P = kTileLanes;
   const int part = threadIdx.x & (P - 1);
   auto maximum = [&](int j) {
     float ub = -INFINITY, mx = -INFINITY;
@@ -258,18 +263,20 @@ __device__ __forceinline__ void tile_rows(unsigned char* sm, const double* __res
   }
 }
 
-// Launch shape of a tile pass: eight lanes a tile below N = 400, else four.
+// Launch shape of a tile pass.  A row is split over several CTAs (at least 64 targets each) where
+// the rows alone are fewer than four per SM: the whole adjoint at eps = 4 h^2, split | one CTA a
+// row (eight lanes a tile): N = 192 461 | 506 us, 320 675 | 740, 384 809 | 842, 512 961 | 1023; at 256 and 448 the
+// split costs 5 % (575 | 546, 855 | 813); from 608 on it is the same.
 struct TileShape {
-  int lanes, per, threads, D4;
+  int per, threads, D4;
   size_t smem;
   dim3 grid;
 };
 inline TileShape tile_shape(int N, double q2, int mom) {
   TileShape t;
-  t.lanes = N < 400 ? 8 : 4;
   const int gy = std::max((N + 1023) / 1024, std::min((N + 63) / 64, (608 + N - 1) / N));
   t.per = ((N + gy - 1) / gy + kTile - 1) / kTile * kTile;
-  t.threads = std::min(512, ((t.per / kTile * t.lanes + 31) / 32) * 32);
+  t.threads = std::min(512, ((t.per / kTile * kTileLanes + 31) / 32) * 32);
   // table: twice the reach of a term within the cut plus the blocks' width, within the exponent range
   const double reach = 2.0 * std::sqrt(66.0 / q2) + 48.0;
   const int D = (int)std::min({(double)N, reach, 1023.0});
