@@ -1657,8 +1657,7 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
     }
     csync();
     // combine the parts (rank order: every CTA gets the same W), gap terms (a4), next alpha (a2)
-    double gl = 0.0;
-    R asum = R(0);
+    R gl = R(0), ge = R(0), asum = R(0);   // gl + ge: the thread's gap terms without rounding
     for (int t = tid; t < nx; t += nthr) {
       R mx = -dd_inf<R>();
       for (int rk = 0; rk < C; ++rk) mx = max(mx, Wx[rk * cap_nx + t]);
@@ -1673,7 +1672,14 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
       const R a = av_c[t];
       const R tt = a + W2 * LN2;         // log(P_X pi / mu)
       const R g = gA + g0[t] - sR * a;   // -alpha/lam
-      gl += (double)(dd_ex2((lm[t] + g) * L2E) * dd_psi<R>(tt - g));
+      const R term = mul_rn(dd_ex2((lm[t] + g) * L2E), dd_psi<R>(tt - g));
+      if constexpr (sizeof(R) == 4) {   // TwoSum (Knuth); at most two terms a thread
+        const R sum = __fadd_rn(gl, term), b = __fsub_rn(sum, gl);
+        ge += __fadd_rn(__fsub_rn(gl, __fsub_rn(sum, b)), __fsub_rn(term, b));
+        gl = sum;
+      } else {
+        gl += term;
+      }
       const R xi1 = R(cd.i0 + r - xc1), xi2 = R(cd.j0 + c - xc2);
       const R an = cA - rR * W2 * LN2 - cD1 * xi1 - cD2 * xi2;
       av_n[t] = an;
@@ -1681,28 +1687,48 @@ __device__ __forceinline__ void cell_solve_dist(const DevState& S, const CellDes
       if (ti) asum += dd_ex2((lm[t] + gA + g0[t] - sR * an) * L2E);   // mu e^{-alpha_new/lam}
     }
     {
-      // The gap in double, as its terms decide when a cell stops: every CTA adds the same
-      // values in the same order (the warps that hold any, then warp 0 over the warps), and one
-      // thread of each decides, so no two threads can disagree.  The parts lie clear of
-      // the scratch of the epilogue's first sum, which a warp may reach before another
-      // has read the decision.
-      double* gpart = red + 384;
+      // The gap is summed in double, as its terms decide when a cell stops: over the
+      // warps that hold any, then by warp 0, and one thread decides, so no two
+      // threads of a CTA can disagree (every CTA adds the same values in the same order).
+      // Float cells first add in float: a tree of 21 roundings of terms >= 0 is within 1.3e-6 of
+      // the sum, so only at or below 1.0001 of the bound (or at the last iteration) can the
+      // double sum stop the cell, and only then it is formed -- each iteration it cost 6 % of a
+      // solve of a thousand iterations.  The parts lie clear of the scratch of the epilogue's
+      // first sum, which a warp may reach before another has read the decision.
       const int nw = nthr >> 5, wid = tid >> 5, lane = tid & 31;
-      if (32 * wid < nx) gl = warp_sum(gl);
-      if (lane == 0) gpart[wid] = gl;
+      const bool some = 32 * wid < nx;
+      R* gfirst = reinterpret_cast<R*>(red + 384);
+      double* gpart = red + 384;
+      const R gw = some ? warp_sum(gl) : R(0);
+      if (lane == 0) gfirst[wid] = gw;
       if (ti) {
         asum = warp_sum(asum);
         if (lane == 0) apart[wid] = asum;
       }
       __syncthreads();
-      if (wid == 0) {
-        gap = warp_sum(lane < nw ? gpart[lane] : 0.0);
-        if (lane == 0) stop = (S.err >= 0.0 && gap <= sk.bound) || it >= S.maxit || !(gap == gap);
+      bool near = true;
+      if constexpr (sizeof(R) == 4) {
+        R gf = R(0);
+        for (int w = 0; w < nw; ++w) gf += gfirst[w];
+        near = (S.err >= 0.0 && gf <= fmaf(sk.tol, 1.0001f, 1e-37f)) || it >= S.maxit || !(gf == gf);
       }
-      __syncthreads();
+      if (near) {   // the same in every thread
+        if constexpr (sizeof(R) == 4) {
+          double gd = (double)gl + (double)ge;
+          if (some) gd = warp_sum(gd);
+          __syncthreads();   // gfirst has been read
+          if (lane == 0) gpart[wid] = gd;
+          __syncthreads();
+        }
+        if (wid == 0) {
+          gap = warp_sum(lane < nw ? gpart[lane] : 0.0);
+          if (lane == 0) stop = (S.err >= 0.0 && gap <= sk.bound) || it >= S.maxit || !(gap == gap);
+        }
+        __syncthreads();
+        if (stop) break;
+      }
     }
     first = false;
-    if (stop) break;
     if (ti) {   // every CTA the same step
       if (tid == 0) {
         double As = 0.0, Bs = 0.0;
