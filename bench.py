@@ -48,9 +48,10 @@ METRIC = "time to stated primal-dual gap and cell-iters/s vs full Sinkhorn on on
 UNIT = "cell-iters/s"
 GAP_TARGET = 1e-5
 # dram read + write bytes of one cell-kernel launch by N (main grid, one staggered
-# sub-batch) from an ncu capture of the current kernel; a size without an entry:
-# not captured since the kernel last changed (reported as null)
-CELL_KERNEL_DRAM_BYTES = {}
+# sub-batch) from an ncu capture of the current kernel in this configuration
+# (profiles/cell_solve_lognormal1024.md); a size without an entry: not captured
+# since the kernel last changed (reported as null)
+CELL_KERNEL_DRAM_BYTES = {1024: 53097984 + 8753408}
 
 
 def peaks_file():

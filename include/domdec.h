@@ -82,7 +82,8 @@ typedef struct {
   int    newton_maxit; /* cap on Newton steps per y in the Y-half */
   int    precision;    /* DOMDEC_FP32 | DOMDEC_FP64 */
   int    box_margin;   /* pixels added around B_J (0 in the paper) */
-  int    max_ny;       /* capacity of a cell Y-box in the kernel (0: default 8192 for FP32, 4096 for FP64) */
+  int    max_ny;       /* capacity of a cell Y-box in the kernel (0: default 8192 for FP32, 3072 for FP64,
+                          less where it does not fit shared memory) */
   double arena_factor; /* box arena capacity in units of N*N doubles (0: default 48, and at least 8x the
                           initial plan).  When the new boxes of a sub-batch would not fit, the sweep kernels
                           stop changing the state from that sub-batch on; the next synchronising call grows

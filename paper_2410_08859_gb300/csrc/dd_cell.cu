@@ -206,8 +206,8 @@ __device__ __forceinline__ float max_nan(float a, float b) {
 // ---- float passes: a tile of B consecutive targets of one line per thread.
 // Chunks of kChunk sources whose terms all lie more than kCut (log2 units) below
 // their targets' shifts are left out.  A sum made that way is accepted between
-// kAccLo and 1e25, so what is left out is below 256 * 2^-60 / 2^-12 = 2^-40 of
-// it: it vanishes in the float sum.  (The floats are summed in one fixed order,
+// kAccLo and 1e25, so what is left out of M sources is below M 2^-60 / 2^-12 = M 2^-48
+// of it: it vanishes in the float sum.  (The floats are summed in one fixed order,
 // eight partial sums by the source index modulo eight: where the background
 // dominates, the Newton root amplifies a rounding of its argument by lam/eps, so
 // a value must not depend on the tile it was computed in.)

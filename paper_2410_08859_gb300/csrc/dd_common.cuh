@@ -343,8 +343,8 @@ template <typename T> __device__ __forceinline__ T warp_max(T v) {
 }
 
 // Block-wide sum of K values per thread; result valid in every thread.
-// Warp 0 adds the per-warp partials in a fixed order (deterministic).
-// `scratch` must hold 32*K values of type T; ends with a barrier.
+// Warp k (modulo the number of warps) adds the per-warp partials of value k in a
+// fixed order (deterministic).  `scratch` must hold 33*K values of type T; ends with a barrier.
 template <int K, typename T>
 __device__ __forceinline__ void block_sum(T (&v)[K], T* scratch) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;

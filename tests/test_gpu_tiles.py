@@ -1,8 +1,8 @@
 """The tile and window kernels at the sizes where they can go wrong, against plain
 64-bit torch: the separable Sinkhorn passes and the adjoint (edges of the
-8-target tiles and of the 16-source blocks, the switch of the lanes at N = 128,
-eps so small that the table of powers does not cover a window, eps so large
-that every source is kept), the tile-wise box test of a dual-initialised plan,
+8-target tiles and of the 16-source blocks, eps so small that the table of
+powers does not cover a window, eps so large that every source is kept), the
+tile-wise box test of a dual-initialised plan,
 and cells whose per-y arrays lie in a spill slot on one CTA and on a cluster."""
 import numpy as np
 import pytest
