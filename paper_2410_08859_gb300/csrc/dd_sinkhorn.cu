@@ -57,9 +57,10 @@ constexpr int kSepBlock = 16;   // sources per block maximum
 // then run over nearly the same window, where a test of every source held all of
 // them for any one's term; the products q2 d come from a table and the
 // logarithms are taken by full warps at the end.  Measured, before -> now:
-// 256 x 256 FAST at eps = 8 h^2 71 -> 33 us, 32 h^2 103 -> 47; float 12.5 -> 9.5 (128 h^2); 1024 x 1024 FAST 802 -> 317 (2 h^2), float
-// 542 -> 127 (128 h^2); 64 x 64 double 27 -> 12 (the rows split over several CTAs
-// to reach all SMs).  WIDE: no windows, every source tested (see sep_pass).
+// 256 x 256 FAST at eps = 8 h^2 71 -> 33 us, 32 h^2 103 -> 47; float 12.5 -> 9.5 (128 h^2);
+// 1024 x 1024 FAST 802 -> 317 (2 h^2), float 542 -> 127 (128 h^2); 64 x 64 double 27 -> 12 (the
+// rows split over several CTAs to reach all SMs).  WIDE: no windows, every source tested
+// (see sep_pass).
 template <typename R, bool FAST, bool WIDE>
 __global__ void __launch_bounds__(1024)
 k_sep_rows_t(const R* __restrict__ src, const float* __restrict__ srcf, R* dst, float* __restrict__ dstf, int N,

@@ -167,7 +167,7 @@ def test_newton_root(env, s, scale):
     is a rounding of g's terms over g', plus the last step's cube (1e-15) and a rounding of u."""
     torch, lib = env
     rng = np.random.default_rng(int(1 / s) + int(scale))
-    n = 20000
+    n = 4000
     lr = scale * rng.normal(size=n)
     lr[::7] = -np.inf
     c0 = scale * rng.normal(size=n)
