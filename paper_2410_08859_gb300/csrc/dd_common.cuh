@@ -245,12 +245,12 @@ __device__ __forceinline__ void log_parts(double x, double& ed, double& log_c, d
   const double m = __hiloint2double(mh | 0x3ff00000, lo);
   const bool up = mh >= 0x00080000;
   const int kk = up ? (mh + 0x2000) >> 14 : (mh + 0x1000) >> 13;
-  double f = m - __hiloint2double(0x3ff00000 + (up ? kk << 14 : kk << 13), 0);   // exact
-  f = up ? 0.5 * f : f;
+  const double f = m - __hiloint2double(0x3ff00000 + (up ? kk << 14 : kk << 13), 0);   // exact
   const int j = up ? kk - 64 : kk;   // -32..64
   e += up ? 1 : 0;
   ed = __hiloint2double(0x43300000, (int)((unsigned)e ^ 0x80000000u)) - 4503601774854144.0;   // 2^52 + 2^31
-  const double r = f * kInvC[j + 32];
+  const double inv = kInvC[j + 32];   // halved in place of f
+  const double r = f * __hiloint2double(__double2hiint(inv) - (up ? 0x00100000 : 0), __double2loint(inv));
   double p = fma(r, 1.0 / 7.0, -1.0 / 6.0);
   p = fma(p, r, 0.2);
   p = fma(p, r, -0.25);

@@ -231,13 +231,16 @@ k_line(DevState S, const CellDesc* __restrict__ cells, int begin, int nbatch, in
   if (S.line[5] != 0.0 || (*(volatile int*)S.status & ST_HALT)) return;   // uniform across blocks
   const double z = first ? 1.0 : S.line[2], lo = S.line[6];
   double v[4] = {0.0, 0.0, 0.0, 0.0};
+  // (comparisons of doubles on the integer pipe; the FP64 pipe bounds the evaluation)
+  auto floored = [](double p) { return __double2hiint(p) > 0x02000000 ? p : fmax(p, kLinePfloor); };   // 2^-991
+  auto nonzero = [](double d) { return ((__double2hiint(d) & 0x7fffffff) | __double2loint(d)) != 0; };
   auto term = [&](double p0, double d, double m) {
-    const double p = fmax(p0 + z * d, kLinePfloor);
+    const double p = floored(p0 + z * d);
     const double t = d * dd_log_quotient(p, m);
     v[0] += t;
     v[1] += dd_div(d * d, p);
     v[2] += fabs(t);
-    if (first) v[3] += d * dd_log_quotient(fmax(p0 + lo * d, kLinePfloor), m);
+    if (first) v[3] += d * dd_log_quotient(floored(p0 + lo * d), m);
   };
   const int N = S.N;
   for (int j = blockIdx.x; j < nbatch; j += gridDim.x) {
@@ -249,13 +252,13 @@ k_line(DevState S, const CellDesc* __restrict__ cells, int begin, int nbatch, in
       const int r = t / cd.nx2, c = t - r * cd.nx2;
       const int x = (cd.i0 + r) * N + cd.j0 + c;
       const double p0 = S.PX[x], d = S.PXnew[x] - p0;
-      if (d != 0.0) term(p0, d, S.mu[x]);
+      if (nonzero(d)) term(p0, d, S.mu[x]);
     }
   }
   const int n = N * N;
   for (int y = blockIdx.x * blockDim.x + threadIdx.x; y < n; y += gridDim.x * blockDim.x) {
     const double d = S.dPY[y];
-    if (d != 0.0) term(S.PY[y], d, S.nu[y]);
+    if (nonzero(d)) term(S.PY[y], d, S.nu[y]);
   }
   block_sum_wide<4>(v, red, 512);
   if (threadIdx.x == 0) {
